@@ -165,6 +165,11 @@ typedef struct {
      * (a tile above 8192 unknowns, several right-hand sides, EL / EMR); with
      * tune set and strategy 0 it is one of the timed candidates. */
     int32_t strategy;
+    /* With one right-hand side and no streaming shape, lane map, pixel
+     * numbering or plain loads asked for (the four options below), strategies
+     * 1 and 2 read strip-ordered copies of A when neighbouring rows (columns)
+     * are alike enough: four at a time, as packets of 128 entries with 16-bit
+     * offsets, about 6.3 bytes per FP32 entry and copy beside the row copy. */
     /* Streaming of A through shared memory by bulk asynchronous copies (TMA)
      * for one right-hand side: 0 automatic (used when eligible), -1 off. */
     int32_t tma;

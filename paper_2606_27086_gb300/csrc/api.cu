@@ -33,6 +33,14 @@ constexpr int kMaxTile = 4096;
 constexpr int kDefaultRowMap = 0;
 constexpr int kDefaultColMap = 0;
 
+// Strip-ordered passes.  Ring bytes: CT 512x512 ran the same from 96 to 192 KB
+// (254-257 us a row pass), so the rest stays with L1.  They are taken while
+// their padding stays below kStripSlots slots per entry: at 1.4 an entry costs
+// 8.6 bytes, about the streamed passes' 8, and CT and travel-time rows lie at
+// 1.05-1.10, their columns at 1.11-1.38.
+constexpr int kStripRing = 160 * 1024;
+constexpr double kStripSlots = 1.4;
+
 // Stored length of an item: rows and columns start at multiples of four
 // elements and are zero-padded to a multiple of four.
 inline long long pad4(long long len) { return (len + 3) & ~3LL; }
@@ -173,6 +181,19 @@ struct suppy_ctx {
     std::vector<size_t> seg_tpart_off, seg_ctpart_off;
     int* d_tpart = nullptr;
     int* d_ctpart = nullptr;
+    // strip-ordered passes (strip.cu, B = 1): rows, and columns (two passes)
+    struct StripSet {
+        unsigned char* d_blob = nullptr;
+        int4* d_meta = nullptr;
+        int* d_cta = nullptr;
+        std::vector<int> grid;          // per block: CTAs
+        std::vector<size_t> cta_off;    // per block: offset of its boundaries in d_cta
+        int nw = 4;                     // warps per strip
+        int keep = 0;                   // the packets stay in L2 between sweeps
+        long long tall = 0;             // rows in strips of tall patches
+    };
+    bool strips = false;            // the sweep uses them
+    StripSet rstrips, cstrips;
     int* d_err = nullptr;           // set by a kernel whose bounded wait gave up
     long long wait_cycles = kDefaultWaitCycles;   // budget of one bounded device wait
     unsigned* d_cticket = nullptr;  // streamed column pass: CTAs finished (fused epilogue)
@@ -515,6 +536,29 @@ suppy_status prepare_ext(suppy_ctx* c) {
     return SUPPY_OK;
 }
 
+// Row pass of block t over the strip-ordered copy.
+StripArgs strip_row_args(suppy_ctx* c, int t, float lam) {
+    StripArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.blob = c->rstrips.d_blob;
+    a.meta = c->rstrips.d_meta;
+    a.cta = c->rstrips.d_cta + c->rstrips.cta_off[t];
+    a.ring = kStripRing;
+    a.keep = c->rstrips.keep;
+    a.err = c->d_err;
+    a.wait_cycles = c->wait_cycles;
+    a.l = c->d_l;
+    a.u = c->d_u;
+    a.wr = c->d_wr;
+    a.x = a.xT = c->d_x;
+    a.delta = a.deltaT = c->d_delta;
+    a.pp = c->d_pp;
+    a.st = c->d_st;
+    a.lam = lam;
+    a.check_stop = 1;
+    return a;
+}
+
 // EL / EMR after the column pass of block t (delta holds A^T(W d)): for EMR
 // the row pass over q = A delta (zero bounds, so d = -q; the proximity
 // machinery sums w_i q_i^2 with the multiplier ||a_i||^2), then the step.
@@ -522,9 +566,20 @@ suppy_status enqueue_ext_step(suppy_ctx* c, const suppy_params* p, int t, int np
     int nqq = 0;
     if (c->mode == SUPPY_EMR) {
         // the launch writes one partial per CTA: check the buffer first
-        nqq = c->use_tma ? c->seg_tgrid[t] : c->seg_grid[t];
+        nqq = c->strips ? c->rstrips.grid[t] : (c->use_tma ? c->seg_tgrid[t] : c->seg_grid[t]);
         if (nqq > c->qq_cap) return fail(c, SUPPY_ECUDA, "q-pass launch exceeds its partials");
-        if (c->use_tma) {
+        if (c->strips) {
+            StripArgs q = strip_row_args(c, t, 0.f);
+            q.l = c->d_zero;
+            q.u = c->d_zero;
+            q.x = q.xT = c->d_delta;
+            q.prox_mul = c->d_rhof;
+            q.pp = c->d_qq;
+            Timed tm{c, 0};
+            CK(tm.begin());
+            CK(launch_strip(q, c->dt, 0, c->rstrips.nw, c->rstrips.grid[t], c->stream));
+            CK(tm.end());
+        } else if (c->use_tma) {
             StreamArgs q;
             std::memset(&q, 0, sizeof(q));
             q.info = c->d_rinfo;
@@ -712,8 +767,8 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
     // one pass with the column-major accumulator (rows running down the image);
     // two passes with those rows read column-major (their indices and a copy
     // of x made before each block's row pass: x changes after every block)
-    const bool tr_scatter = c->use_tma && c->strategy == 1 && c->scat == 1 && c->d_rowT && c->tr_on;
-    const bool tr_gather = c->use_tma && c->strategy == 2 && c->d_colT && c->tr_on;
+    const bool tr_scatter = !c->strips && c->use_tma && c->strategy == 1 && c->scat == 1 && c->d_rowT && c->tr_on;
+    const bool tr_gather = !c->strips && c->use_tma && c->strategy == 2 && c->d_colT && c->tr_on;
     // one pass in the patch numbering: patch indices, gathers from the patch
     // copies of x, both accumulators in patch layouts
     const bool patch = tr_scatter && c->tr_patch && c->d_colP;
@@ -721,7 +776,94 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
         SweepArgs a = row_args(c, t, lam_row);
         if (c->mode == SUPPY_EMR) a.coef_mul = c->d_rhof;
         const EpiArgs epi = epi_args(c, t, sp);
-        if (c->use_tma) {
+        if (c->strips) {
+            const bool strip_patch = c->strategy == 1 && c->tr_patch;
+            EpiArgs e2 = epi;
+            e2.npp = c->rstrips.grid[t];
+            {
+                StripArgs ra = strip_row_args(c, t, lam_row);
+                ra.coef = (c->strategy == 2) ? c->d_coef : nullptr;
+                ra.coef_mul = (c->mode == SUPPY_EMR) ? c->d_rhof : nullptr;
+                if (strip_patch) {
+                    ra.x = c->d_xA;
+                    ra.xT = c->d_xB;
+                    ra.deltaT = c->d_deltaT;
+                }
+                Timed tm{c, 0};
+                CK(tm.begin());
+                // the patch copies of x at the sweep's start, unless the
+                // perturbation phase just left them (a CQ step changes x);
+                // later blocks find them written by the box step before
+                if (strip_patch && t == 0 && !(copies_fresh && !c->dvc_on)) {
+                    CK(launch_patch_image(c->d_x, c->d_xA, c->d_xB, c->gH, c->gW, c->gWp, c->stream));
+                    note_launch(c);
+                }
+                CK(launch_strip(ra, c->dt, c->strategy == 2 ? 0 : 1, c->rstrips.nw, c->rstrips.grid[t],
+                                c->stream));
+                CK(tm.end());
+                note_launch(c);
+            }
+            if (c->strategy == 2) {
+                StripArgs ca;
+                std::memset(&ca, 0, sizeof(ca));
+                ca.blob = c->cstrips.d_blob;
+                ca.meta = c->cstrips.d_meta;
+                ca.cta = c->cstrips.d_cta + c->cstrips.cta_off[t];
+                ca.ring = kStripRing;
+                ca.keep = c->cstrips.keep;
+                ca.err = c->d_err;
+                ca.wait_cycles = c->wait_cycles;
+                ca.x = ca.xT = c->d_coef;
+                ca.xw = c->d_x;
+                ca.lo = c->d_lo;
+                ca.hi = c->d_hi;
+                ca.zc = c->d_zc;
+                ca.delta_out = ext ? c->d_delta : nullptr;
+                ca.box_len = c->box_len;
+                ca.epi = e2;
+                const bool fuse_epi = !ext && e2.last_seg && c->d_cticket;
+                ca.ticket = fuse_epi ? c->d_cticket : nullptr;
+                {
+                    Timed tm{c, 1};
+                    CK(tm.begin());
+                    CK(launch_strip(ca, c->dt, 2, c->cstrips.nw, c->cstrips.grid[t], c->stream));
+                    CK(tm.end());
+                    note_launch(c);
+                }
+                if (ext && (s = enqueue_ext_step(c, p, t, e2.npp)) != SUPPY_OK) return s;
+                if (e2.last_seg && !fuse_epi) {
+                    CK(launch_epilogue(e2, c->stream));
+                    note_launch(c);
+                }
+            } else {
+                FinalizeArgs f{};
+                f.x = c->d_x;
+                f.delta = c->d_delta;
+                if (strip_patch) {
+                    f.deltaT = c->d_deltaT;
+                    f.imgW = c->gW;
+                    f.imgH = c->gH;
+                    f.patch = 1;
+                    f.imgWp = c->gWp;
+                    if (t + 1 < c->nseg) {
+                        f.xA = c->d_xA;
+                        f.xB = c->d_xB;
+                    }
+                }
+                f.zc = c->d_zc;
+                f.lo = c->d_lo;
+                f.hi = c->d_hi;
+                f.nB = c->n;
+                f.B = 1;
+                f.box_len = c->box_len;
+                f.epi = e2;
+                Timed tm{c, 1};
+                CK(tm.begin());
+                CK(launch_finalize(f, c->grid_fin, c->stream));
+                CK(tm.end());
+                note_launch(c);
+            }
+        } else if (c->use_tma) {
             StreamArgs sa;
             std::memset(&sa, 0, sizeof(sa));
             sa.info = c->d_rinfo;
@@ -950,8 +1092,8 @@ suppy_status enqueue_perturb(suppy_ctx* c, const suppy_params* p, int record_onl
     a.pA = nullptr;
     a.pB = nullptr;
     a.pWp = 0;
-    const bool patch_next = c->use_tma && c->strategy == 1 && c->scat == 1 && c->d_rowT && c->tr_on &&
-                            c->tr_patch && c->d_colP && c->B == 1;
+    const bool patch_next = c->strategy == 1 && c->tr_patch && c->B == 1 &&
+                            (c->strips || (c->use_tma && c->scat == 1 && c->d_rowT && c->tr_on && c->d_colP));
     if (copies) *copies = false;
     if (copies && patch_next && c->wide && !record_only) {
         a.pA = c->d_xA;
@@ -1391,6 +1533,180 @@ void free_csc(suppy_ctx* c) {
     c->cpref.shrink_to_fit();
 }
 
+// Both accumulators of the one-pass scatter over the grid padded to multiples
+// of 8 (the patch numbering's lines; the padding is never added into).
+suppy_status alloc_accumulators(suppy_ctx* c) {
+    c->gWp = (c->gW + 7) & ~7;
+    const size_t acc = std::max((size_t)c->n, (size_t)((c->gH + 7) & ~7) * (size_t)c->gWp);
+    suppy_status s;
+    if (acc > c->acc_len) {
+        dfree(c, c->d_delta);
+        c->d_delta = nullptr;
+        if ((s = dalloc(c, &c->d_delta, acc)) != SUPPY_OK) return s;
+        CK(cudaMemsetAsync(c->d_delta, 0, sizeof(float) * acc, c->stream));
+    }
+    c->acc_len = acc;
+    if (c->d_deltaT) return SUPPY_OK;
+    if ((s = dalloc(c, &c->d_deltaT, acc)) != SUPPY_OK) return s;
+    CK(cudaMemsetAsync(c->d_deltaT, 0, sizeof(float) * acc, c->stream));
+    return SUPPY_OK;
+}
+
+// The patch-layout copies of x.
+suppy_status alloc_patch_copies(suppy_ctx* c) {
+    if (c->d_xA) return SUPPY_OK;
+    suppy_status s;
+    if ((s = dalloc(c, &c->d_xA, c->acc_len)) != SUPPY_OK) return s;
+    if ((s = dalloc(c, &c->d_xB, c->acc_len)) != SUPPY_OK) return s;
+    CK(cudaMemsetAsync(c->d_xA, 0, sizeof(float) * c->acc_len, c->stream));
+    CK(cudaMemsetAsync(c->d_xB, 0, sizeof(float) * c->acc_len, c->stream));
+    return SUPPY_OK;
+}
+
+void free_strips(suppy_ctx* c, suppy_ctx::StripSet& S) {
+    for (void* p : {(void*)S.d_blob, (void*)S.d_meta, (void*)S.d_cta})
+        if (p) dfree(c, p);
+    S = suppy_ctx::StripSet{};
+}
+
+// The strip-ordered copy of a packed item list (rows, or the columns of every
+// block), built on the device; *ok says whether it pays.  block_of: first
+// item of every block in `info` (and the end); a row's number is its index
+// there, a column's its index inside the block.
+suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info, const int* idx,
+                          const void* val, const std::vector<long long>& block_of, bool columns, int max_len,
+                          long long entries, bool patch, bool* ok) {
+    *ok = false;
+    if (max_len < 1 || max_len > kStripMaxItem) return SUPPY_OK;
+    const int nseg = (int)block_of.size() - 1;
+    std::vector<int4> strips;
+    std::vector<int> seg_first(nseg + 1, 0);
+    for (int t = 0; t < nseg; ++t) {
+        for (long long i = block_of[t]; i < block_of[t + 1]; i += 4)
+            strips.push_back(make_int4((int)i, (int)std::min<long long>(4, block_of[t + 1] - i),
+                                       (int)(columns ? i - block_of[t] : i), 0));
+        seg_first[t + 1] = (int)strips.size();
+    }
+    const int ns = (int)strips.size();
+    const size_t vsz = (c->dt == SUPPY_F32) ? 4 : 2;
+    TempGuard tg;
+    tg.s = c->stream;
+    suppy_status s;
+    int4* d_strips = nullptr;
+    if ((s = stage(c, strips.data(), strips.size(), 0, &d_strips, tg.v)) != SUPPY_OK) return s;
+    void* q = nullptr;
+    CK(cudaMalloc(&q, sizeof(int4) * (size_t)std::max(ns, 1)));
+    tg.v.push_back(q);
+    StripBuild b;
+    std::memset(&b, 0, sizeof(b));
+    b.strips = d_strips;
+    b.nstrips = ns;
+    b.info = info;
+    b.idx = idx;
+    b.val = val;
+    b.max_len = max_len;
+    // rows walk an image grid along their rays; columns are rows' numbers
+    if (!columns && c->gH >= 2 && c->gW >= 2) {
+        b.H = c->gH;
+        b.W = c->gW;
+        b.Wp = (c->gW + 7) & ~7;
+        b.recipW = ~0ULL / (unsigned long long)c->gW + 1ULL;
+    }
+    b.patch = patch;
+    b.all_items = columns;
+    b.meta = static_cast<int4*>(q);
+    CK(launch_strip_build(b, c->dt, 0, c->stream));
+    note_launch(c);
+    std::vector<int4> meta(ns);
+    CK(cudaMemcpyAsync(meta.data(), q, sizeof(int4) * (size_t)ns, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    // strips without entries drop out (columns still take the box step)
+    long long packets = 0, tall = 0;
+    int most = 0, kept = 0;
+    std::vector<int> first(nseg + 1, 0);
+    for (int t = 0; t < nseg; ++t) {
+        for (int k = seg_first[t]; k < seg_first[t + 1]; ++k) {
+            int4 m = meta[k];
+            const int npk = m.y & kStripPackets;
+            if (npk == 0 && !columns) continue;
+            const long long at = packets * (strip_packet_bytes((int)vsz) / 16);
+            m.x = (int)(unsigned)at;
+            packets += npk;
+            most = std::max(most, npk);
+            if (m.y & kStripTall) tall += __builtin_popcount((unsigned)m.w);
+            meta[kept] = m;
+            strips[kept++] = strips[k];
+        }
+        first[t + 1] = kept;
+    }
+    const long long bytes = packets * strip_packet_bytes((int)vsz);
+    if (packets < 1 || (double)packets * 128.0 > kStripSlots * (double)entries + 128.0 ||
+        (long long)most * strip_packet_bytes((int)vsz) > kStripRing / 2 || (bytes >> 4) > 0xffffffffLL)
+        return SUPPY_OK;
+    S.tall = tall;
+    const double mean = (double)packets / std::max(kept, 1);
+    // warps a strip: a few packets each, so that the strips in work leave the
+    // ring room to stream ahead (CT 512x512, 14.5 packets a strip: 4, 2 and 1
+    // warps took 254, 265 and 294 us; CT 128x128 blocks have 4.4)
+    S.nw = mean >= 8.0 ? 4 : (mean >= 4.0 ? 2 : 1);
+    // packets that fit L2 (129 MB) beside the vectors stay there between sweeps
+    S.keep = bytes <= 80LL * 1024 * 1024;
+    // per block: contiguous strip ranges of equal packets (and a constant a
+    // strip), one per SM
+    int sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
+    std::vector<int> cta;
+    std::vector<long long> pref(kept + 1, 0);
+    for (int k = 0; k < kept; ++k) pref[k + 1] = pref[k] + (meta[k].y & kStripPackets) + 2;
+    S.grid.assign(nseg, 0);
+    S.cta_off.assign(nseg + 1, 0);
+    for (int t = 0; t < nseg; ++t) {
+        const int g = std::max(1, std::min(sms, first[t + 1] - first[t]));
+        S.grid[t] = g;
+        S.cta_off[t + 1] = S.cta_off[t] + g + 1;
+        cta.resize(S.cta_off[t + 1]);
+        tma_partition(pref, first[t], first[t + 1], g, cta.data() + S.cta_off[t]);
+    }
+    meta.resize(kept);
+    if ((s = dalloc(c, &S.d_blob, (size_t)bytes)) == SUPPY_ENOMEM) return SUPPY_OK;   // the other forms need less
+    if (s != SUPPY_OK) return s;
+    // every CTA's ring, laid out ahead: a strip goes in one piece behind the
+    // newest one, or at the ring's start, once the oldest strips in the way
+    // (and all but kStripInFlight - 1) have been read
+    for (int t = 0; t < nseg; ++t)
+        for (int g = 0; g < S.grid[t]; ++g) {
+            const int k0 = cta[S.cta_off[t] + g], k1 = cta[S.cta_off[t] + g + 1];
+            int oldest = k0, head = 0;
+            for (int k = k0; k < k1; ++k) {
+                const int need = (meta[k].y & kStripPackets) * strip_packet_bytes((int)vsz);
+                int at = -1;
+                for (; at < 0; oldest += at < 0) {
+                    if (oldest == k) {
+                        at = 0;
+                    } else if (k - oldest < kStripInFlight) {
+                        const int tail = strip_at(meta[oldest].w);
+                        if (head > tail) at = head + need <= kStripRing ? head : (need <= tail ? 0 : -1);
+                        else if (head + need <= tail) at = head;
+                    }
+                }
+                meta[k].w |= (at >> 4) << 4 | (k - oldest) << 18;
+                head = at + need;
+            }
+        }
+    if ((s = upload(c, cta, &S.d_cta)) != SUPPY_OK) return s;
+    if ((s = upload(c, meta, &S.d_meta)) != SUPPY_OK) return s;
+    CK(cudaMemcpyAsync(d_strips, strips.data(), sizeof(int4) * (size_t)kept, cudaMemcpyHostToDevice,
+                       c->stream));
+    b.nstrips = kept;
+    b.meta = S.d_meta;
+    b.blob = S.d_blob;
+    CK(launch_strip_build(b, c->dt, 1, c->stream));
+    note_launch(c);
+    CK(cudaStreamSynchronize(c->stream));
+    *ok = true;
+    return SUPPY_OK;
+}
+
 // Rows of A that run down the image (they span more image rows than image
 // columns) scatter their corrections column-major, where their consecutive
 // entries are neighbours: flags in device row order, the column-major
@@ -1419,19 +1735,7 @@ suppy_status build_row_orientation(suppy_ctx* c, const std::vector<int>& rp, con
     if (nt == 0) return SUPPY_OK;
     suppy_status s;
     if ((s = upload(c, flag, &c->d_rowT)) != SUPPY_OK) return s;
-    // both accumulators cover the grid padded to multiples of 8 (the patch
-    // numbering's lines); the padding is never added into
-    c->gWp = (W + 7) & ~7;
-    const size_t acc = std::max((size_t)c->n, (size_t)((c->gH + 7) & ~7) * (size_t)c->gWp);
-    if (acc > c->acc_len) {
-        dfree(c, c->d_delta);
-        c->d_delta = nullptr;
-        if ((s = dalloc(c, &c->d_delta, acc)) != SUPPY_OK) return s;
-        CK(cudaMemsetAsync(c->d_delta, 0, sizeof(float) * acc, c->stream));
-    }
-    c->acc_len = acc;
-    if ((s = dalloc(c, &c->d_deltaT, acc)) != SUPPY_OK) return s;
-    CK(cudaMemsetAsync(c->d_deltaT, 0, sizeof(float) * acc, c->stream));
+    if ((s = alloc_accumulators(c)) != SUPPY_OK) return s;
     c->trows = nt;
     CK(cudaStreamSynchronize(c->stream));   // the flags' host copy goes out of scope
     return SUPPY_OK;
@@ -1463,10 +1767,7 @@ suppy_status build_col_patch(suppy_ctx* c) {
     suppy_status s;
     const size_t rlen = (size_t)c->nnz_pad + kMaxTile + 16;
     if ((s = dalloc(c, &c->d_colP, rlen)) != SUPPY_OK) return s;
-    if ((s = dalloc(c, &c->d_xA, c->acc_len)) != SUPPY_OK) return s;
-    if ((s = dalloc(c, &c->d_xB, c->acc_len)) != SUPPY_OK) return s;
-    CK(cudaMemsetAsync(c->d_xA, 0, sizeof(float) * c->acc_len, c->stream));
-    CK(cudaMemsetAsync(c->d_xB, 0, sizeof(float) * c->acc_len, c->stream));
+    if ((s = alloc_patch_copies(c)) != SUPPY_OK) return s;
     CK(cudaMemcpyAsync(c->d_colP, c->d_col, sizeof(int) * rlen, cudaMemcpyDeviceToDevice, c->stream));
     CK(launch_patch_cols(c->d_rinfo, c->d_rowT, c->m, c->recipW, c->gW, c->gWp, c->d_colP, c->stream));
     note_launch(c);
@@ -2188,9 +2489,52 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         return fail(c, SUPPY_EINVAL, "scatter_transpose needs an image of fewer than 2^31 padded pixels");
     const bool tr_cand = tr_grid && o->scatter_transpose != -1 && !ext_mode && want != 3 &&
                          A->nnz > 0;
+    // strip-ordered passes: one right-hand side, unless the caller fixed a
+    // form of the streaming passes or of the scatter.  The one-pass scatter
+    // takes them in the patch numbering on an image grid too large for the
+    // staged scatter (smaller images fit L1 and L2 in any numbering, and the
+    // patch copies of x would cost a launch), else in the plain one.
+    const bool strips_allowed = c->B == 1 && o->tma == 0 && !o->stream_tile && !o->stream_stages &&
+                                !o->stream_lanes && !o->stream_map && !o->stream_col_map &&
+                                o->scatter_transpose == 0 && want != 3 && A->nnz > 0;
+    const bool strip_patch = tr_grid && !smem_ok &&
+                             (long long)((c->gH + 7) & ~7) * ((c->gW + 7) & ~7) < (1LL << 31);
+    std::vector<long long> row_blocks(c->seg_start.begin(), c->seg_start.end());
+    int strips_are = -1;   // the row strips built: -1 none, 0 plain, 1 patch numbering
+    // builds what a strategy's strip-ordered passes need; *ok false: they do
+    // not pay on this matrix
+    auto make_strips = [&](int strategy, bool* ok) -> suppy_status {
+        const bool patch = strategy == 1 && strip_patch;
+        suppy_status st;
+        *ok = true;
+        if (strips_are != (int)patch) {
+            free_strips(c, c->rstrips);
+            strips_are = -1;
+            if ((st = build_strips(c, c->rstrips, c->d_rinfo, c->d_col, c->d_val, row_blocks, false, max_len,
+                                   A->nnz, patch, ok)) != SUPPY_OK)
+                return st;
+            if (!*ok) return SUPPY_OK;
+            strips_are = patch;
+        }
+        if (patch) {
+            if ((st = alloc_accumulators(c)) != SUPPY_OK) return st;
+            if ((st = alloc_patch_copies(c)) != SUPPY_OK) return st;
+        }
+        if (strategy == 2 && !c->cstrips.d_blob) {
+            std::vector<long long> col_blocks(c->nseg + 1);
+            for (int t = 0; t <= c->nseg; ++t) col_blocks[t] = (long long)t * n;
+            if ((st = build_strips(c, c->cstrips, c->d_cinfo, c->d_ridx, c->d_cval, col_blocks, true, c->max_col,
+                                   c->nnz_csc, false, ok)) != SUPPY_OK)
+                return st;
+        }
+        return SUPPY_OK;
+    };
+    bool strips_ok = false;
+    if (strips_allowed && !o->tune && !need_csc && (s = make_strips(1, &strips_ok)) != SUPPY_OK) return s;
     std::vector<int> hcol_buf;
     const int* hcol = A->col;
-    if ((need_csc || tile_cand || tr_cand) && on_dev) {
+    const bool orient = tr_cand && !strips_ok;
+    if ((need_csc || tile_cand || orient) && on_dev) {
         hcol_buf.resize((size_t)std::max<long long>(A->nnz, 1));
         if (A->nnz)
             CK(cudaMemcpyAsync(hcol_buf.data(), A->col, sizeof(int) * A->nnz, cudaMemcpyDeviceToHost,
@@ -2202,6 +2546,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         if ((s = build_csc(c, rp, hcol, perm, seg_of_row, rinfo)) != SUPPY_OK) return s;
         choose_col_shape(c, mean_col);
         if ((s = build_col_partition(c)) != SUPPY_OK) return s;
+        if (strips_allowed && !o->tune && (s = make_strips(2, &strips_ok)) != SUPPY_OK) return s;
     }
     bool tile_ok = false;
     if (tile_cand) {
@@ -2214,7 +2559,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
             return s;
         if (want == 3 && !tile_ok) return fail(c, SUPPY_EINVAL, c->err);
     }
-    if (tr_cand && (s = build_row_orientation(c, rp, hcol, perm)) != SUPPY_OK) return s;
+    if (orient && !strips_ok && (s = build_row_orientation(c, rp, hcol, perm)) != SUPPY_OK) return s;
     hcol_buf.clear();
     hcol_buf.shrink_to_fit();
     // tr: the one pass with L2 reductions takes the rows running down the
@@ -2225,6 +2570,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
     struct Cand {
         int strategy, scat;
         int tr;   // 0 none, 1 column-major rows, 2 patch numbering (one pass)
+        bool strip = false;
     };
     const bool have_tr = c->d_rowT != nullptr;
     const int tr_one = !have_tr ? 0 : (o->scatter_transpose == 1 ? 1 : 2);
@@ -2241,9 +2587,16 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         if (need_csc) cands.push_back({2, 0, (o->scatter_transpose >= 1 && have_tr) ? 1 : 0});
         if (need_csc && have_tr && o->tune && o->scatter_transpose == 0) cands.push_back({2, 0, 1});
         if (tile_ok) cands.push_back({3, 0, 0});
+        if (strips_allowed && o->tune && want != 2)
+            cands.push_back({1, smem_ok ? 2 : 1, strip_patch ? 2 : 0, true});
+        if (strips_allowed && o->tune && need_csc) cands.push_back({2, 0, 0, true});
     }
     Cand best = cands[0];
     if (want == 0 && !o->tune) best = smem_ok ? Cand{1, 2, 0} : Cand{2, 0, 0};
+    if (strips_ok) {
+        best.strip = true;
+        if (best.strategy == 1) best.tr = strip_patch ? 2 : 0;
+    }
     const bool fixed_shape = o->stream_tile || o->stream_stages || o->stream_lanes;
     // Launch shape of a candidate: the register-fed sweep's row shape, then
     // (when the streamed passes serve it) their ring shapes and lane maps,
@@ -2257,7 +2610,8 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         c->scat = cd.scat;
         c->tr_on = cd.tr != 0;
         c->tr_patch = cd.tr == 2 && cd.strategy == 1;
-        if (c->tr_patch) {
+        c->strips = cd.strip;
+        if (c->tr_patch && !c->strips) {
             suppy_status st2 = build_col_patch(c);
             if (st2 != SUPPY_OK) return st2;
         }
@@ -2278,7 +2632,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
             (!group_fits(c->tG, c->max_row, c->tile, c->stages) ||
              (c->strategy == 2 && !group_fits(c->tGc, c->max_col, c->ctile, c->cstages))))
             c->use_tma = false;
-        if (c->use_tma) {
+        if (c->use_tma && !c->strips) {
             if ((st = build_tma_partitions(c)) != SUPPY_OK) return st;
             if (tune_streams && !fixed_shape &&
                 (st = tune_tma(c, o->stream_map == 0 && o->stream_col_map == 0)) != SUPPY_OK)
@@ -2297,6 +2651,11 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         // comparison is between the best form of each
         float best_ms = 1e30f;
         for (const Cand& cd : cands) {
+            if (cd.strip) {
+                bool pays = false;
+                if ((s = make_strips(cd.strategy, &pays)) != SUPPY_OK) return s;
+                if (!pays) continue;
+            }
             if ((s = set_up(cd, true)) != SUPPY_OK) return s;
             float ms = 0.f;
             if ((s = time_config(c, &ms, 12)) != SUPPY_OK) return s;
@@ -2313,6 +2672,12 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         c->scat = best.scat;
         c->tr_on = best.tr != 0;
         c->tr_patch = best.tr == 2 && best.strategy == 1;
+        c->strips = best.strip;
+        if (best.strip) {
+            bool pays = false;
+            if ((s = make_strips(best.strategy, &pays)) != SUPPY_OK) return s;
+            if (!pays) return fail(c, SUPPY_ENOMEM, "the strip-ordered copy no longer fits");
+        }
         choose_row_shape(c, mean_len, max_len);
         if ((s = build_row_partition(c)) != SUPPY_OK) return s;
         c->tG = best_sh.tG;
@@ -2324,13 +2689,27 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         c->cstages = best_sh.cstages;
         c->tMapc = best_sh.tMapc;
         c->use_tma = best_sh.use_tma;
-        if (c->use_tma && (s = build_tma_partitions(c)) != SUPPY_OK) return s;
+        if (c->use_tma && !c->strips && (s = build_tma_partitions(c)) != SUPPY_OK) return s;
     } else if ((s = set_up(best, o->tune != 0)) != SUPPY_OK) {
         return s;
     }
     if (c->strategy != 2 && c->d_cinfo) free_csc(c);
     if (!(c->strategy == 2 && c->tr_on) && c->d_colT) free_col_transposed(c);
-    if (!(c->strategy == 1 && c->tr_patch) && c->d_colP) free_col_patch(c);
+    if (!(c->strategy == 1 && c->tr_patch) && c->d_xA) free_col_patch(c);
+    if (c->strips && c->d_colP) {
+        dfree(c, c->d_colP);
+        c->d_colP = nullptr;
+    }
+    // the strip-ordered passes read their own copies: the CSC entries go (the
+    // row copy stays for the proximity)
+    if (!c->strips) free_strips(c, c->rstrips);
+    if (!(c->strips && c->strategy == 2)) free_strips(c, c->cstrips);
+    if (c->strips && c->strategy == 2) {
+        dfree(c, c->d_ridx);
+        dfree(c, c->d_cval);
+        c->d_ridx = nullptr;
+        c->d_cval = nullptr;
+    }
     if (c->strategy != 3 && c->d_tstream) free_tile(c);
     if ((s = reset_state(c)) != SUPPY_OK) return s;
     dfree(c, d_flags);
@@ -3172,10 +3551,20 @@ suppy_status suppy_info_get(const suppy_ctx* cc, suppy_info* out) {
     out->a_dtype = (int32_t)c->dt;
     out->transposed_rows = (((c->strategy == 1 && c->scat == 1 && c->d_rowT) ||
                              (c->strategy == 2 && c->d_colT)) && c->use_tma && c->tr_on) ? c->trows : 0;
+    if (c->strips) out->transposed_rows = (c->strategy == 1 && c->tr_patch) ? c->rstrips.tall : 0;
     out->scatter_patch = (out->transposed_rows > 0 && c->strategy == 1 && c->tr_patch) ? 1 : 0;
     out->map = c->use_tma ? c->tMap + 1 : 0;
     out->col_map = (c->use_tma && c->strategy == 2) ? c->tMapc + 1 : 0;
-    if (c->use_tma) {
+    if (c->strips) {
+        // eight lanes take one row (column) of a strip
+        out->grid = c->rstrips.grid[0];
+        out->block = kStripThreads;
+        out->lanes_per_row = 8;
+        if (c->strategy == 2) {
+            out->col_grid = c->cstrips.grid[0];
+            out->col_lanes = 8;
+        }
+    } else if (c->use_tma) {
         out->grid = c->seg_tgrid[0];
         out->block = kStreamThreads;
         out->lanes_per_row = c->tG;

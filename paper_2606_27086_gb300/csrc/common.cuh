@@ -232,6 +232,72 @@ struct StreamArgs {
     int patch, imgWp;
 };
 
+// One launch of a strip-ordered streaming pass (strip.cu) over the strips
+// [cta[0], cta[grid]) of one block, B = 1.  A strip is up to four consecutive
+// rows (or columns) whose entries are stored as packets of 128 slots.
+constexpr int kStripPackets = 0xffffff;   // int4 record .y: packets of the strip
+constexpr int kStripTall = 1 << 30;       // .y: rows running down the image (tall patches)
+constexpr int kStripThreads = 800;         // 24 consumer warps and one producer
+constexpr int kStripMaxItem = 4096;       // longest row or column of a strip
+constexpr int kStripInFlight = 48;         // strips a CTA's ring holds at most
+// .w: item mask (4 bits), place in the ring / 16 (14 bits), strips that may
+// still be in the ring when this one is copied in (6 bits)
+__host__ __device__ constexpr int strip_at(int w) { return ((w >> 4) & 0x3fff) << 4; }
+__host__ __device__ constexpr int strip_live(int w) { return (w >> 18) & 0x3f; }
+__host__ __device__ constexpr int strip_packet_bytes(int value_bytes) {
+    return 16 + 128 * 2 + 128 * value_bytes;   // bases, offsets, values
+}
+struct StripArgs {
+    const unsigned char* blob;   // packets
+    const int4* meta;            // per strip {offset / 16, packets and flags, first item, mask and place}
+    const int* cta;              // grid + 1 strip boundaries
+    int ring;                    // bytes of the shared-memory ring
+    int keep;                    // 1: the packets fit L2 beside the vectors (normal eviction priority)
+    int* err;                    // set to 1 when a bounded wait gives up
+    long long wait_cycles;
+    // row pass: as in StreamArgs; x / delta in the strips' numbering (wide
+    // patches or plain), xT / deltaT for the strips marked tall
+    const float* l;
+    const float* u;
+    const float* wr;
+    const float* x;              // column pass: the coefficients
+    const float* xT;
+    float* delta;
+    float* deltaT;
+    float* coef;
+    const float* coef_mul;
+    const float* prox_mul;
+    double* pp;
+    RhsState* st;
+    float lam;
+    int check_stop;
+    // column pass
+    float* xw;
+    const float* lo;
+    const float* hi;
+    const float* zc;
+    float* delta_out;
+    int box_len;
+    EpiArgs epi;
+    unsigned* ticket;
+};
+
+// Building the strips of one item list from its packed copy.
+struct StripBuild {
+    const int4* strips;          // per strip {first item in info, items, first item's number, 0}
+    int nstrips;
+    const int2* info;            // per item {start, length}
+    const int* idx;
+    const void* val;
+    int max_len;                 // longest item (at most kStripMaxItem)
+    int H, W, Wp;                // image grid of the indices (W = 0: none), W padded to 8
+    unsigned long long recipW;
+    int patch;                   // positions in the patch numbering
+    int all_items;               // items without entries count too (columns)
+    int4* meta;
+    unsigned char* blob;
+};
+
 // Tiled one-pass sweep (tile.cu): one cooperative launch of P CTAs, CTA b
 // owning tile b of the unknowns (x and the correction in shared memory) and
 // streaming tile b's segments of A once per sweep.  A CTA is one warp for the
@@ -368,6 +434,11 @@ cudaError_t launch_rows_tma(const StreamArgs& a, suppy_dtype dt, int G, int scat
                             cudaStream_t s);
 cudaError_t launch_cols_tma(const StreamArgs& a, suppy_dtype dt, int G, int map, int grid,
                             cudaStream_t s);
+// kind: 0 row pass (coefficients out), 1 row pass with the scatter, 2 column
+// pass; nw: warps per strip (1, 2 or 4)
+cudaError_t launch_strip(const StripArgs& a, suppy_dtype dt, int kind, int nw, int grid, cudaStream_t s);
+// fill 0: count the packets into meta; 1: write them at the offsets of meta
+cudaError_t launch_strip_build(const StripBuild& b, suppy_dtype dt, int fill, cudaStream_t s);
 // scat: 0 no scatter (proximity / coefficient output), 1 global reductions,
 // 2 shared-memory staged reductions (n * 4 bytes of shared memory)
 cudaError_t launch_sweep(const SweepArgs& a, suppy_dtype dt, int G, int maxe, int scat, int grid,

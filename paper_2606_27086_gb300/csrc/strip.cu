@@ -1,0 +1,571 @@
+// Strip-ordered streaming passes of the simultaneous projection sweep
+// (Sec. 2.1.1, Eq. (3)) for one right-hand side.
+//
+// A strip is up to four consecutive items: rows of the CSR copy (row pass) or
+// columns of the CSC copy (column pass) of A.  Its entries are stored as a
+// sequence of packets of 128 slots, in the order the lanes of a warp take
+// them: lanes 8r .. 8r+7 hold item r, and step s of a packet (s = 0..3) gives
+// each item eight consecutive entries.  A packet's entries come from the same
+// stretch of all four items (windows of at most 32 entries an item, cut where
+// the sorted keys of the items agree), so that the four neighbouring rays of a
+// CT or travel-time matrix are read side by side: one warp instruction covers
+// a patch of 4 x 8 neighbouring pixels instead of a line of 32.  Sectors are
+// what the gathers of x and the L2 reductions cost, and counted on CT 512x512
+// (360 angles x 725 bins) in the patch numbering they fall from 41.6 M to
+// 27.0 M a sweep; the padding of the windows costs 4.6% more slots.
+//
+// A packet is {four bases (int32, one an item), 128 16-bit offsets, 128
+// values}: position = base of the item + offset, so an entry costs 6 bytes
+// instead of 8 (FP32 values; nothing is rounded, a window ends where an
+// offset would not fit) and a lane reads its four entries of a packet with
+// one 4-byte, one 8-byte and one 16-byte shared-memory load.
+//
+// Each CTA (one per SM) owns a contiguous range of strips, balanced by their
+// packets.  One producer warp streams whole strips into a shared-memory ring
+// with bulk copies (cp.async.bulk) tracked by mbarriers, each strip in one
+// contiguous piece; 24 consumer warps in groups of NW take the strips in
+// turn, each warp a contiguous share of the strip's packets.  The dot
+// products are summed over the eight lanes and then over the group's warps in
+// a fixed order; the scatter reads the strip again from the ring.
+//
+// Measured (GB300, CT 512x512, 120.3 M entries, FP32; the streamed passes of
+// stream.cu in their default shapes before): two-pass row pass 227 -> 156 us,
+// column pass 196 -> 144 us (5.4 TB/s of the 6.7 copied), one-pass row pass
+// 342 -> 242 us.  The first two are bound by HBM; the scatter adds its L2
+// reductions, which share the load/store pipe with the gathers (without them
+// the one-pass row pass takes 127 us).
+#include <algorithm>
+#include <climits>
+
+#include "common.cuh"
+#include "tma.cuh"
+
+namespace suppy {
+
+namespace {
+
+using tma::bulk_g2s;
+using tma::mbar_arrive;
+using tma::mbar_arrive_expect_tx;
+using tma::mbar_init;
+
+constexpr int kConsumers = kStripThreads / 32 - 1;    // consumer warps (and one producer)
+constexpr int kInFlight = kStripInFlight;             // strips in the ring: their barriers
+constexpr int kPad = 0xffff;                          // offset of an empty slot
+constexpr long long kDrainCycles = 4000000000LL;      // copies in flight get this long to land
+
+template <typename VT>
+struct Val4;
+template <>
+struct Val4<float> {
+    static __device__ __forceinline__ float4 load(const unsigned char* p) {
+        return *reinterpret_cast<const float4*>(p);
+    }
+};
+template <>
+struct Val4<__nv_bfloat16> {
+    static __device__ __forceinline__ float4 load(const unsigned char* p) {
+        const uint2 u = *reinterpret_cast<const uint2*>(p);
+        return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                           __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+    }
+};
+template <>
+struct Val4<__half> {
+    static __device__ __forceinline__ float4 load(const unsigned char* p) {
+        const uint2 u = *reinterpret_cast<const uint2*>(p);
+        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
+        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+};
+
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(tma::smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Bounded wait: gives up (false) when `abort` is raised or `limit` cycles pass
+// before the phase completes.
+__device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                             long long limit) {
+    if (mbar_test(bar, parity)) return true;
+    const long long t0 = clock64();
+    do {
+        if (*abort || clock64() - t0 > limit) return false;
+    } while (!tma::mbar_try_wait(bar, parity));
+    return true;
+}
+
+// Barrier of a consumer group that also decides whether every thread is ok.
+template <int NW>
+__device__ __forceinline__ bool group_all(int grp, bool ok) {
+    if constexpr (NW == 1) {
+        return __all_sync(0xffffffffu, ok);
+    } else {
+        int r;
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t"
+            "setp.ne.s32 q, %3, 0;\n\t"
+            "barrier.cta.red.and.pred p, %1, %2, q;\n\t"
+            "selp.s32 %0, 1, 0, p;\n\t}"
+            : "=r"(r)
+            : "r"(grp + 1), "r"(NW * 32), "r"((int)ok)
+            : "memory");
+        return r != 0;
+    }
+}
+
+template <typename VT>
+struct Packet {
+    static constexpr int kBytes = strip_packet_bytes(sizeof(VT));
+    static constexpr int kIdx = 16, kVal = 16 + 256;
+};
+
+// Gather and L2 reduction at x[base + o] unless o marks an empty slot, as
+// predicated instructions.
+__device__ __forceinline__ float gather(const float* x, int base, unsigned o) {
+    float g;
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %2, 65535;\n\t"
+        "mov.f32 %0, 0f00000000;\n\t"
+        "@p ld.global.nc.f32 %0, [%1];\n\t}"
+        : "=f"(g)
+        : "l"(x + (base + (int)o)), "r"(o));
+    return g;
+}
+__device__ __forceinline__ void reduce(float* x, int base, unsigned o, float v) {
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "setp.ne.u32 p, %1, 65535;\n\t"
+                 "@p red.global.add.f32 [%0], %2;\n\t}" ::"l"(x + (base + (int)o)),
+                 "r"(o), "f"(v)
+                 : "memory");
+}
+
+// N packets from p: their loads, then their gathers together, then the
+// products, so that they cost one gather latency.
+template <typename VT, int N>
+__device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, const float* __restrict__ x,
+                                            float& acc0, float& acc1) {
+    int base[N];
+    uint2 w[N];
+    float4 v[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const unsigned char* q = p + k * Packet<VT>::kBytes;
+        base[k] = *reinterpret_cast<const int*>(q + 4 * (lane >> 3));
+        w[k] = *reinterpret_cast<const uint2*>(q + Packet<VT>::kIdx + 8 * lane);
+        v[k] = Val4<VT>::load(q + Packet<VT>::kVal + lane * 4 * (int)sizeof(VT));
+    }
+    float g[N][4];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const unsigned o[4] = {w[k].x & 0xffffu, w[k].x >> 16, w[k].y & 0xffffu, w[k].y >> 16};
+#pragma unroll
+        for (int s = 0; s < 4; ++s) g[k][s] = gather(x, base[k], o[s]);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        acc0 = fmaf(v[k].x, g[k][0], acc0);
+        acc1 = fmaf(v[k].y, g[k][1], acc1);
+        acc0 = fmaf(v[k].z, g[k][2], acc0);
+        acc1 = fmaf(v[k].w, g[k][3], acc1);
+    }
+}
+
+// KIND 0: row pass, coefficients out; 1: row pass with the scatter by L2
+// reductions; 2: column pass.
+template <typename VT, int NW, int KIND>
+__global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
+    if (KIND == 2) {
+        if (a.epi.st[0].stopped) return;   // the row pass left no coefficients
+    } else if (a.check_stop && a.st[0].stopped) {
+        return;
+    }
+    extern __shared__ __align__(128) unsigned char ring[];
+    __shared__ __align__(8) uint64_t full[kInFlight], empty[kInFlight];
+    __shared__ float part[2][kConsumers][4];
+    __shared__ volatile int abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s0 = a.cta[blockIdx.x], s1 = a.cta[blockIdx.x + 1];
+    constexpr int NG = kConsumers / NW;
+    // a group waits for the fills of its own barriers only, in order: the wait
+    // for one fill can never be taken for the fill before it
+    static_assert(kInFlight % NG == 0, "a barrier's strips belong to one group");
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < kInFlight; ++k) {
+            mbar_init(&full[k], 1);
+            mbar_init(&empty[k], NW);
+        }
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    // the row pass's proximity terms: FP32 sums with Kahan compensation per
+    // thread (FP64 arithmetic is scarce on GB300), widened for the CTA's sum
+    float ps = 0.f, pc = 0.f;
+    int oldest = 0, issued = 0;   // producer: strips whose ring space came back, strips issued
+    if (warp == 0) {
+        uint64_t pol;
+        if (a.keep) asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+        else pol = tma::policy_evict_first();
+        // 32 strips at a time, one a lane: each goes out as soon as the strips
+        // whose ring space it takes have come back (the places in the ring
+        // were laid out with the records), so that a strip costs the producer
+        // one wait and one copy
+        int4 nxt = (s0 + lane < s1) ? a.meta[s0 + lane] : make_int4(0, 0, 0, 0);
+        bool ok = true;
+        for (int b = s0; ok && b < s1; b += 32) {
+            const int4 m = nxt;
+            nxt = (b + 32 + lane < s1) ? a.meta[b + 32 + lane] : make_int4(0, 0, 0, 0);
+            const int q = b - s0 + lane;
+            const int need = q - strip_live(m.w);
+            const uint32_t bytes = (uint32_t)((m.y & kStripPackets) * Packet<VT>::kBytes);
+            bool done = b + lane >= s1;
+            for (;;) {
+                if (!done && need <= oldest) {
+                    uint64_t* bar = &full[q % kInFlight];
+                    mbar_arrive_expect_tx(bar, bytes);
+                    if (bytes)
+                        bulk_g2s(ring + strip_at(m.w), a.blob + ((size_t)(unsigned)m.x << 4), bytes, bar, pol);
+                    done = true;
+                }
+                issued = b - s0 + __popc(__ballot_sync(0xffffffffu, done && b + lane < s1));
+                if (__all_sync(0xffffffffu, done)) break;
+                ok = __all_sync(0xffffffffu, bounded_wait(&empty[oldest % kInFlight], (oldest / kInFlight) & 1,
+                                                          &abort_flag, a.wait_cycles));
+                if (!ok) break;
+                ++oldest;
+            }
+        }
+        if (lane == 0 && !ok) {
+            abort_flag = 1;
+            atomicExch(a.err, 1);
+        }
+    } else {
+        const int cw = warp - 1, grp = cw / NW, wi = cw % NW;
+        const int r = lane >> 3;
+        int par = 0;
+        int4 nxt = (grp < s1 - s0) ? __ldg(a.meta + s0 + grp) : make_int4(0, 0, 0, 0);
+        for (int q = grp; q < s1 - s0; q += NG, par ^= 1) {
+            const int slot = q % kInFlight;
+            const int4 m = nxt;
+            nxt = (q + NG < s1 - s0) ? __ldg(a.meta + s0 + q + NG) : make_int4(0, 0, 0, 0);
+            const int npk = m.y & kStripPackets;
+            const bool tall = (m.y & kStripTall) != 0;
+            const int p0 = npk * wi / NW, p1 = npk * (wi + 1) / NW;
+            const int item = m.z + r;
+            const bool has = ((m.w >> r) & 1) != 0;   // a row with entries; a column of the strip
+            const unsigned char* strip = ring + strip_at(m.w);
+            float li = 0.f, ui = 0.f, w = 0.f, mul = 1.f;
+            if (KIND != 2 && has) {
+                li = __ldg(a.l + item);
+                ui = __ldg(a.u + item);
+                w = __ldg(a.wr + item);
+                const float* mp = a.coef_mul ? a.coef_mul : a.prox_mul;
+                if (mp) mul = __ldg(mp + item);
+            }
+            if (KIND == 2 && has && wi == 0) {
+                li = __ldg(a.lo + (a.box_len == 1 ? 0 : item));
+                ui = __ldg(a.hi + (a.box_len == 1 ? 0 : item));
+                w = a.xw[item];   // owned by this strip alone during the pass
+                if (a.zc) mul = __ldg(a.zc + item);
+            }
+            bool ok = bounded_wait(&full[slot], (q / kInFlight) & 1, &abort_flag, a.wait_cycles);
+            float dot = 0.f;
+            if (ok) {
+                const float* xs = tall ? a.xT : a.x;
+                float acc0 = 0.f, acc1 = 0.f;
+                int p = p0;
+                const unsigned char* sp = strip + p0 * Packet<VT>::kBytes;
+                for (; p + 4 <= p1; p += 4, sp += 4 * Packet<VT>::kBytes)
+                    dot_packets<VT, 4>(sp, lane, xs, acc0, acc1);
+                if (p1 - p == 3) dot_packets<VT, 3>(sp, lane, xs, acc0, acc1);
+                else if (p1 - p == 2) dot_packets<VT, 2>(sp, lane, xs, acc0, acc1);
+                else if (p1 - p == 1) dot_packets<VT, 1>(sp, lane, xs, acc0, acc1);
+                dot = acc0 + acc1;
+            }
+            if (KIND != 1) {
+                // the strip is read once: its ring space goes back now
+                __syncwarp();
+                if (ok && lane == 0) mbar_arrive(&empty[slot]);
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+            if (NW > 1 && (lane & 7) == 0) part[par][cw][r] = dot;
+            ok = group_all<NW>(grp, ok);
+            if (!ok) {
+                abort_flag = 1;
+                if (lane == 0) atomicExch(a.err, 1);
+                break;
+            }
+            if constexpr (NW > 1) {
+                // the other buffer takes the next strip's sums: a warp writes
+                // this one again only after the group's next barrier
+                dot = part[par][grp * NW][r];
+#pragma unroll
+                for (int k = 1; k < NW; ++k) dot += part[par][grp * NW + k][r];
+            }
+            if constexpr (KIND == 2) {
+                if (has && wi == 0 && (lane & 7) == 0) {
+                    const float s = a.zc ? dot * mul : dot;
+                    if (a.delta_out) a.delta_out[item] = s;
+                    else a.xw[item] = clampf(w + s, li, ui);
+                }
+            } else {
+                const float d = clampf(dot, li, ui) - dot;
+                const float coef = a.lam * w * d * (a.coef_mul ? mul : 1.f);
+                if (has && wi == 0 && (lane & 7) == 0) {
+                    const float t = d * d * w * (a.prox_mul ? mul : 1.f);
+                    const float y = t - pc, sum = ps + y;
+                    pc = (sum - ps) - y;
+                    ps = sum;
+                    if (KIND == 0 && a.coef) a.coef[item] = coef;
+                }
+                if constexpr (KIND == 1) {
+                    if (has && coef != 0.f) {
+                        float* dst = tall ? a.deltaT : a.delta;
+                        const unsigned char* sp = strip + p0 * Packet<VT>::kBytes;
+#pragma unroll 2
+                        for (int p = p0; p < p1; ++p, sp += Packet<VT>::kBytes) {
+                            const int base = *reinterpret_cast<const int*>(sp + 4 * r);
+                            const uint2 ix = *reinterpret_cast<const uint2*>(sp + Packet<VT>::kIdx + 8 * lane);
+                            const float4 v = Val4<VT>::load(sp + Packet<VT>::kVal + lane * 4 * (int)sizeof(VT));
+                            const unsigned o0 = ix.x & 0xffffu, o1 = ix.x >> 16, o2 = ix.y & 0xffffu,
+                                           o3 = ix.y >> 16;
+                            reduce(dst, base, o0, coef * v.x);
+                            reduce(dst, base, o1, coef * v.y);
+                            reduce(dst, base, o2, coef * v.z);
+                            reduce(dst, base, o3, coef * v.w);
+                        }
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&empty[slot]);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (abort_flag && threadIdx.x == 0) {
+        // let the copies in flight land before the CTA leaves
+        volatile int never = 0;
+        for (int q = oldest; q < issued; ++q)
+            tma::mbar_wait(&full[q % kInFlight], (q / kInFlight) & 1, &never, kDrainCycles);
+    }
+    if constexpr (KIND != 2) {
+        __shared__ double sw[kConsumers + 1];
+        const double v = warp_sum((double)ps - (double)pc);
+        if (lane == 0) sw[warp] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int k = 1; k <= kConsumers; ++k) s += sw[k];
+            a.pp[blockIdx.x] = s;
+        }
+    } else {
+        __syncthreads();
+        if (a.epi.last_seg && a.ticket) {
+            // the last CTA to finish runs the sweep epilogue: every CTA of the
+            // launch has read the stop flag by then, so the flag it may set is
+            // seen by the next launch only
+            __shared__ bool last;
+            __threadfence();
+            if (threadIdx.x == 0) last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+            __syncthreads();
+            if (last) {
+                __threadfence();
+                sweep_epilogue(a.epi);
+                if (threadIdx.x == 0) *a.ticket = 0u;
+            }
+        } else if (blockIdx.x == 0 && !a.epi.last_seg) {
+            sweep_epilogue(a.epi);
+        }
+    }
+}
+
+// ------------------------------------------------------------- building ----
+// One CTA of four warps per strip, warp r for item r: the item's entries as
+// keys in the order the strip walks them, then windows of at most 32 entries
+// an item, each window one packet.  Keys: on an image grid the pixel in
+// row-major order for strips whose rows run down the image and column-major
+// order for the others (so that a ray's entries come in the order of its
+// path), else the index itself.  A window ends at the smallest key that an
+// item could not take (its 33rd entry, or one whose offset from the window's
+// smallest position would not fit 16 bits): all items of the strip then stop
+// at the same place.  FILL 0 counts the packets and writes the strip's
+// record, FILL 1 writes the packets.
+template <typename VT, int FILL>
+__global__ void __launch_bounds__(128) k_strip_build(const StripBuild b) {
+    extern __shared__ unsigned key_s[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned* raw = key_s + (size_t)warp * 2 * b.max_len;
+    unsigned* key = raw + b.max_len;
+    unsigned short* ord = reinterpret_cast<unsigned short*>(key_s + (size_t)8 * b.max_len) +
+                          (size_t)warp * b.max_len;
+    __shared__ int span_s[4][2], cnt_s[4], len_s[4];
+    __shared__ unsigned lim_s[4];
+    const VT* val = static_cast<const VT*>(b.val);
+    for (int t = blockIdx.x; t < b.nstrips; t += gridDim.x) {
+        const int4 st = b.strips[t];   // first item in info, items, first item's number
+        const int2 inf = warp < st.y ? b.info[st.x + warp] : make_int2(0, 0);
+        const int len = inf.y;
+        const int* idx = b.idx + inf.x;
+        int r0 = INT_MAX, r1 = -1, c0 = INT_MAX, c1 = -1;
+        if (b.W > 0)
+            for (int e = lane; e < len; e += 32) {
+                const int y = idx[e] / b.W, x = idx[e] - y * b.W;
+                r0 = min(r0, y);
+                r1 = max(r1, y);
+                c0 = min(c0, x);
+                c1 = max(c1, x);
+            }
+        r0 = __reduce_min_sync(0xffffffffu, r0);
+        r1 = __reduce_max_sync(0xffffffffu, r1);
+        c0 = __reduce_min_sync(0xffffffffu, c0);
+        c1 = __reduce_max_sync(0xffffffffu, c1);
+        if (lane == 0) {
+            span_s[warp][0] = r1 < 0 ? 0 : r1 - r0;
+            span_s[warp][1] = c1 < 0 ? 0 : c1 - c0;
+            len_s[warp] = len;
+        }
+        __syncthreads();
+        const bool tall = b.W > 0 && span_s[0][0] + span_s[1][0] + span_s[2][0] + span_s[3][0] >
+                                         span_s[0][1] + span_s[1][1] + span_s[2][1] + span_s[3][1];
+        bool sorted = true;
+        for (int e = lane; e < len; e += 32) {
+            const int c = idx[e];
+            unsigned k = (unsigned)c;
+            if (b.W > 0 && !tall) {
+                const int y = c / b.W;
+                k = (unsigned)((c - y * b.W) * b.H + y);
+            }
+            raw[e] = k;
+        }
+        __syncwarp();
+        for (int e = lane; e + 1 < len; e += 32) sorted = sorted && raw[e] <= raw[e + 1];
+        sorted = __all_sync(0xffffffffu, sorted);
+        for (int e = lane; e < len; e += 32) {
+            const unsigned k = raw[e];
+            int rank = e;
+            if (!sorted) {
+                rank = 0;
+                for (int f = 0; f < len; ++f) rank += raw[f] < k || (raw[f] == k && f < e);
+            }
+            key[rank] = k;
+            ord[rank] = (unsigned short)e;
+        }
+        __syncwarp();
+        int p = 0, npk = 0;
+        unsigned char* out = FILL ? b.blob + ((size_t)(unsigned)b.meta[t].x << 4) : nullptr;
+        const bool tall_pos = FILL ? (b.meta[t].y & kStripTall) != 0 : tall;
+        for (;;) {
+            const int left = len - p;
+            if (!__syncthreads_or(left > 0)) break;
+            int pos = 0, src = 0;
+            if (lane < left) {
+                src = inf.x + ord[p + lane];
+                const int c = b.idx[src];
+                pos = b.patch ? patch_index(c, b.recipW, b.W, b.Wp, tall_pos) : c;
+            }
+            // running extremes of the positions over the window
+            int mn = lane < left ? pos : INT_MAX, mx = lane < left ? pos : INT_MIN;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int a0 = __shfl_up_sync(0xffffffffu, mn, o), a1 = __shfl_up_sync(0xffffffffu, mx, o);
+                if (lane >= o) {
+                    mn = min(mn, a0);
+                    mx = max(mx, a1);
+                }
+            }
+            const bool fits = lane < left && (long long)mx - mn < kPad;
+            const int c = __popc(__ballot_sync(0xffffffffu, fits));   // a prefix of the lanes
+            if (lane == 0) lim_s[warp] = p + c < len ? key[p + c] : 0xffffffffu;
+            __syncthreads();
+            const unsigned lim = min(min(lim_s[0], lim_s[1]), min(lim_s[2], lim_s[3]));
+            int n = __popc(__ballot_sync(0xffffffffu, lane < c && key[p + lane] < lim));
+            if (lane == 0) cnt_s[warp] = n;
+            __syncthreads();
+            // equal keys (repeated columns) may leave nothing below the limit
+            if (cnt_s[0] + cnt_s[1] + cnt_s[2] + cnt_s[3] == 0) n = c;
+            if constexpr (FILL) {
+                const int base = n > 0 ? __shfl_sync(0xffffffffu, mn, n - 1) : 0;
+                unsigned char* q = out + (size_t)npk * strip_packet_bytes(sizeof(VT));
+                if (lane == 0) reinterpret_cast<int*>(q)[warp] = base;
+                const int L = warp * 8 + (lane & 7), s = lane >> 3;
+                reinterpret_cast<unsigned short*>(q + 16)[L * 4 + s] =
+                    lane < n ? (unsigned short)(pos - base) : (unsigned short)kPad;
+                reinterpret_cast<VT*>(q + 16 + 256)[L * 4 + s] = lane < n ? val[src] : VT(0.f);
+            }
+            p += n;
+            ++npk;
+        }
+        if (!FILL && threadIdx.x == 0) {
+            int mask = 0;
+            for (int r = 0; r < st.y; ++r)
+                if (b.all_items || len_s[r] > 0) mask |= 1 << r;
+            b.meta[t] = make_int4(0, npk | (tall ? kStripTall : 0), st.z, mask);
+        }
+        __syncthreads();
+    }
+}
+
+using StripFn = void (*)(StripArgs);
+
+template <typename VT, int KIND>
+StripFn pick_nw(int nw) {
+    switch (nw) {
+        case 1: return k_strip<VT, 1, KIND>;
+        case 2: return k_strip<VT, 2, KIND>;
+        default: return k_strip<VT, 4, KIND>;
+    }
+}
+
+template <typename VT>
+StripFn pick_kind(int kind, int nw) {
+    if (kind == 0) return pick_nw<VT, 0>(nw);
+    return kind == 1 ? pick_nw<VT, 1>(nw) : pick_nw<VT, 2>(nw);
+}
+
+StripFn strip_fn(suppy_dtype dt, int kind, int nw) {
+    if (dt == SUPPY_F32) return pick_kind<float>(kind, nw);
+    if (dt == SUPPY_BF16) return pick_kind<__nv_bfloat16>(kind, nw);
+    return pick_kind<__half>(kind, nw);
+}
+
+template <typename VT>
+cudaError_t build(const StripBuild& b, int fill, int grid, cudaStream_t s) {
+    const size_t smem = (size_t)b.max_len * 4 * (2 * sizeof(unsigned) + sizeof(unsigned short));
+    auto f = fill ? k_strip_build<VT, 1> : k_strip_build<VT, 0>;
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    f<<<grid, 128, smem, s>>>(b);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_strip(const StripArgs& a, suppy_dtype dt, int kind, int nw, int grid, cudaStream_t s) {
+    StripFn f = strip_fn(dt, kind, nw);
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, a.ring);
+    if (e != cudaSuccess) return e;
+    f<<<grid, kStripThreads, a.ring, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_strip_build(const StripBuild& b, suppy_dtype dt, int fill, cudaStream_t s) {
+    if (b.nstrips < 1) return cudaSuccess;
+    if (b.max_len < 1 || b.max_len > kStripMaxItem) return cudaErrorInvalidValue;
+    const int grid = std::min(b.nstrips, 152 * 64);
+    if (dt == SUPPY_F32) return build<float>(b, fill, grid, s);
+    if (dt == SUPPY_BF16) return build<__nv_bfloat16>(b, fill, grid, s);
+    return build<__half>(b, fill, grid, s);
+}
+
+}  // namespace suppy
