@@ -185,7 +185,7 @@ typedef struct {
      * applied -- the same choice as the sequential trial loop -- and grid
      * barriers between passes; several right-hand sides one after the
      * other); 1 -- one thread-block cluster per right-hand side; 0 --
-     * automatic: 2 for one right-hand side with n >= 65536, else 1. */
+     * automatic: 2 for one right-hand side with n >= 32768, else 1. */
     int32_t perturb_path;
     /* Lane map of the streaming passes: 0 automatic (measured when tune is
      * set), 1 four consecutive elements per lane (16-byte ring reads),

@@ -208,8 +208,11 @@ struct suppy_ctx {
     // whole-GPU perturbation phase (one cooperative launch)
     bool wide = false;
     int wide_grid = 0;
+    bool wide_tiled = false;        // its tile-resident form (else the image does not fit shared memory)
+    PhaseTiles wtiles;
     double* d_wpart = nullptr;
-    unsigned* d_ticket = nullptr;   // grid barrier of the whole-GPU perturbation {count, generation}
+    unsigned* d_ticket = nullptr;   // grid barrier of the whole-GPU perturbation: {count, generation}, or
+                                    // 64-bit {count, count at the launch} (tile-resident form)
     std::vector<long long> rpref;   // row-work prefix (m + 1)
     // split feasibility: dose rows A_q (CSR and CSC), structures, DVCs
     bool dvc_on = false;
@@ -1065,7 +1068,7 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
 // one-pass sweep that follows it (whole-GPU phase, patch numbering), and
 // *copies says whether it does.
 suppy_status enqueue_perturb(suppy_ctx* c, const suppy_params* p, int record_only, bool* copies = nullptr) {
-    PerturbArgs a;
+    PerturbArgs a{};
     a.x = c->d_x;
     a.g = c->d_g;
     a.c32 = c->d_c32;
@@ -1104,7 +1107,8 @@ suppy_status enqueue_perturb(suppy_ctx* c, const suppy_params* p, int record_onl
     Timed tm{c, 2};
     CK(tm.begin());
     if (c->wide && !record_only) {
-        CK(launch_perturb_wide(a, c->wide_grid, c->stream));
+        if (c->wide_tiled) CK(launch_phase_tiles(a, c->wtiles, c->stream));
+        else CK(launch_perturb_wide(a, c->wide_grid, c->stream));
         note_launch(c);
     } else {
         CK(launch_perturb(a, c->perturb_cluster, c->stream));
@@ -1943,7 +1947,7 @@ suppy_status build_tile(suppy_ctx* c, const std::vector<int>& rp, const int* hco
 // counters) after a bounded wait gave up: a CTA that left early may have left
 // a count behind.
 suppy_status reset_sync_words(suppy_ctx* c) {
-    if (c->d_ticket) CK(cudaMemsetAsync(c->d_ticket, 0, 2 * sizeof(unsigned), c->stream));
+    if (c->d_ticket) CK(cudaMemsetAsync(c->d_ticket, 0, 4 * sizeof(unsigned), c->stream));
     if (c->d_cticket) CK(cudaMemsetAsync(c->d_cticket, 0, sizeof(unsigned), c->stream));
     if (c->d_xticket) CK(cudaMemsetAsync(c->d_xticket, 0, sizeof(unsigned), c->stream));
     if (c->d_vticket) CK(cudaMemsetAsync(c->d_vticket, 0, sizeof(unsigned), c->stream));
@@ -2385,11 +2389,13 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         // cluster's per-pixel work); with two or more right-hand sides their
         // clusters already share the GPU, while the whole-GPU kernel takes
         // them one after the other, so the cluster path is faster; 2 forces
-        // it, 1 disables it
+        // it, 1 disables it.  At 65317 pixels the phase took 16.8 us in a
+        // cluster of 16 and 12.5 us on the whole GPU, at 16384 10.0 and
+        // about 12 us
         // (its pixel loops step an int index by the grid's thread count)
         const bool wide_fits = (long long)c->n + 2LL * sms * kPhaseThreads < (long long)INT_MAX;
         if (wide_fits && (o->perturb_path == 2 ||
-                          (o->perturb_path == 0 && (long long)nB >= 65536 && c->B == 1))) {
+                          (o->perturb_path == 0 && (long long)nB >= 32768 && c->B == 1))) {
             // a cooperative launch: every CTA must be resident at once
             const int per_sm = std::min(1, wide_phase_blocks_per_sm());
             if (per_sm < 1) return fail(c, SUPPY_ECUDA, "whole-GPU perturbation kernel cannot be resident");
@@ -2397,9 +2403,11 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
             c->wide_grid = (int)std::max<long long>(
                 1, std::min<long long>((long long)per_sm * sms,
                                        ((long long)c->n + kPhaseThreads - 1) / kPhaseThreads));
+            c->wide_tiled = wide_phase_tiles((int)c->obj, n, c->H, c->W, sms, &c->wtiles);
+            if (c->wide_tiled) c->wide_grid = c->wtiles.TR * c->wtiles.TC;
             if ((s = dalloc(c, &c->d_wpart, wide_part_doubles(c->wide_grid))) != SUPPY_OK) return s;
-            if ((s = dalloc(c, &c->d_ticket, 2)) != SUPPY_OK) return s;
-            CK(cudaMemsetAsync(c->d_ticket, 0, 2 * sizeof(unsigned), c->stream));
+            if ((s = dalloc(c, &c->d_ticket, 4)) != SUPPY_OK) return s;
+            CK(cudaMemsetAsync(c->d_ticket, 0, 4 * sizeof(unsigned), c->stream));
         }
     }
     if ((s = dalloc(c, &c->d_st, (size_t)c->B)) != SUPPY_OK) return s;

@@ -157,6 +157,14 @@ struct PerturbArgs {
     float* pA;
     float* pB;
     int pWp;
+    // tile-resident phase: TR x TC rectangles of at most tmh x tmw pixels
+    int TR, TC, tmh, tmw;
+    int th, tw, xh, xw;
+    unsigned mP0, mP1, mG0, mG1;
+};
+
+struct PhaseTiles {
+    int TR = 1, TC = 1, h = 1, w = 1;   // rectangles per column and row, largest one
 };
 
 // Threads per CTA of the whole-GPU reduction kernels (variance rule), of the
@@ -463,6 +471,10 @@ cudaError_t launch_perturb(const PerturbArgs& a, int cluster, cudaStream_t s);
 // `grid` CTAs of kPhaseThreads threads, all resident (subgradient pass,
 // kWideTrials trial evaluations per pass, update, grid barriers between).
 cudaError_t launch_perturb_wide(const PerturbArgs& a, int grid, cudaStream_t s);
+// The tile-resident form of the phase on the whole GPU: its rectangles (false
+// when they do not fit shared memory), and one cooperative launch.
+bool wide_phase_tiles(int obj, int n, int H, int W, int sms, PhaseTiles* out);
+cudaError_t launch_phase_tiles(const PerturbArgs& a, const PhaseTiles& t, cudaStream_t s);
 size_t wide_part_doubles(int grid);   // partials the whole-GPU kernel needs
 int wide_phase_blocks_per_sm();       // its resident CTAs per SM
 int choose_perturb_cluster(int n, int B);

@@ -10,6 +10,9 @@
 // every CTA sums them in the same order -- so all CTAs take the same decision
 // and the run is bitwise reproducible.  The trial loop is bounded by
 // max_trials, so the kernel always ends.
+#include <algorithm>
+#include <type_traits>
+
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -76,10 +79,10 @@ __device__ __forceinline__ float trial_scale(double gamma, double log2_alpha, lo
 // phase that starts at f_start -- fixed, or the lowest phase-start objective
 // so far, this one included -- and beta / ||g|| = (f - f_ref) / ||g||^2, the
 // subgradient projection onto the level set of f's linearisation.
-__device__ __forceinline__ double adaptive_ref(const PerturbArgs& a, const RhsState& st,
+__device__ __forceinline__ double adaptive_ref(const PerturbArgs& a, bool has_ref, double st_ref,
                                                double f_start) {
     if (a.adaptive == 2) return a.f_ref;
-    return st.has_ref ? fmin(st.f_ref, f_start) : f_start;
+    return has_ref ? fmin(st_ref, f_start) : f_start;
 }
 
 __device__ __forceinline__ float adaptive_scale(double fy, double f_ref, double gg) {
@@ -162,6 +165,10 @@ __device__ __forceinline__ float subgrad(int obj, int p, int H, int W, const flo
     if (j > 0) g += sgnf(y0 - y(p - 1));
     return g;
 }
+
+// dx^2 + dy^2 with one rounding order wherever a TV term is formed, so that
+// equal images give equal objective values.
+__device__ __forceinline__ float sq2(float dx, float dy) { return __fmaf_rn(dx, dx, __fmul_rn(dy, dy)); }
 
 // Per-thread compensated FP32 sum (Kahan), handed to the CTA and cluster
 // reductions as a float-float value.  FP64 arithmetic is scarce on GB300: one
@@ -249,13 +256,13 @@ struct StepDecision {
     float inv_gnorm, asc;
 };
 
-__device__ __forceinline__ StepDecision step_decision(const PerturbArgs& a, const RhsState& st,
+__device__ __forceinline__ StepDecision step_decision(const PerturbArgs& a, bool has_ref, double st_ref,
                                                       double gg, double fy, double f_start) {
     StepDecision d{0, 0.f, 0.f};
     if (a.record_only || gg == 0.0) return d;
     d.inv_gnorm = 1.0f / sqrtf((float)gg);
     if (a.adaptive) {
-        const double f_ref = adaptive_ref(a, st, f_start);
+        const double f_ref = adaptive_ref(a, has_ref, st_ref, f_start);
         if (!(fy > f_ref)) return d;
         d.asc = adaptive_scale(fy, f_ref, gg);
     }
@@ -294,7 +301,7 @@ __device__ __forceinline__ void phase_end(const PerturbArgs& a, RhsState& st, co
     st.f_valid = 1;
     if (a.record_only) return;
     if (a.adaptive == 1) {
-        st.f_ref = adaptive_ref(a, st, f_start);
+        st.f_ref = adaptive_ref(a, st.has_ref != 0, st.f_ref, f_start);
         st.has_ref = 1;
     }
     st.ell = ell;
@@ -325,6 +332,9 @@ __global__ void __launch_bounds__(kPerturbThreads) k_perturb(const PerturbArgs a
     Vec g{a.g + b, a.B};
 
     const PhaseStart ps = phase_start(a, b);
+    // read before the first barrier: rank 0 rewrites it at the phase's end
+    const bool has_ref = st.has_ref != 0;
+    const double st_ref = st.f_ref;
     long long ell = ps.ell;
     int accepted = 0, trials = 0;
     double f_start = 0.0;   // thread 0 of each CTA
@@ -352,7 +362,7 @@ __global__ void __launch_bounds__(kPerturbThreads) k_perturb(const PerturbArgs a
                 f_start = fy;
                 have_f = true;
             }
-            dec = step_decision(a, st, r.x, fy, f_start);
+            dec = step_decision(a, has_ref, st_ref, r.x, fy, f_start);
         }
         __syncthreads();
         if (!dec.go) break;
@@ -394,34 +404,14 @@ __global__ void __launch_bounds__(kPerturbThreads) k_perturb(const PerturbArgs a
     if (rank == 0 && threadIdx.x == 0) phase_end(a, st, ps, ell, accepted, trials, f_start);
 }
 
-// ------------------------------------------- shared-memory resident phase ----
-// Same algorithm as k_perturb, with the right-hand side's iterate and
-// subgradient held in the shared memory of the cluster for the whole phase:
-// CTA r owns image rows [R_r, R_{r+1}) (TV) or elements [P_r, P_{r+1})
-// (linear); the one halo row above and below a band is read from the
-// neighbouring CTA's shared memory (distributed shared memory).  HBM / L2
-// see one read and one write of x per phase.
-struct Band {
-    const float* own;
-    const float* up;     // previous rank's band (DSMEM) or null
-    const float* down;   // next rank's band (DSMEM) or null
-    int r0, r1, up_r0, W;
-    __device__ __forceinline__ float operator()(int i, int j) const {
-        if (i >= r0 && i < r1) return own[(i - r0) * W + j];
-        if (i < r0) return up[(i - up_r0) * W + j];
-        return down[j];
-    }
-};
-
-__device__ __forceinline__ int band_start(int r, int H, int cs) { return (int)((long long)H * r / cs); }
-
+// ------------------------------------------------------ stencil helpers ----
 template <class Y>
 __device__ __forceinline__ float tv_term(int obj, int i, int j, int H, int W, const Y& y) {
     const float y0 = y(i, j);
     if (obj == SUPPY_OBJ_TV_ISO) {
         if (i < H - 1 && j < W - 1) {
             const float dx = y(i + 1, j) - y0, dy = y(i, j + 1) - y0;
-            return sqrtf(dx * dx + dy * dy);
+            return sqrtf(sq2(dx, dy));
         }
         return 0.f;
     }
@@ -439,19 +429,19 @@ __device__ __forceinline__ float tv_subgrad(int obj, int i, int j, int H, int W,
         // each term contributes (its partial derivative) * 1/phi, phi = 0 -> 0
         if (i < H - 1 && j < W - 1) {
             const float dx = y(i + 1, j) - y0, dy = y(i, j + 1) - y0;
-            const float q = dx * dx + dy * dy;
+            const float q = sq2(dx, dy);
             if (q > 0.f) g -= (dx + dy) * rsqrtf(q);
         }
         if (i > 0 && j < W - 1) {
             const float ym = y(i - 1, j);
             const float dx = y0 - ym, dy = y(i - 1, j + 1) - ym;
-            const float q = dx * dx + dy * dy;
+            const float q = sq2(dx, dy);
             if (q > 0.f) g += dx * rsqrtf(q);
         }
         if (j > 0 && i < H - 1) {
             const float yl = y(i, j - 1);
             const float dx = y(i + 1, j - 1) - yl, dy = y0 - yl;
-            const float q = dx * dx + dy * dy;
+            const float q = sq2(dx, dy);
             if (q > 0.f) g += dy * rsqrtf(q);
         }
         return g;
@@ -484,142 +474,454 @@ struct StrideWalk {
     }
 };
 
-__global__ void __launch_bounds__(kPerturbThreads) k_perturb_smem(const PerturbArgs a) {
-    extern __shared__ float smem[];
-    cg::cluster_group cluster = cg::this_cluster();
-    __shared__ FF swf[2 * (kPerturbThreads / 32)];
-    __shared__ double2 scta, sres;
-    __shared__ StepDecision dec;
-    __shared__ float sc_s;
-    const int cs = (int)cluster.num_blocks();
-    const int b = blockIdx.x / cs;
-    RhsState& st = a.st[b];
-    if (st.stopped) return;
-    const PhaseStart ps = phase_start(a, b);
-    const int rank = (int)cluster.block_rank();
-    const bool lin = (a.obj == SUPPY_OBJ_LINEAR);
-    const bool elem = elementwise(a.obj);
-    const int H = elem ? a.n : a.H, W = elem ? 1 : a.W;   // element-wise: a column of n "rows"
-    const int r0 = band_start(rank, H, cs), r1 = band_start(rank + 1, H, cs);
-    int band = (r1 - r0) * W;
-    const int maxband = ((H + cs - 1) / cs) * W;
-    if (!PCHECKED(band >= 0 && band <= maxband && (elem || cs <= H), 401, rank)) band = 0;
-    float* ys = smem;
-    float* gs = smem + maxband;
-    float* X = a.x + b;
-    const int B = a.B;
-    const int p0 = r0 * W;
-    for (int q = threadIdx.x; q < band; q += kPerturbThreads) {
-        ys[q] = X[(size_t)(p0 + q) * B];
-        if (lin) gs[q] = a.c32[p0 + q];
-    }
-    cluster.sync();
-    Band yb{ys, nullptr, nullptr, r0, r1, 0, W};
-    Band gb{gs, nullptr, nullptr, r0, r1, 0, W};
-    if (!elem) {
-        if (rank > 0) {
-            yb.up = cluster.map_shared_rank(ys, rank - 1);
-            gb.up = cluster.map_shared_rank(gs, rank - 1);
-            yb.up_r0 = gb.up_r0 = band_start(rank - 1, H, cs);
+// The values a TV term of pixel (i, j) reads at every trial point z = y - s g:
+// y and g at (i, j), (i + 1, j) and (i, j + 1), loaded once per pixel.
+struct TvNbr {
+    float y0, g0, yd, gd, yr, gr;
+    bool down, right;
+};
+
+__device__ __forceinline__ TvNbr tv_nbr(int i, int j, int H, int W, const float* y, const float* g,
+                                        int B) {
+    const size_t p = (size_t)i * W + j;
+    TvNbr t;
+    t.down = i < H - 1;
+    t.right = j < W - 1;
+    t.y0 = y[p * B];
+    t.g0 = g[p * B];
+    t.yd = t.down ? y[(p + W) * B] : 0.f;
+    t.gd = t.down ? g[(p + W) * B] : 0.f;
+    t.yr = t.right ? y[(p + 1) * B] : 0.f;
+    t.gr = t.right ? g[(p + 1) * B] : 0.f;
+    return t;
+}
+
+// TV term at the trial point with step s (computed as in the cluster kernels).
+__device__ __forceinline__ float tv_trial_term(int obj, const TvNbr& t, float s) {
+    const float z0 = trial(t.y0, t.g0, s);
+    if (obj == SUPPY_OBJ_TV_ISO) {
+        if (t.down && t.right) {
+            const float dx = trial(t.yd, t.gd, s) - z0;
+            const float dy = trial(t.yr, t.gr, s) - z0;
+            return sqrtf(sq2(dx, dy));
         }
-        if (rank < cs - 1) {
-            yb.down = cluster.map_shared_rank(ys, rank + 1);
-            gb.down = cluster.map_shared_rank(gs, rank + 1);
+        return 0.f;
+    }
+    float v = 0.f;
+    if (t.down) v += fabsf(trial(t.yd, t.gd, s) - z0);
+    if (t.right) v += fabsf(trial(t.yr, t.gr, s) - z0);
+    return v;
+}
+
+// -------------------------------------------------- tile-resident phase ----
+// Same algorithm as k_perturb with every CTA's share of the image held in
+// shared memory for the whole phase: the image is cut into a TR x TC grid of
+// rectangles (element-wise objectives: into ranges), one per CTA, and a CTA
+// loads its rectangle of y with a halo once, computes the subgradient on it
+// (and on the one row and column the trial terms reach into), and evaluates
+// the trial points from shared memory.  HBM / L2 see one read and one write of
+// x per phase.  The CTAs of a right-hand side meet only in the sums that the
+// decisions need, and every CTA takes the same decisions from the same FP64
+// sums.  Two forms:
+//  * GRID false: one thread-block cluster per right-hand side; the CTA sums
+//    travel to every CTA's shared memory before one cluster barrier;
+//  * GRID true: the whole GPU (a cooperative launch) for one right-hand side
+//    after the other; the CTA sums go through L2 and one counter.
+// The phase is bound by the latency of its two reductions and of the loads, so
+// what was taken out is serial work: all loads of a thread in flight together,
+// warps reduce in parallel, one barrier a reduction, no second copy of the
+// image in L2.  Measured (GB300, isotropic TV, one step): cluster form, 64x64
+// 22.4 -> 9.5 us, 128x128 22.6 -> 10.0 us; whole GPU, 512x512 25.1 -> 15.6 us,
+// 1024x1024 45.9 -> 24.0 us; 16 images of 256x512 77.7 -> 61.6 us (before: image
+// bands read element by element through the neighbours' shared memory, sums
+// by one thread per CTA, and in the whole-GPU form y and g re-read from L2
+// with a barrier of 5 us around a last CTA's reduction).
+constexpr int kFirstTrials = 1;   // trial points of a step's first pass (the first usually passes)
+constexpr int kMaxCluster = 16;
+
+__device__ __forceinline__ FF ff_warp(FF a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        a = ff_add(a, FF{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)});
+    return a;
+}
+
+// q / d for q d < 2^32 and d >= 2, m = ceil(2^32 / d).
+__device__ __forceinline__ int div_by(int q, unsigned m) { return (int)__umulhi((unsigned)q, m); }
+
+template <bool GRID, int NT>
+struct PhaseSums {
+    FF* sw;                      // NT / 32 x kWideTrials warp sums
+    FF* peer;                    // cluster: 2 x kMaxCluster x kWideTrials CTA sums, written by every CTA
+    double* part;                // grid: 2 x tiles x kWideTrials CTA sums
+    unsigned long long* bar;     // grid: arrivals; [1] their count when the launch began
+    unsigned long long target;   // grid, thread 0: arrivals at the next barrier's end
+    int* err;
+    long long limit;
+    int* flag;                   // shared
+    int rank, tiles, par;
+
+    // Every CTA's writes before are visible to every CTA after; false on
+    // timeout (whole CTA alike).
+    __device__ bool barrier() {
+        if constexpr (!GRID) {
+            if (tiles > 1) cg::this_cluster().sync();
+            else __syncthreads();
+            return true;
+        } else {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int ok = 1;
+                target += (unsigned long long)tiles;
+                // release: the CTA's writes ordered before by the barrier above
+                asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(bar), "l"(1ULL) : "memory");
+                const long long t0 = clock64();
+                for (int k = 0;; ++k) {
+                    unsigned long long v;
+                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(bar) : "memory");
+                    if (v >= target) break;
+                    if (clock64() - t0 > limit || ((k & 63) == 63 && *(volatile int*)err)) {
+                        atomicExch(err, 2);
+                        ok = 0;
+                        break;
+                    }
+                }
+                *flag = ok;
+            }
+            __syncthreads();
+            return *flag != 0;
         }
     }
 
-    long long ell = ps.ell;
-    int accepted = 0, trials = 0;
-    double f_start = 0.0;   // thread 0 of each CTA
-    bool have_f = false;
-    for (int s = 0; s < (a.record_only ? 1 : a.n_red); ++s) {
-        KSum kg, kf;
-        double fl = 0.0;
-        {
-            StrideWalk px(threadIdx.x, kPerturbThreads, W);
-            for (int q = threadIdx.x; q < band; q += kPerturbThreads, px.next()) {
-                if (lin) {
-                    const int p = p0 + q;
-                    fl += a.c64[p] * (double)ys[q];
-                    const float gp = gs[q];
-                    kg.add(gp * gp);
-                } else if (elem) {
-                    kf.add(norm_term(a.obj, ys[q]));
-                    if (!a.record_only) {
-                        const float gp = norm_grad(a.obj, ys[q]);
-                        gs[q] = gp;
-                        kg.add(gp * gp);
+    // Sums of NV values over every thread of the right-hand side's CTAs, in a
+    // fixed order: float-float over lanes, then warps, FP64 over the CTAs.
+    // Warp k's `out` is the sum of value k.
+    template <int NV>
+    __device__ bool sum(FF (&v)[NV], double& out) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        constexpr int NW = NT / 32;
+        static_assert(NV <= NW && NV <= kWideTrials && NW <= 32, "one warp a value, one lane a warp sum");
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            v[k] = ff_warp(v[k]);
+            if (lane == 0) sw[warp * kWideTrials + k] = v[k];
+        }
+        __syncthreads();
+        FF s{0.f, 0.f};
+        if (warp < NV) {
+            if (lane < NW) s = sw[lane * kWideTrials + warp];
+            s = ff_warp(s);
+        }
+        if (!GRID && tiles == 1) {
+            out = (double)s.hi + (double)s.lo;
+            return true;
+        }
+        if (warp < NV) {
+            if constexpr (GRID) {
+                if (lane == 0)
+                    __stcg(part + ((size_t)par * tiles + rank) * kWideTrials + warp, (double)s.hi + (double)s.lo);
+            } else if (lane < tiles) {
+                FF* dst = cg::this_cluster().map_shared_rank(peer, lane);
+                dst[(par * kMaxCluster + rank) * kWideTrials + warp] = s;
+            }
+        }
+        const bool ok = barrier();
+        if (ok && warp < NV) {
+            double t = 0.0;
+            if constexpr (GRID) {
+                // five loads in flight: one round trip for up to 160 CTAs
+                for (int c = lane; c < tiles; c += 160) {
+                    double p[5];
+#pragma unroll
+                    for (int u = 0; u < 5; ++u)
+                        p[u] = c + 32 * u < tiles
+                                   ? __ldcg(part + ((size_t)par * tiles + c + 32 * u) * kWideTrials + warp)
+                                   : 0.0;
+                    t += ((p[0] + p[1]) + (p[2] + p[3])) + p[4];
+                }
+                out = warp_sum(t);
+            } else {
+                if (lane < tiles) {
+                    const FF p = peer[(par * kMaxCluster + lane) * kWideTrials + warp];
+                    t = (double)p.hi + (double)p.lo;
+                }
+                for (int o = tiles >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                out = t;   // tiles is a power of two
+            }
+        }
+        // the next sum uses the other buffer; this one is written again only
+        // after the barrier of that sum, which every CTA reaches after reading
+        par ^= 1;
+        return ok;
+    }
+};
+
+// KIND 0 isotropic TV, 1 anisotropic TV, 2 element-wise objectives.
+template <int KIND, bool GRID, int NT>
+__global__ void __launch_bounds__(NT) k_phase(const PerturbArgs a) {
+    extern __shared__ float smem[];
+    __shared__ FF sw[(NT / 32) * kWideTrials];
+    __shared__ FF peer[GRID ? 1 : 2 * kMaxCluster * kWideTrials];
+    __shared__ double gy_s[2];              // ||g||^2, f(y)
+    __shared__ float pow_s[kWideTrials];    // gamma alpha^(l + j)
+    __shared__ int pass_s[kWideTrials];     // trial j passed
+    __shared__ StepDecision dec;
+    __shared__ int flag;
+    const int tiles = a.TR * a.TC;
+    const int tile = GRID ? (int)blockIdx.x : (int)(blockIdx.x % tiles);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n = a.n, B = a.B, obj = a.obj;
+    const int H = KIND == 2 ? 1 : a.H, W = KIND == 2 ? n : a.W;
+    // the first xh rows (xw columns) of rectangles are one pixel larger
+    const int ti = (int)((unsigned)tile / (unsigned)a.TC), tj = tile - ti * a.TC;
+    const int h = a.th + (ti < a.xh ? 1 : 0), w = a.tw + (tj < a.xw ? 1 : 0), own = h * w;
+    const int r0 = ti * a.th + min(ti, a.xh), c0 = tj * a.tw + min(tj, a.xw);
+    const bool lin = KIND == 2 && obj == SUPPY_OBJ_LINEAR;
+    // y with a halo of one pixel up / left and two down / right (the
+    // subgradient is needed one pixel down / right of the rectangle)
+    const int P = KIND == 2 ? w : w + 3, PG = KIND == 2 ? w : w + 1;
+    float* ys = smem;
+    float* gs = smem + (KIND == 2 ? a.tmw : (a.tmh + 3) * (a.tmw + 3));
+    const int ylen = KIND == 2 ? own : (h + 3) * P, glen = KIND == 2 ? own : (h + 1) * PG;
+    const unsigned mP = tj < a.xw ? a.mP1 : a.mP0, mG = tj < a.xw ? a.mG1 : a.mG0;
+    PhaseSums<GRID, NT> sums{sw, peer, a.part, reinterpret_cast<unsigned long long*>(a.ticket), 0ULL, a.err,
+                             a.wait_cycles, &flag, tile, tiles, 0};
+    if (GRID && tid == 0) sums.target = __ldcg(sums.bar + 1);
+    for (int b = GRID ? 0 : (int)(blockIdx.x / tiles); b < (GRID ? B : (int)(blockIdx.x / tiles) + 1); ++b) {
+        RhsState& st = a.st[b];
+        // the state as the phase finds it: its end is written while slower CTAs
+        // may still decide
+        const int stopped = st.stopped;
+        const PhaseStart ps = phase_start(a, b);
+        const bool has_ref = st.has_ref != 0;
+        const double st_ref = st.f_ref;
+        float* X = a.x + b;
+        // pixel of element q of the y tile, or -1 outside the image
+        auto pixel = [&](int q) {
+            if constexpr (KIND == 2) return c0 + q;
+            const int qi = div_by(q, mP), i = r0 - 1 + qi, j = c0 - 1 + (q - qi * P);
+            return (i >= 0 && i < H && j >= 0 && j < W) ? i * W + j : -1;
+        };
+        auto load = [&](bool halo_only) {
+            for (int q0 = tid; q0 < ylen; q0 += 4 * NT) {
+                float v[4];
+                bool in[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int q = q0 + u * NT;
+                    int p = q < ylen ? pixel(q) : -1;
+                    if (halo_only && p >= 0) {
+                        const int qi = div_by(q, mP), i = qi - 1, j = q - qi * P - 1;
+                        if (i >= 0 && i < h && j >= 0 && j < w) p = -1;
                     }
+                    in[u] = p >= 0;
+                    v[u] = in[u] ? __ldcg(X + (size_t)p * B) : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (in[u]) ys[q0 + u * NT] = v[u];
+            }
+        };
+        // a CTA's shared memory may be written by its peers once it runs
+        if (!GRID && tiles > 1) cg::this_cluster().barrier_arrive();
+        load(false);
+        if (!GRID && tiles > 1) cg::this_cluster().barrier_wait();
+        if (stopped) continue;   // uniform over the right-hand side's CTAs
+        if (lin)
+            for (int q = tid; q < own; q += NT) gs[q] = a.c32[c0 + q];
+        long long ell = ps.ell;
+        if (tid < kWideTrials) pow_s[tid] = trial_scale(a.gamma, a.log2_alpha, ell + tid, 1.f);
+        int accepted = 0, trials = 0;
+        double f_start = 0.0;   // thread 0
+        bool copied = false;
+        __syncthreads();
+        for (int s = 0; s < a.n_red; ++s) {
+            // subgradient, ||g||^2 and f(y)
+            KSum kg, kf;
+            double fl = 0.0;
+            for (int q = tid; q < glen; q += NT) {
+                float g = 0.f, term = 0.f;
+                if constexpr (KIND == 2) {
+                    const float y = ys[q];
+                    if (lin) {
+                        g = gs[q];
+                        fl += a.c64[c0 + q] * (double)y;
+                    } else {
+                        term = norm_term(obj, y);
+                        g = norm_grad(obj, y);
+                        gs[q] = g;
+                    }
+                    kf.add(term);
+                    kg.add(g * g);
                 } else {
-                    const int i = r0 + px.i, j = px.j;
-                    kf.add(tv_term(a.obj, i, j, H, W, yb));
-                    if (!a.record_only) {
-                        const float gp = tv_subgrad(a.obj, i, j, H, W, yb);
-                        gs[q] = gp;
-                        kg.add(gp * gp);
+                    const int qi = div_by(q, mG), qj = q - qi * PG, i = r0 + qi, j = c0 + qj;
+                    if (i >= H || j >= W) continue;
+                    const float* yp = ys + (qi + 1) * P + qj + 1;
+                    const float y0 = yp[0];
+                    const bool up = i > 0, left = j > 0, down = i < H - 1, right = j < W - 1;
+                    if constexpr (KIND == 0) {
+                        if (down && right) {
+                            const float dx = yp[P] - y0, dy = yp[1] - y0, e = sq2(dx, dy);
+                            term = sqrtf(e);
+                            if (e > 0.f) g -= (dx + dy) * rsqrtf(e);
+                        }
+                        if (up && right) {
+                            const float ym = yp[-P], dx = y0 - ym, dy = yp[1 - P] - ym, e = sq2(dx, dy);
+                            if (e > 0.f) g += dx * rsqrtf(e);
+                        }
+                        if (left && down) {
+                            const float yl = yp[-1], dx = yp[P - 1] - yl, dy = y0 - yl, e = sq2(dx, dy);
+                            if (e > 0.f) g += dy * rsqrtf(e);
+                        }
+                    } else {
+                        if (down) {
+                            const float d = yp[P] - y0;
+                            term += fabsf(d);
+                            g -= sgnf(d);
+                        }
+                        if (up) g += sgnf(y0 - yp[-P]);
+                        if (right) {
+                            const float d = yp[1] - y0;
+                            term += fabsf(d);
+                            g -= sgnf(d);
+                        }
+                        if (left) g += sgnf(y0 - yp[-1]);
+                    }
+                    gs[q] = g;
+                    if (qi < h && qj < w) {
+                        kf.add(term);
+                        kg.add(g * g);
                     }
                 }
             }
-        }
-        const double2 r = cluster_sum2(ff_of(kg), lin ? ff_of(fl) : ff_of(kf), swf, &scta, &sres,
-                                       cluster);
-        const double fy = r.y;
-        if (threadIdx.x == 0) {
-            if (!have_f) {
-                f_start = fy;
-                have_f = true;
-            }
-            dec = step_decision(a, st, r.x, fy, f_start);
-        }
-        __syncthreads();
-        if (!dec.go) break;
-        const float inv_gnorm = dec.inv_gnorm, asc = dec.asc;
-        bool ok = false;
-        const int jmax = a.adaptive ? 1 : a.max_trials;
-        for (int jt = 0; jt < jmax; ++jt) {
-            if (threadIdx.x == 0)
-                sc_s = a.adaptive ? asc : trial_scale(a.gamma, a.log2_alpha, ell, inv_gnorm);
+            FF v2[2] = {ff_of(kg), lin ? ff_of(fl) : ff_of(kf)};
+            double out = 0.0;
+            if (!sums.sum(v2, out)) return;
+            if (warp < 2 && lane == 0) gy_s[warp] = out;
             __syncthreads();
-            const float sc = sc_s;
-            if (!a.adaptive) ell += 1;
-            trials += 1;
-            FF fzp;
-            if (lin) {
-                double fzl = 0.0;
-                for (int q = threadIdx.x; q < band; q += kPerturbThreads)
-                    fzl += a.c64[p0 + q] * (double)trial(ys[q], gs[q], sc);
-                fzp = ff_of(fzl);
-            } else if (elem) {
-                KSum kz;
-                for (int q = threadIdx.x; q < band; q += kPerturbThreads)
-                    kz.add(norm_term(a.obj, trial(ys[q], gs[q], sc)));
-                fzp = ff_of(kz);
-            } else {
-                auto z = [&yb, &gb, sc](int i, int j) { return trial(yb(i, j), gb(i, j), sc); };
-                KSum kz;
-                StrideWalk px(threadIdx.x, kPerturbThreads, W);
-                for (int q = threadIdx.x; q < band; q += kPerturbThreads, px.next())
-                    kz.add(tv_term(a.obj, r0 + px.i, px.j, H, W, z));
-                fzp = ff_of(kz);
+            const double fy = gy_s[1];
+            if (tid == 0) {
+                if (s == 0) f_start = fy;
+                dec = step_decision(a, has_ref, st_ref, gy_s[0], fy, f_start);
             }
-            const double fz = cluster_sum2(fzp, FF{0.f, 0.f}, swf, &scta, &sres, cluster).x;
-            if (fz <= fy) {
-                for (int q = threadIdx.x; q < band; q += kPerturbThreads)
-                    ys[q] = trial(ys[q], gs[q], sc);
-                cluster.sync();
-                accepted += 1;
-                ok = true;
-                break;
+            __syncthreads();
+            if (!dec.go) break;
+            const float inv_gnorm = dec.inv_gnorm, asc = dec.asc;
+            const int jmax = a.adaptive ? 1 : a.max_trials;
+            bool ok = false;
+            // f at N consecutive trial points; the first that passes, or -1,
+            // or -2 when a wait gave up
+            auto try_points = [&](auto NC, int cnt, const float* sj) -> int {
+                constexpr int N = decltype(NC)::value;
+                KSum kz[N];
+                double fz[N];
+#pragma unroll
+                for (int k = 0; k < N; ++k) fz[k] = 0.0;
+                // the same pixels in the same order as f(y): where a step leaves
+                // y as it is, f(z) is f(y) to the last bit
+                for (int q = tid; q < glen; q += NT) {
+                    if constexpr (KIND == 2) {
+                        const float y0 = ys[q], g0 = gs[q];
+                        const double c = lin ? a.c64[c0 + q] : 0.0;
+#pragma unroll
+                        for (int k = 0; k < N; ++k) {
+                            const float z = trial(y0, g0, sj[k]);
+                            if (lin) fz[k] += c * (double)z;
+                            else kz[k].add(norm_term(obj, z));
+                        }
+                    } else {
+                        const int qi = div_by(q, mG), qj = q - qi * PG, i = r0 + qi, j = c0 + qj;
+                        if (qi >= h || qj >= w) continue;
+                        const float* yp = ys + (qi + 1) * P + qj + 1;
+                        const float* gp = gs + q;
+                        TvNbr t;
+                        t.down = i < H - 1;
+                        t.right = j < W - 1;
+                        t.y0 = yp[0];
+                        t.g0 = gp[0];
+                        t.yd = yp[P];
+                        t.gd = gp[PG];
+                        t.yr = yp[1];
+                        t.gr = gp[1];
+#pragma unroll
+                        for (int k = 0; k < N; ++k) kz[k].add(tv_trial_term(obj, t, sj[k]));
+                    }
+                }
+                FF v[N];
+#pragma unroll
+                for (int k = 0; k < N; ++k) v[k] = lin ? ff_of(fz[k]) : ff_of(kz[k]);
+                double o = 0.0;
+                if (!sums.sum(v, o)) return -2;
+                if (warp < N && lane == 0) pass_s[warp] = o <= fy;
+                __syncthreads();
+                int hit = -1;
+#pragma unroll
+                for (int k = N - 1; k >= 0; --k)
+                    if (k < cnt && pass_s[k]) hit = k;
+                return hit;
+            };
+            for (int jt = 0; jt < jmax && !ok;) {
+                const int cnt = min(jt == 0 ? kFirstTrials : kWideTrials, jmax - jt);
+                float sj[kWideTrials];
+#pragma unroll
+                for (int k = 0; k < kWideTrials; ++k) sj[k] = a.adaptive ? asc : pow_s[k] * inv_gnorm;
+                const int hit = jt == 0 ? try_points(std::integral_constant<int, kFirstTrials>{}, cnt, sj)
+                                        : try_points(std::integral_constant<int, kWideTrials>{}, cnt, sj);
+                if (hit == -2) return;
+                const int used = hit >= 0 ? hit + 1 : cnt;
+                if (!a.adaptive) {
+                    ell += used;
+                    // every thread has its step sizes in registers (the sums'
+                    // barriers lie between)
+                    if (tid < kWideTrials && (hit < 0 || s + 1 < a.n_red)) pow_s[tid] = trial_scale(a.gamma, a.log2_alpha, ell + tid, 1.f);
+                }
+                trials += used;
+                jt += used;
+                if (hit >= 0) {
+                    float sc = sj[0];
+#pragma unroll
+                    for (int k = 1; k < kWideTrials; ++k) sc = k == hit ? sj[k] : sc;
+                    for (int q = tid; q < glen; q += NT) {
+                        const int qi = KIND == 2 ? 0 : div_by(q, mG), qj = KIND == 2 ? q : q - qi * PG;
+                        if (qi >= h || qj >= w) continue;
+                        const int e = KIND == 2 ? q : (qi + 1) * P + qj + 1;
+                        const float z = trial(ys[e], gs[q], sc);
+                        ys[e] = z;
+                        const int i = r0 + qi, j = c0 + qj;
+                        X[(size_t)(i * W + j) * B] = z;
+                        if (GRID && KIND != 2 && a.pA) {
+                            a.pA[patch_pos(i, j, a.pWp, false)] = z;
+                            a.pB[patch_pos(i, j, a.pWp, true)] = z;
+                        }
+                    }
+                    copied = true;
+                    accepted += 1;
+                    ok = true;
+                }
+                __syncthreads();   // pow_s, pass_s
+            }
+            if (!ok) break;
+            if (s + 1 < a.n_red && tiles > 1 && KIND != 2) {
+                // the next step reads the neighbours' new y around the rectangle
+                if (!sums.barrier()) return;
+                load(true);
+                __syncthreads();
             }
         }
-        if (!ok) break;
+        if (GRID && KIND != 2 && a.pA && !copied)
+            // no step was taken: the patch copies of y as it stands
+            for (int q = tid; q < glen; q += NT) {
+                const int qi = div_by(q, mG), qj = q - qi * PG, i = r0 + qi, j = c0 + qj;
+                if (qi >= h || qj >= w) continue;
+                const float z = ys[(qi + 1) * P + qj + 1];
+                a.pA[patch_pos(i, j, a.pWp, false)] = z;
+                a.pB[patch_pos(i, j, a.pWp, true)] = z;
+            }
+        if (tile == 0 && tid == 0) phase_end(a, st, ps, ell, accepted, trials, f_start);
+        if (GRID && b + 1 < B) __syncthreads();   // the tile is loaded anew
     }
-    if (!a.record_only) {
-        for (int q = threadIdx.x; q < band; q += kPerturbThreads) X[(size_t)(p0 + q) * B] = ys[q];
-    }
-    if (rank == 0 && threadIdx.x == 0) phase_end(a, st, ps, ell, accepted, trials, f_start);
-    // no CTA may leave while a neighbour can still read its shared memory
-    cluster.sync();
+    // the next launch counts on from here (this CTA has passed the last barrier)
+    if (GRID && tile == 0 && tid == 0) __stcg(sums.bar + 1, sums.target);
 }
 
 // ------------------------------------------------ whole-GPU phase ----
@@ -711,8 +1013,6 @@ __device__ __forceinline__ void grid_sums(const double* part, int B, double* res
 // budget is a launch argument (about two seconds of SM clock by default).
 // The partials need no second buffer: they are read before the release, and
 // written again only after it.
-constexpr int kFirstTrials = 2;
-
 template <int NV>
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, int* err, const double* part,
                                              double* gsum, double* res, long long limit) {
@@ -773,45 +1073,6 @@ struct CohImage {
         return y[((size_t)i * W + j) * B];
     }
 };
-
-// The values a TV term of pixel (i, j) reads at every trial point z = y - s g:
-// y and g at (i, j), (i + 1, j) and (i, j + 1), loaded once per pixel.
-struct TvNbr {
-    float y0, g0, yd, gd, yr, gr;
-    bool down, right;
-};
-
-__device__ __forceinline__ TvNbr tv_nbr(int i, int j, int H, int W, const float* y, const float* g,
-                                        int B) {
-    const size_t p = (size_t)i * W + j;
-    TvNbr t;
-    t.down = i < H - 1;
-    t.right = j < W - 1;
-    t.y0 = y[p * B];
-    t.g0 = g[p * B];
-    t.yd = t.down ? y[(p + W) * B] : 0.f;
-    t.gd = t.down ? g[(p + W) * B] : 0.f;
-    t.yr = t.right ? y[(p + 1) * B] : 0.f;
-    t.gr = t.right ? g[(p + 1) * B] : 0.f;
-    return t;
-}
-
-// TV term at the trial point with step s (computed as in the cluster kernels).
-__device__ __forceinline__ float tv_trial_term(int obj, const TvNbr& t, float s) {
-    const float z0 = trial(t.y0, t.g0, s);
-    if (obj == SUPPY_OBJ_TV_ISO) {
-        if (t.down && t.right) {
-            const float dx = trial(t.yd, t.gd, s) - z0;
-            const float dy = trial(t.yr, t.gr, s) - z0;
-            return sqrtf(dx * dx + dy * dy);
-        }
-        return 0.f;
-    }
-    float v = 0.f;
-    if (t.down) v += fabsf(trial(t.yd, t.gd, s) - z0);
-    if (t.right) v += fabsf(trial(t.yr, t.gr, s) - z0);
-    return v;
-}
 
 __global__ void __launch_bounds__(kPhaseThreads, 1) k_wide_phase(const PerturbArgs a) {
     __shared__ FF sw[(kPhaseThreads / 32) * kWideTrials * 32];
@@ -1060,22 +1321,109 @@ __global__ void __launch_bounds__(256) k_objective(const ObjArgs a) {
 
 }  // namespace
 
-size_t perturb_smem_bytes(int obj, int n, int H, int W, int cs);
+namespace {
 
+// Shared memory of the tile-resident phase for rectangles of th x tw pixels.
+size_t phase_smem(bool elem, int th, int tw) {
+    if (elem) return sizeof(float) * 2 * (size_t)tw;
+    return sizeof(float) * ((size_t)(th + 3) * (tw + 3) + (size_t)(th + 1) * (tw + 1));
+}
+
+constexpr size_t kPhaseSmem = 200 * 1024;
+
+bool elem_obj(int obj) {
+    return obj == SUPPY_OBJ_LINEAR || obj == SUPPY_OBJ_L1 || obj == SUPPY_OBJ_L2;
+}
+
+// The grid of at most `tiles` rectangles whose largest one, halo included, is
+// smallest; false when it does not fit shared memory.
+bool phase_tiles(int obj, int n, int H, int W, int tiles, bool exact, PhaseTiles* out) {
+    PhaseTiles best;
+    if (elem_obj(obj)) {
+        if (tiles > n && exact) return false;
+        best.TR = 1;
+        best.TC = std::min(tiles, n);
+        best.h = 1;
+        best.w = (n + best.TC - 1) / best.TC;
+        H = 1;
+        W = n;
+    } else {
+        long long cost = -1;
+        for (int r = 1; r <= std::min(tiles, H); ++r) {
+            const int c = std::min(tiles / r, W);
+            if (c < 1 || (exact && r * c != tiles)) continue;
+            const int h = (H + r - 1) / r, w = (W + c - 1) / c;
+            const long long k = (long long)(h + 3) * (w + 3);
+            if (cost < 0 || k < cost) {
+                cost = k;
+                best = PhaseTiles{r, c, h, w};
+            }
+        }
+        if (cost < 0) return false;
+    }
+    if (phase_smem(elem_obj(obj), best.h, best.w) > kPhaseSmem) return false;
+    *out = best;
+    return true;
+}
+
+// The rectangles as the kernel takes them: the size of the smaller ones, how
+// many rows and columns of them are one pixel larger, and the factors that
+// divide by the widths of their y (w + 3) and subgradient (w + 1) tiles.
+void set_phase_tiles(PerturbArgs& a, const PhaseTiles& t) {
+    const int H = elem_obj(a.obj) ? 1 : a.H, W = elem_obj(a.obj) ? a.n : a.W;
+    a.TR = t.TR;
+    a.TC = t.TC;
+    a.tmh = t.h;
+    a.tmw = t.w;
+    a.th = H / t.TR;
+    a.xh = H % t.TR;
+    a.tw = W / t.TC;
+    a.xw = W % t.TC;
+    auto magic = [](int d) { return (unsigned)(((1ULL << 32) + d - 1) / d); };
+    a.mP0 = magic(a.tw + 3);
+    a.mP1 = magic(a.tw + 4);
+    a.mG0 = magic(a.tw + 1);
+    a.mG1 = magic(a.tw + 2);
+}
+
+using PhaseFn = void (*)(PerturbArgs);
+
+PhaseFn phase_fn(int obj, bool grid, int threads) {
+    const int kind = obj == SUPPY_OBJ_TV_ISO ? 0 : (obj == SUPPY_OBJ_TV_ANISO ? 1 : 2);
+    if (!grid) return kind == 0 ? k_phase<0, false, 512> : (kind == 1 ? k_phase<1, false, 512> : k_phase<2, false, 512>);
+    if (threads == 512)
+        return kind == 0 ? k_phase<0, true, 512> : (kind == 1 ? k_phase<1, true, 512> : k_phase<2, true, 512>);
+    return kind == 0 ? k_phase<0, true, 1024> : (kind == 1 ? k_phase<1, true, 1024> : k_phase<2, true, 1024>);
+}
+
+// Threads per CTA of the whole-GPU form: 1024 where 512 would take more than
+// two pixels each.
+int phase_threads(const PhaseTiles& t) { return (long long)t.h * t.w > 1024 ? 1024 : 512; }
+
+}  // namespace
+
+// CTAs per right-hand side of the cluster form: two pixels a thread for one
+// right-hand side (64x64 and 128x128 images: 9.5-10 us, where one thread took
+// eight pixels 22 us), eight for several, whose clusters share the GPU (16
+// images of 256x512: 61.6 us in clusters of 16, 67.0 us in clusters of 8 with
+// 1024 threads); at most 16 (one GPC).
 int choose_perturb_cluster(int n, int B) {
-    // enough CTAs that each thread owns a handful of pixels; at most 16 (one GPC)
-    int want = (n + kPerturbThreads * 8 - 1) / (kPerturbThreads * 8);
+    const long long per_cta = kPerturbThreads * (B == 1 ? 2 : 8);
     int cs = 1;
-    while (cs < want && cs < 16) cs <<= 1;
-    (void)B;
+    while (cs < 16 && cs * per_cta < n) cs <<= 1;
     return cs;
 }
 
 int fit_perturb_cluster(int want, int obj, int n, int H, int W) {
-    // largest power of two <= want for which a cluster can be resident
-    for (int cs = want; cs >= 1; cs >>= 1) {
-        const size_t smem = perturb_smem_bytes(obj, n, H, W, cs);
-        auto kern = smem ? k_perturb_smem : k_perturb;
+    // more CTAs where their rectangles would not fit shared memory, then the
+    // largest power of two for which a cluster can be resident
+    PhaseTiles t;
+    int most = want;
+    while (most < 16 && !phase_tiles(obj, n, H, W, most, true, &t)) most <<= 1;
+    for (int cs = most; cs >= 1; cs >>= 1) {
+        const bool tiled = phase_tiles(obj, n, H, W, cs, true, &t);
+        const size_t smem = tiled ? phase_smem(elem_obj(obj), t.h, t.w) : 0;
+        auto kern = tiled ? phase_fn(obj, false, kPerturbThreads) : k_perturb;
         cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaLaunchConfig_t cfg = {};
@@ -1096,18 +1444,17 @@ int fit_perturb_cluster(int want, int obj, int n, int H, int W) {
     return 1;
 }
 
-size_t perturb_smem_bytes(int obj, int n, int H, int W, int cs) {
-    const bool elem = (obj == SUPPY_OBJ_LINEAR || obj == SUPPY_OBJ_L1 || obj == SUPPY_OBJ_L2);
-    const long long rows = elem ? n : H, w = elem ? 1 : W;
-    if (!elem && cs > H) return 0;
-    const long long maxband = ((rows + cs - 1) / cs) * w;
-    const size_t bytes = (size_t)(2 * maxband) * sizeof(float);
-    return bytes <= 200 * 1024 ? bytes : 0;
-}
-
-cudaError_t launch_perturb(const PerturbArgs& a, int cluster, cudaStream_t s) {
-    const size_t smem = perturb_smem_bytes(a.obj, a.n, a.H, a.W, cluster);
-    auto kern = smem ? k_perturb_smem : k_perturb;
+cudaError_t launch_perturb(const PerturbArgs& args, int cluster, cudaStream_t s) {
+    PerturbArgs a = args;
+    PhaseTiles t;
+    const bool tiled = !a.record_only && phase_tiles(a.obj, a.n, a.H, a.W, cluster, true, &t);
+    size_t smem = 0;
+    auto kern = k_perturb;
+    if (tiled) {
+        set_phase_tiles(a, t);
+        smem = phase_smem(elem_obj(a.obj), t.h, t.w);
+        kern = phase_fn(a.obj, false, kPerturbThreads);
+    }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     if (smem) {
@@ -1129,8 +1476,45 @@ cudaError_t launch_perturb(const PerturbArgs& a, int cluster, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-// kWideTrials partials per CTA, then the kWideTrials grid sums
-size_t wide_part_doubles(int grid) { return ((size_t)grid + 1) * kWideTrials; }
+bool wide_phase_tiles(int obj, int n, int H, int W, int sms, PhaseTiles* out) {
+    // a few hundred pixels a CTA at least: fewer CTAs meet sooner
+    const int tiles = (int)std::max<long long>(1, std::min<long long>(sms, ((long long)n + 255) / 256));
+    if (!phase_tiles(obj, n, H, W, tiles, false, out)) return false;
+    const size_t smem = phase_smem(elem_obj(obj), out->h, out->w);
+    auto kern = phase_fn(obj, true, phase_threads(*out));
+    int nb = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, phase_threads(*out), smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return nb >= 1;
+}
+
+cudaError_t launch_phase_tiles(const PerturbArgs& args, const PhaseTiles& t, cudaStream_t s) {
+    PerturbArgs a = args;
+    if (!a.ticket || !a.err || !a.part) return cudaErrorInvalidValue;
+    set_phase_tiles(a, t);
+    const size_t smem = phase_smem(elem_obj(a.obj), t.h, t.w);
+    auto kern = phase_fn(a.obj, true, phase_threads(t));
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(t.TR * t.TC, 1, 1);
+    cfg.blockDim = dim3(phase_threads(t), 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+// kWideTrials partials per CTA, two buffers (the tile-resident phase) or one
+// and the grid sums
+size_t wide_part_doubles(int grid) { return 2 * ((size_t)grid + 1) * kWideTrials; }
 
 int wide_phase_blocks_per_sm() {
     int nb = 0;
