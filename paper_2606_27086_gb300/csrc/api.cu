@@ -188,7 +188,7 @@ struct suppy_ctx {
         int* d_cta = nullptr;
         std::vector<int> grid;          // per block: CTAs
         std::vector<size_t> cta_off;    // per block: offset of its boundaries in d_cta
-        int nw = 4;                     // warps per strip
+        int nw = 4;                     // warps per strip (1, 2, 4 or 8)
         int keep = 0;                   // the packets stay in L2 between sweeps
         long long tall = 0;             // rows in strips of tall patches
     };
@@ -1579,7 +1579,7 @@ void free_strips(suppy_ctx* c, suppy_ctx::StripSet& S) {
 // there, a column's its index inside the block.
 suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info, const int* idx,
                           const void* val, const std::vector<long long>& block_of, bool columns, int max_len,
-                          long long entries, bool patch, bool* ok) {
+                          long long entries, bool scatter, bool patch, bool* ok) {
     *ok = false;
     if (max_len < 1 || max_len > kStripMaxItem) return SUPPY_OK;
     const int nseg = (int)block_of.size() - 1;
@@ -1592,7 +1592,7 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
         seg_first[t + 1] = (int)strips.size();
     }
     const int ns = (int)strips.size();
-    const size_t vsz = (c->dt == SUPPY_F32) ? 4 : 2;
+    const int pbytes = strip_packet_bytes(c->dt == SUPPY_F32 ? 4 : 2, scatter);
     TempGuard tg;
     tg.s = c->stream;
     suppy_status s;
@@ -1617,6 +1617,7 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
         b.recipW = ~0ULL / (unsigned long long)c->gW + 1ULL;
     }
     b.patch = patch;
+    b.scatter = scatter;
     b.all_items = columns;
     b.meta = static_cast<int4*>(q);
     CK(launch_strip_build(b, c->dt, 0, c->stream));
@@ -1633,7 +1634,7 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
             int4 m = meta[k];
             const int npk = m.y & kStripPackets;
             if (npk == 0 && !columns) continue;
-            const long long at = packets * (strip_packet_bytes((int)vsz) / 16);
+            const long long at = packets * (pbytes / 16);
             m.x = (int)(unsigned)at;
             packets += npk;
             most = std::max(most, npk);
@@ -1643,22 +1644,33 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
         }
         first[t + 1] = kept;
     }
-    const long long bytes = packets * strip_packet_bytes((int)vsz);
+    const long long bytes = packets * pbytes;
     if (packets < 1 || (double)packets * 128.0 > kStripSlots * (double)entries + 128.0 ||
-        (long long)most * strip_packet_bytes((int)vsz) > kStripRing / 2 || (bytes >> 4) > 0xffffffffLL)
+        (long long)most * pbytes > kStripRing / 2 || (bytes >> 4) > 0xffffffffLL)
         return SUPPY_OK;
     S.tall = tall;
-    const double mean = (double)packets / std::max(kept, 1);
-    // warps a strip: a few packets each, so that the strips in work leave the
-    // ring room to stream ahead (CT 512x512, 14.5 packets a strip: 4, 2 and 1
-    // warps took 254, 265 and 294 us; CT 128x128 blocks have 4.4)
-    S.nw = mean >= 8.0 ? 4 : (mean >= 4.0 ? 2 : 1);
+    // Warps a strip: as few as leave the strips in work about half the ring
+    // (the scatter holds a strip until it is added; the other passes give it
+    // back at once), since every warp pays about 150 instructions a strip --
+    // and not so few that consumer groups go without strips.  Row passes in
+    // us with 8 / 4 / 2 / 1 warps: CT 512x512 scatter 269 / 214 / 234 / 332
+    // (12.3 KB a strip), 1024x1024 40 angles 117 / 127 / 177 / 301 (24.6 KB),
+    // 384x384 FP16 143 / 107 / 96 / 117 (6.4 KB), 128x128 blocks 11.6 / 10.4
+    // / 11.0 / 12.3 (2.7 strips a CTA); 512x512 two passes, rows 196 / 151 /
+    // 145 / 158.
+    int sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
+    const double strip_bytes = (double)bytes / std::max(kept, 1);
+    const double per_cta = (double)kept / ((double)nseg * sms);
+    constexpr int consumers = kStripThreads / 32 - 1;
+    S.nw = 1;
+    while (S.nw < 8 && (consumers / S.nw * strip_bytes > (scatter ? 100.0 : 150.0) * 1024 ||
+                        (S.nw < 4 && consumers / S.nw > 2.5 * per_cta)))
+        S.nw *= 2;
     // packets that fit L2 (129 MB) beside the vectors stay there between sweeps
     S.keep = bytes <= 80LL * 1024 * 1024;
     // per block: contiguous strip ranges of equal packets (and a constant a
     // strip), one per SM
-    int sms = 0;
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
     std::vector<int> cta;
     std::vector<long long> pref(kept + 1, 0);
     for (int k = 0; k < kept; ++k) pref[k + 1] = pref[k] + (meta[k].y & kStripPackets) + 2;
@@ -1682,7 +1694,7 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
             const int k0 = cta[S.cta_off[t] + g], k1 = cta[S.cta_off[t] + g + 1];
             int oldest = k0, head = 0;
             for (int k = k0; k < k1; ++k) {
-                const int need = (meta[k].y & kStripPackets) * strip_packet_bytes((int)vsz);
+                const int need = (meta[k].y & kStripPackets) * pbytes;
                 int at = -1;
                 for (; at < 0; oldest += at < 0) {
                     if (oldest == k) {
@@ -2508,21 +2520,21 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
     const bool strip_patch = tr_grid && !smem_ok &&
                              (long long)((c->gH + 7) & ~7) * ((c->gW + 7) & ~7) < (1LL << 31);
     std::vector<long long> row_blocks(c->seg_start.begin(), c->seg_start.end());
-    int strips_are = -1;   // the row strips built: -1 none, 0 plain, 1 patch numbering
+    int strips_are = -1;   // the row strips built: -1 none, else their strategy
     // builds what a strategy's strip-ordered passes need; *ok false: they do
     // not pay on this matrix
     auto make_strips = [&](int strategy, bool* ok) -> suppy_status {
         const bool patch = strategy == 1 && strip_patch;
         suppy_status st;
         *ok = true;
-        if (strips_are != (int)patch) {
+        if (strips_are != strategy) {
             free_strips(c, c->rstrips);
             strips_are = -1;
             if ((st = build_strips(c, c->rstrips, c->d_rinfo, c->d_col, c->d_val, row_blocks, false, max_len,
-                                   A->nnz, patch, ok)) != SUPPY_OK)
+                                   A->nnz, strategy == 1, patch, ok)) != SUPPY_OK)
                 return st;
             if (!*ok) return SUPPY_OK;
-            strips_are = patch;
+            strips_are = strategy;
         }
         if (patch) {
             if ((st = alloc_accumulators(c)) != SUPPY_OK) return st;
@@ -2532,7 +2544,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
             std::vector<long long> col_blocks(c->nseg + 1);
             for (int t = 0; t <= c->nseg; ++t) col_blocks[t] = (long long)t * n;
             if ((st = build_strips(c, c->cstrips, c->d_cinfo, c->d_ridx, c->d_cval, col_blocks, true, c->max_col,
-                                   c->nnz_csc, false, ok)) != SUPPY_OK)
+                                   c->nnz_csc, false, false, ok)) != SUPPY_OK)
                 return st;
         }
         return SUPPY_OK;

@@ -252,8 +252,8 @@ constexpr int kStripInFlight = 48;         // strips a CTA's ring holds at most
 // still be in the ring when this one is copied in (6 bits)
 __host__ __device__ constexpr int strip_at(int w) { return ((w >> 4) & 0x3fff) << 4; }
 __host__ __device__ constexpr int strip_live(int w) { return (w >> 18) & 0x3f; }
-__host__ __device__ constexpr int strip_packet_bytes(int value_bytes) {
-    return 16 + 128 * 2 + 128 * value_bytes;   // bases, offsets, values
+__host__ __device__ constexpr int strip_packet_bytes(int value_bytes, bool scatter) {
+    return 16 + (scatter ? 64 : 0) + 128 * 2 + 128 * value_bytes;   // bases, flags, offsets, values
 }
 struct StripArgs {
     const unsigned char* blob;   // packets
@@ -301,6 +301,7 @@ struct StripBuild {
     int H, W, Wp;                // image grid of the indices (W = 0: none), W padded to 8
     unsigned long long recipW;
     int patch;                   // positions in the patch numbering
+    int scatter;                 // packets of the one-pass scatter (with flags)
     int all_items;               // items without entries count too (columns)
     int4* meta;
     unsigned char* blob;
@@ -443,7 +444,7 @@ cudaError_t launch_rows_tma(const StreamArgs& a, suppy_dtype dt, int G, int scat
 cudaError_t launch_cols_tma(const StreamArgs& a, suppy_dtype dt, int G, int map, int grid,
                             cudaStream_t s);
 // kind: 0 row pass (coefficients out), 1 row pass with the scatter, 2 column
-// pass; nw: warps per strip (1, 2 or 4)
+// pass; nw: warps per strip (1, 2, 4 or 8)
 cudaError_t launch_strip(const StripArgs& a, suppy_dtype dt, int kind, int nw, int grid, cudaStream_t s);
 // fill 0: count the packets into meta; 1: write them at the offsets of meta
 cudaError_t launch_strip_build(const StripBuild& b, suppy_dtype dt, int fill, cudaStream_t s);

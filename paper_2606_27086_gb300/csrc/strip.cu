@@ -14,8 +14,8 @@
 // (360 angles x 725 bins) in the patch numbering they fall from 41.6 M to
 // 27.0 M a sweep; the padding of the windows costs 4.6% more slots.
 //
-// A packet is {four bases (int32, one an item), 128 16-bit offsets, 128
-// values}: position = base of the item + offset, so an entry costs 6 bytes
+// A packet is {four bases (int32, one an item), for the scatter the lanes'
+// flags, 128 16-bit offsets, 128 values}: position = base of the item + offset, so an entry costs 6 bytes
 // instead of 8 (FP32 values; nothing is rounded, a window ends where an
 // offset would not fit) and a lane reads its four entries of a packet with
 // one 4-byte, one 8-byte and one 16-byte shared-memory load.
@@ -28,12 +28,19 @@
 // products are summed over the eight lanes and then over the group's warps in
 // a fixed order; the scatter reads the strip again from the ring.
 //
+// In the one-pass scatter, entries of neighbouring rows on the same pixel (18%
+// of CT entries, most of a dose matrix's) are placed in the same slot of their
+// items: the first item's lane adds the others' shares to its own (their
+// values lie beside its own in the packet), so that a pixel is reduced once
+// and no instruction reduces an address twice, which would split it.
+//
 // Measured (GB300, CT 512x512, 120.3 M entries, FP32; the streamed passes of
-// stream.cu in their default shapes before): two-pass row pass 227 -> 156 us,
-// column pass 196 -> 144 us (5.4 TB/s of the 6.7 copied), one-pass row pass
-// 342 -> 242 us.  The first two are bound by HBM; the scatter adds its L2
-// reductions, which share the load/store pipe with the gathers (without them
-// the one-pass row pass takes 127 us).
+// stream.cu in their default shapes before): two-pass row pass 227 -> 145 us,
+// column pass 196 -> 135 us (both 5.3 TB/s of the 6.7 copied, bound by HBM),
+// one-pass row pass 342 -> 209 us.  The scatter's L2 reductions (26.7 M
+// sectors; 39 M before shared pixels were joined, 253 us) share the
+// load/store pipe and the issue slots with the gathers: without them the
+// one-pass row pass takes 127 us.
 #include <algorithm>
 #include <climits>
 
@@ -123,14 +130,13 @@ __device__ __forceinline__ bool group_all(int grp, bool ok) {
     }
 }
 
-template <typename VT>
+template <typename VT, int KIND>
 struct Packet {
-    static constexpr int kBytes = strip_packet_bytes(sizeof(VT));
-    static constexpr int kIdx = 16, kVal = 16 + 256;
+    static constexpr int kBytes = strip_packet_bytes(sizeof(VT), KIND == 1);
+    static constexpr int kIdx = KIND == 1 ? 80 : 16, kVal = kIdx + 256;   // after bases and flags
 };
 
-// Gather and L2 reduction at x[base + o] unless o marks an empty slot, as
-// predicated instructions.
+// x[base + o], 0 in an empty slot.
 __device__ __forceinline__ float gather(const float* x, int base, unsigned o) {
     float g;
     asm("{\n\t.reg .pred p;\n\t"
@@ -141,17 +147,9 @@ __device__ __forceinline__ float gather(const float* x, int base, unsigned o) {
         : "l"(x + (base + (int)o)), "r"(o));
     return g;
 }
-__device__ __forceinline__ void reduce(float* x, int base, unsigned o, float v) {
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "setp.ne.u32 p, %1, 65535;\n\t"
-                 "@p red.global.add.f32 [%0], %2;\n\t}" ::"l"(x + (base + (int)o)),
-                 "r"(o), "f"(v)
-                 : "memory");
-}
-
 // N packets from p: their loads, then their gathers together, then the
 // products, so that they cost one gather latency.
-template <typename VT, int N>
+template <typename VT, int KIND, int N>
 __device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, const float* __restrict__ x,
                                             float& acc0, float& acc1) {
     int base[N];
@@ -159,10 +157,10 @@ __device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, co
     float4 v[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        const unsigned char* q = p + k * Packet<VT>::kBytes;
-        base[k] = *reinterpret_cast<const int*>(q + 4 * (lane >> 3));
-        w[k] = *reinterpret_cast<const uint2*>(q + Packet<VT>::kIdx + 8 * lane);
-        v[k] = Val4<VT>::load(q + Packet<VT>::kVal + lane * 4 * (int)sizeof(VT));
+        const unsigned char* q = p + k * Packet<VT, KIND>::kBytes;
+        base[k] = *reinterpret_cast<const int*>(q + 4 * (lane >> 3)) & 0x7fffffff;
+        w[k] = *reinterpret_cast<const uint2*>(q + Packet<VT, KIND>::kIdx + 8 * lane);
+        v[k] = Val4<VT>::load(q + Packet<VT, KIND>::kVal + lane * 4 * (int)sizeof(VT));
     }
     float g[N][4];
 #pragma unroll
@@ -178,6 +176,73 @@ __device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, co
         acc0 = fmaf(v[k].z, g[k][2], acc0);
         acc1 = fmaf(v[k].w, g[k][3], acc1);
     }
+}
+
+// s += c u where bit `B` of f is set, as predicated instructions (the compiler
+// makes a branch of each otherwise).
+template <unsigned B>
+__device__ __forceinline__ void fma_if(unsigned f, float c, float u, float& s) {
+    asm("{\n\t.reg .pred p;\n\t.reg .u32 t;\n\t"
+        "and.b32 t, %1, %4;\n\t"
+        "setp.ne.u32 p, t, 0;\n\t"
+        "@p fma.rn.f32 %0, %2, %3, %0;\n\t}"
+        : "+f"(s)
+        : "r"(f), "f"(c), "f"(u), "n"(B));
+}
+
+// L2 reduction of v into *p where bit B of f is clear.
+template <unsigned B>
+__device__ __forceinline__ void red_unless(unsigned f, float* p, float v) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 t;\n\t"
+                 "and.b32 t, %1, %3;\n\t"
+                 "setp.eq.u32 p, t, 0;\n\t"
+                 "@p red.relaxed.gpu.global.add.f32 [%0], %2;\n\t}" ::"l"(p),
+                 "r"(f), "f"(v), "n"(B)
+                 : "memory");
+}
+
+// The corrections of one packet (KIND 1).  The lane's flags: bits 0-3, entries
+// it does not add (empty, or added by an earlier item's lane); bits 4-7, 8-11,
+// 12-15, entries whose position the first, second and third item after its own
+// hold in the same slot, which it adds with its own.  c0 .. c3: the
+// coefficients of the lane's item and of those after it (0 past the strip).
+template <typename VT>
+__device__ __forceinline__ void scatter_packet(const unsigned char* sp, int lane, float c0, float c1, float c2,
+                                               float c3, float* __restrict__ dst) {
+    using Pk = Packet<VT, 1>;
+    constexpr int kItem = 8 * 4 * (int)sizeof(VT);   // bytes from one item's values to the next's
+    const int word = *reinterpret_cast<const int*>(sp + 4 * (lane >> 3));
+    const int base = word & 0x7fffffff;
+    unsigned f = *reinterpret_cast<const unsigned short*>(sp + 16 + 2 * lane);
+    const uint2 ix = *reinterpret_cast<const uint2*>(sp + Pk::kIdx + 8 * lane);
+    const unsigned char* vp = sp + Pk::kVal + lane * 4 * (int)sizeof(VT);
+    const float4 v = Val4<VT>::load(vp);
+    // the next item's values (its own again for the last item: no flags)
+    const float4 u = Val4<VT>::load(lane < 24 ? vp + kItem : vp);
+    float s[4] = {c0 * v.x, c0 * v.y, c0 * v.z, c0 * v.w};
+    fma_if<0x10u>(f, c1, u.x, s[0]);
+    fma_if<0x20u>(f, c1, u.y, s[1]);
+    fma_if<0x40u>(f, c1, u.z, s[2]);
+    fma_if<0x80u>(f, c1, u.w, s[3]);
+    if (word < 0) {   // uniform: the packet has positions of three or four items
+        const float4 u2 = Val4<VT>::load(lane < 16 ? vp + 2 * kItem : vp);
+        const float4 u3 = Val4<VT>::load(lane < 8 ? vp + 3 * kItem : vp);
+        fma_if<0x100u>(f, c2, u2.x, s[0]);
+        fma_if<0x200u>(f, c2, u2.y, s[1]);
+        fma_if<0x400u>(f, c2, u2.z, s[2]);
+        fma_if<0x800u>(f, c2, u2.w, s[3]);
+        fma_if<0x1000u>(f, c3, u3.x, s[0]);
+        fma_if<0x2000u>(f, c3, u3.y, s[1]);
+        fma_if<0x4000u>(f, c3, u3.z, s[2]);
+        fma_if<0x8000u>(f, c3, u3.w, s[3]);
+    }
+    // a row inside its slab adds nothing of its own
+    if (c0 == 0.f) f |= ~(f >> 4) & 0xfu;
+    float* const d = dst + base;
+    red_unless<1u>(f, d + (ix.x & 0xffffu), s[0]);
+    red_unless<2u>(f, d + (ix.x >> 16), s[1]);
+    red_unless<4u>(f, d + (ix.y & 0xffffu), s[2]);
+    red_unless<8u>(f, d + (ix.y >> 16), s[3]);
 }
 
 // KIND 0: row pass, coefficients out; 1: row pass with the scatter by L2
@@ -221,13 +286,14 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
         // were laid out with the records), so that a strip costs the producer
         // one wait and one copy
         int4 nxt = (s0 + lane < s1) ? a.meta[s0 + lane] : make_int4(0, 0, 0, 0);
+        int back = 0, back_fill = 0;   // barriers of the oldest strip in the ring
         bool ok = true;
         for (int b = s0; ok && b < s1; b += 32) {
             const int4 m = nxt;
             nxt = (b + 32 + lane < s1) ? a.meta[b + 32 + lane] : make_int4(0, 0, 0, 0);
             const int q = b - s0 + lane;
             const int need = q - strip_live(m.w);
-            const uint32_t bytes = (uint32_t)((m.y & kStripPackets) * Packet<VT>::kBytes);
+            const uint32_t bytes = (uint32_t)((m.y & kStripPackets) * Packet<VT, KIND>::kBytes);
             bool done = b + lane >= s1;
             for (;;) {
                 if (!done && need <= oldest) {
@@ -239,10 +305,13 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 }
                 issued = b - s0 + __popc(__ballot_sync(0xffffffffu, done && b + lane < s1));
                 if (__all_sync(0xffffffffu, done)) break;
-                ok = __all_sync(0xffffffffu, bounded_wait(&empty[oldest % kInFlight], (oldest / kInFlight) & 1,
-                                                          &abort_flag, a.wait_cycles));
+                ok = __all_sync(0xffffffffu, bounded_wait(&empty[back], back_fill, &abort_flag, a.wait_cycles));
                 if (!ok) break;
                 ++oldest;
+                if (++back == kInFlight) {
+                    back = 0;
+                    back_fill ^= 1;
+                }
             }
         }
         if (lane == 0 && !ok) {
@@ -252,10 +321,9 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     } else {
         const int cw = warp - 1, grp = cw / NW, wi = cw % NW;
         const int r = lane >> 3;
-        int par = 0;
+        int par = 0, slot = grp, fill = 0;   // the strip's barriers, and which fill of them
         int4 nxt = (grp < s1 - s0) ? __ldg(a.meta + s0 + grp) : make_int4(0, 0, 0, 0);
         for (int q = grp; q < s1 - s0; q += NG, par ^= 1) {
-            const int slot = q % kInFlight;
             const int4 m = nxt;
             nxt = (q + NG < s1 - s0) ? __ldg(a.meta + s0 + q + NG) : make_int4(0, 0, 0, 0);
             const int npk = m.y & kStripPackets;
@@ -278,18 +346,18 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 w = a.xw[item];   // owned by this strip alone during the pass
                 if (a.zc) mul = __ldg(a.zc + item);
             }
-            bool ok = bounded_wait(&full[slot], (q / kInFlight) & 1, &abort_flag, a.wait_cycles);
+            bool ok = bounded_wait(&full[slot], fill, &abort_flag, a.wait_cycles);
             float dot = 0.f;
             if (ok) {
                 const float* xs = tall ? a.xT : a.x;
                 float acc0 = 0.f, acc1 = 0.f;
                 int p = p0;
-                const unsigned char* sp = strip + p0 * Packet<VT>::kBytes;
-                for (; p + 4 <= p1; p += 4, sp += 4 * Packet<VT>::kBytes)
-                    dot_packets<VT, 4>(sp, lane, xs, acc0, acc1);
-                if (p1 - p == 3) dot_packets<VT, 3>(sp, lane, xs, acc0, acc1);
-                else if (p1 - p == 2) dot_packets<VT, 2>(sp, lane, xs, acc0, acc1);
-                else if (p1 - p == 1) dot_packets<VT, 1>(sp, lane, xs, acc0, acc1);
+                const unsigned char* sp = strip + p0 * Packet<VT, KIND>::kBytes;
+                for (; p + 4 <= p1; p += 4, sp += 4 * Packet<VT, KIND>::kBytes)
+                    dot_packets<VT, KIND, 4>(sp, lane, xs, acc0, acc1);
+                if (p1 - p == 3) dot_packets<VT, KIND, 3>(sp, lane, xs, acc0, acc1);
+                else if (p1 - p == 2) dot_packets<VT, KIND, 2>(sp, lane, xs, acc0, acc1);
+                else if (p1 - p == 1) dot_packets<VT, KIND, 1>(sp, lane, xs, acc0, acc1);
                 dot = acc0 + acc1;
             }
             if (KIND != 1) {
@@ -330,25 +398,27 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                     if (KIND == 0 && a.coef) a.coef[item] = coef;
                 }
                 if constexpr (KIND == 1) {
-                    if (has && coef != 0.f) {
+                    // an entry whose slot holds the same position in the item
+                    // before is added by that item's lane (eight lanes back),
+                    // which reads its value beside its own: one reduction a
+                    // position, and none twice in one instruction
+                    const float c0 = has ? coef : 0.f;
+                    float c1 = __shfl_down_sync(0xffffffffu, c0, 8), c2 = __shfl_down_sync(0xffffffffu, c0, 16),
+                          c3 = __shfl_down_sync(0xffffffffu, c0, 24);
+                    if (__any_sync(0xffffffffu, c0 != 0.f)) {
                         float* dst = tall ? a.deltaT : a.delta;
-                        const unsigned char* sp = strip + p0 * Packet<VT>::kBytes;
-#pragma unroll 2
-                        for (int p = p0; p < p1; ++p, sp += Packet<VT>::kBytes) {
-                            const int base = *reinterpret_cast<const int*>(sp + 4 * r);
-                            const uint2 ix = *reinterpret_cast<const uint2*>(sp + Packet<VT>::kIdx + 8 * lane);
-                            const float4 v = Val4<VT>::load(sp + Packet<VT>::kVal + lane * 4 * (int)sizeof(VT));
-                            const unsigned o0 = ix.x & 0xffffu, o1 = ix.x >> 16, o2 = ix.y & 0xffffu,
-                                           o3 = ix.y >> 16;
-                            reduce(dst, base, o0, coef * v.x);
-                            reduce(dst, base, o1, coef * v.y);
-                            reduce(dst, base, o2, coef * v.z);
-                            reduce(dst, base, o3, coef * v.w);
-                        }
+                        const unsigned char* sp = strip + p0 * Packet<VT, KIND>::kBytes;
+                        for (int p = p0; p < p1; ++p, sp += Packet<VT, KIND>::kBytes)
+                            scatter_packet<VT>(sp, lane, c0, c1, c2, c3, dst);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&empty[slot]);
                 }
+            }
+            slot += NG;
+            if (slot >= kInFlight) {
+                slot -= kInFlight;
+                fill ^= 1;
             }
         }
     }
@@ -411,6 +481,8 @@ __global__ void __launch_bounds__(128) k_strip_build(const StripBuild b) {
                           (size_t)warp * b.max_len;
     __shared__ int span_s[4][2], cnt_s[4], len_s[4];
     __shared__ unsigned lim_s[4];
+    __shared__ int slot_s[4][32];   // positions by slot of the window (-1: none)
+    __shared__ unsigned shared_s[4];   // slots shared with the item before
     const VT* val = static_cast<const VT*>(b.val);
     for (int t = blockIdx.x; t < b.nstrips; t += gridDim.x) {
         const int4 st = b.strips[t];   // first item in info, items, first item's number
@@ -496,12 +568,56 @@ __global__ void __launch_bounds__(128) k_strip_build(const StripBuild b) {
             if (cnt_s[0] + cnt_s[1] + cnt_s[2] + cnt_s[3] == 0) n = c;
             if constexpr (FILL) {
                 const int base = n > 0 ? __shfl_sync(0xffffffffu, mn, n - 1) : 0;
-                unsigned char* q = out + (size_t)npk * strip_packet_bytes(sizeof(VT));
+                // the entry's slot of 32: in order, or -- for the scatter -- that
+                // of the same position in the item before, the others in order
+                // in the slots left
+                int slot = lane;
+                if (b.scatter) {
+                    for (int i = 0; i < 4; ++i) {
+                        if (warp == i) {
+                            int m = -1;
+                            if (i > 0 && lane < n)
+                                for (int f = 0; f < 32; ++f)
+                                    if (slot_s[i - 1][f] == pos) m = f;
+                            // a position twice in one item keeps its first entry there
+                            const unsigned same = __match_any_sync(0xffffffffu, m < 0 ? ~lane : m);
+                            const bool forced = m >= 0 && (same & ((1u << lane) - 1u)) == 0;
+                            const unsigned taken = __reduce_or_sync(0xffffffffu, forced ? 1u << m : 0u);
+                            const unsigned rest = __ballot_sync(0xffffffffu, !forced);
+                            slot = forced ? m : (int)__fns(~taken, 0, __popc(rest & ((1u << lane) - 1u)) + 1);
+                            slot_s[i][lane] = -1;
+                            if (lane == 0) shared_s[i] = taken;
+                            __syncwarp();
+                            if (lane < n) slot_s[i][slot] = pos;
+                        }
+                        __syncthreads();
+                    }
+                }
+                unsigned char* q = out + (size_t)npk * strip_packet_bytes(sizeof(VT), b.scatter);
+                const int kidx = b.scatter ? 80 : 16;
                 if (lane == 0) reinterpret_cast<int*>(q)[warp] = base;
-                const int L = warp * 8 + (lane & 7), s = lane >> 3;
-                reinterpret_cast<unsigned short*>(q + 16)[L * 4 + s] =
+                if (b.scatter) {
+                    // runs of shared slots: entry of slot j of this item
+                    const unsigned n1 = warp < 3 ? shared_s[warp + 1] : 0u;
+                    const unsigned n2 = warp < 2 ? n1 & shared_s[warp + 2] : 0u;
+                    const unsigned n3 = warp < 1 ? n2 & shared_s[3] : 0u;
+                    const bool chains = ((shared_s[1] & shared_s[2]) | (shared_s[2] & shared_s[3])) != 0;
+                    if (lane == 0 && chains) reinterpret_cast<int*>(q)[warp] = base | INT_MIN;
+                    if (lane < 8) {
+                        unsigned f = 0;
+                        for (int s = 0; s < 4; ++s) {
+                            const int j = 8 * s + lane;
+                            const bool skip = slot_s[warp][j] < 0 || ((shared_s[warp] >> j) & 1u);
+                            f |= (skip ? 1u : 0u) << s | ((n1 >> j) & 1u) << (4 + s) | ((n2 >> j) & 1u) << (8 + s) |
+                                 ((n3 >> j) & 1u) << (12 + s);
+                        }
+                        reinterpret_cast<unsigned short*>(q + 16)[warp * 8 + lane] = (unsigned short)f;
+                    }
+                }
+                const int L = warp * 8 + (slot & 7), s = slot >> 3;
+                reinterpret_cast<unsigned short*>(q + kidx)[L * 4 + s] =
                     lane < n ? (unsigned short)(pos - base) : (unsigned short)kPad;
-                reinterpret_cast<VT*>(q + 16 + 256)[L * 4 + s] = lane < n ? val[src] : VT(0.f);
+                reinterpret_cast<VT*>(q + kidx + 256)[L * 4 + s] = lane < n ? val[src] : VT(0.f);
             }
             p += n;
             ++npk;
@@ -523,7 +639,8 @@ StripFn pick_nw(int nw) {
     switch (nw) {
         case 1: return k_strip<VT, 1, KIND>;
         case 2: return k_strip<VT, 2, KIND>;
-        default: return k_strip<VT, 4, KIND>;
+        case 4: return k_strip<VT, 4, KIND>;
+        default: return k_strip<VT, 8, KIND>;
     }
 }
 
