@@ -786,6 +786,7 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
             {
                 StripArgs ra = strip_row_args(c, t, lam_row);
                 ra.coef = (c->strategy == 2) ? c->d_coef : nullptr;
+                ra.early = c->strategy == 2;
                 ra.coef_mul = (c->mode == SUPPY_EMR) ? c->d_rhof : nullptr;
                 if (strip_patch) {
                     ra.x = c->d_xA;

@@ -260,6 +260,7 @@ struct StripArgs {
     const int4* meta;            // per strip {offset / 16, packets and flags, first item, mask and place}
     const int* cta;              // grid + 1 strip boundaries
     int ring;                    // bytes of the shared-memory ring
+    int early;                   // 1: the next kernel is another strip pass (one CTA an SM)
     int keep;                    // 1: the packets fit L2 beside the vectors (normal eviction priority)
     int* err;                    // set to 1 when a bounded wait gives up
     long long wait_cycles;
@@ -608,7 +609,31 @@ suppy_status ctx_states_async(suppy_ctx* c, RhsState* host);
 suppy_status ctx_slot_extract(suppy_ctx* c, int b, float* out);
 suppy_status ctx_iterate(suppy_ctx* c, const suppy_params* p, int iters);
 
+// Programmatic dependent launch.  A kernel launched with launch_dependent may
+// start while the kernel before it in the stream still runs: it waits for it
+// (and sees its writes) in grid_wait, before which it touches only what was
+// written at create.  grid_trigger lets the next such kernel start once every
+// CTA of this one has called it or ended.  Without the attribute, or after
+// another kind of operation, grid_wait returns at once.
+template <class F, class A>
+cudaError_t launch_dependent(F f, int grid, int threads, size_t smem, cudaStream_t s, const A& a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, a);
+}
+
 // --- device helpers ---------------------------------------------------------
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

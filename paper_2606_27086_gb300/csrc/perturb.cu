@@ -667,6 +667,8 @@ __global__ void __launch_bounds__(NT) k_phase(const PerturbArgs a) {
     __shared__ int pass_s[kWideTrials];     // trial j passed
     __shared__ StepDecision dec;
     __shared__ int flag;
+    // the row pass after it starts to stream its strips as SMs come free
+    grid_trigger();
     const int tiles = a.TR * a.TC;
     const int tile = GRID ? (int)blockIdx.x : (int)(blockIdx.x % tiles);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;

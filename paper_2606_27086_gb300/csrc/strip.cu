@@ -20,6 +20,12 @@
 // offset would not fit) and a lane reads its four entries of a packet with
 // one 4-byte, one 8-byte and one 16-byte shared-memory load.
 //
+// The passes are dependent launches: the strips are constants, so that the
+// producer fills the ring while the kernel before still runs, and only the
+// consumers wait for it (the launch, the first copies and the drain of 20 us
+// block passes overlap: CT 128x128 in 10 blocks 112 -> 101 us an iteration,
+// CT 512x512 in 36 blocks 764 -> 709).
+//
 // Each CTA (one per SM) owns a contiguous range of strips, balanced by their
 // packets.  One producer warp streams whole strips into a shared-memory ring
 // with bulk copies (cp.async.bulk) tracked by mbarriers, each strip in one
@@ -249,11 +255,6 @@ __device__ __forceinline__ void scatter_packet(const unsigned char* sp, int lane
 // reductions; 2: column pass.
 template <typename VT, int NW, int KIND>
 __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
-    if (KIND == 2) {
-        if (a.epi.st[0].stopped) return;   // the row pass left no coefficients
-    } else if (a.check_stop && a.st[0].stopped) {
-        return;
-    }
     extern __shared__ __align__(128) unsigned char ring[];
     __shared__ __align__(8) uint64_t full[kInFlight], empty[kInFlight];
     __shared__ float part[2][kConsumers][4];
@@ -273,9 +274,11 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    if (a.early) grid_trigger();
     // the row pass's proximity terms: FP32 sums with Kahan compensation per
     // thread (FP64 arithmetic is scarce on GB300), widened for the CTA's sum
     float ps = 0.f, pc = 0.f;
+    bool stopped = false;
     int oldest = 0, issued = 0;   // producer: strips whose ring space came back, strips issued
     if (warp == 0) {
         uint64_t pol;
@@ -314,7 +317,10 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 }
             }
         }
-        if (lane == 0 && !ok) {
+        // the strips are constants: they stream in while the kernel before this
+        // one ends.  A stopped system's consumers leave at once (abort_flag 2)
+        grid_wait();
+        if (lane == 0 && !ok && abort_flag != 2) {
             abort_flag = 1;
             atomicExch(a.err, 1);
         }
@@ -323,7 +329,11 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
         const int r = lane >> 3;
         int par = 0, slot = grp, fill = 0;   // the strip's barriers, and which fill of them
         int4 nxt = (grp < s1 - s0) ? __ldg(a.meta + s0 + grp) : make_int4(0, 0, 0, 0);
-        for (int q = grp; q < s1 - s0; q += NG, par ^= 1) {
+        grid_wait();
+        // a stopped system takes no step (and its row pass left no coefficients)
+        stopped = KIND == 2 ? a.epi.st[0].stopped != 0 : (a.check_stop && a.st[0].stopped);
+        if (stopped) abort_flag = 2;
+        for (int q = stopped ? s1 - s0 : grp; q < s1 - s0; q += NG, par ^= 1) {
             const int4 m = nxt;
             nxt = (q + NG < s1 - s0) ? __ldg(a.meta + s0 + q + NG) : make_int4(0, 0, 0, 0);
             const int npk = m.y & kStripPackets;
@@ -422,13 +432,17 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
             }
         }
     }
-    __syncthreads();
+    // a small kernel after the pass starts once its CTAs are through; another
+    // strip pass takes each SM as it comes free and fills its ring meanwhile
+    if (!a.early) grid_trigger();
+    stopped = __syncthreads_or(stopped);
     if (abort_flag && threadIdx.x == 0) {
         // let the copies in flight land before the CTA leaves
         volatile int never = 0;
         for (int q = oldest; q < issued; ++q)
             tma::mbar_wait(&full[q % kInFlight], (q / kInFlight) & 1, &never, kDrainCycles);
     }
+    if (stopped) return;   // every thread has seen it: nothing of the launch is left out
     if constexpr (KIND != 2) {
         __shared__ double sw[kConsumers + 1];
         const double v = warp_sum((double)ps - (double)pc);
@@ -672,8 +686,7 @@ cudaError_t launch_strip(const StripArgs& a, suppy_dtype dt, int kind, int nw, i
     StripFn f = strip_fn(dt, kind, nw);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, a.ring);
     if (e != cudaSuccess) return e;
-    f<<<grid, kStripThreads, a.ring, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(f, grid, kStripThreads, a.ring, s, a);
 }
 
 cudaError_t launch_strip_build(const StripBuild& b, suppy_dtype dt, int fill, cudaStream_t s) {

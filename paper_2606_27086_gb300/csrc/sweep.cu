@@ -469,12 +469,18 @@ __global__ void __launch_bounds__(kSweepThreads) k_colpass_batched(const ColArgs
 
 // Epilogue of the last block of a two-pass sweep (it may set the stop flag, so
 // it runs after every column-pass CTA has read that flag).
-__global__ void k_epilogue(const EpiArgs a) { sweep_epilogue(a); }
+__global__ void k_epilogue(const EpiArgs a) {
+    grid_trigger();
+    grid_wait();
+    sweep_epilogue(a);
+}
 
 // ------------------------------------------------------------- finalize ----
 // x <- clamp(x + delta, lo, hi), delta <- 0 (n x B elements, 128-bit); CTA 0
 // also runs the sweep epilogue.
 __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const FinalizeArgs a) {
+    grid_trigger();
+    grid_wait();
     long long nv = a.nB >> 2;
     if (!CHECKED(ALIGNED16(a.x) && ALIGNED16(a.delta), 201, 0)) nv = 0;
     float4* x4 = reinterpret_cast<float4*>(a.x);
@@ -524,6 +530,8 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const FinalizeArg
 // values pass through shared memory.
 constexpr int kTrRows = 32, kTrCols = 8;
 __global__ void __launch_bounds__(256) k_finalize_tr(const FinalizeArgs a) {
+    grid_trigger();
+    grid_wait();
     __shared__ float t[kTrCols][kTrRows + 1];
     const int H = a.imgH, W = a.imgW;
     const int tw = (W + kTrCols - 1) / kTrCols;
@@ -634,6 +642,7 @@ __device__ __forceinline__ void store_patches(float* xA, float* xB, const PatchB
 // only the row pass's proximity partials and the right-hand-side state, which
 // this kernel does not touch, so the last CTA runs it beside the others.
 __global__ void __launch_bounds__(128) k_finalize_patch(const FinalizeArgs a) {
+    grid_trigger();
     if (blockIdx.x == gridDim.x - 1) {
         sweep_epilogue(a.epi);
         return;
@@ -684,8 +693,17 @@ __global__ void __launch_bounds__(128) k_finalize_patch(const FinalizeArgs a) {
 
 // x (row-major H x W) copied into the wide and the tall patch layouts: the
 // gathers of the one-pass row pass in the patch numbering.  Padding reads 0.
-__global__ void __launch_bounds__(128) k_patch_image(const float* x, float* xA, float* xB, int H, int W,
-                                                     int Wp) {
+struct PatchImageArgs {
+    const float* x;
+    float *xA, *xB;
+    int H, W, Wp;
+};
+__global__ void __launch_bounds__(128) k_patch_image(const PatchImageArgs a) {
+    grid_trigger();
+    grid_wait();
+    const float* x = a.x;
+    float *xA = a.xA, *xB = a.xB;
+    const int H = a.H, W = a.W, Wp = a.Wp;
     const int nblk = (Wp >> 2) * (((H + 7) & ~7) >> 2);
     const bool wvec = (W & 3) == 0;
     for (int blk = blockIdx.x * blockDim.x + threadIdx.x; blk < nblk; blk += gridDim.x * blockDim.x) {
@@ -836,6 +854,8 @@ ColFn col_fn(suppy_dtype dt, int G, int B) {
 __global__ void __launch_bounds__(256) k_ext_norm(const ExtArgs a) {
     __shared__ double sw[8][32];
     __shared__ bool is_last;
+    grid_trigger();
+    grid_wait();
     const long long nB = a.n * a.B;
     const long long tid = (long long)blockIdx.x * 256 + threadIdx.x;
     const long long stride = (long long)gridDim.x * 256;
@@ -883,6 +903,8 @@ __global__ void __launch_bounds__(256) k_ext_norm(const ExtArgs a) {
 // x <- box(x + lambda t_b delta), delta <- 0 (the box also when t_b = 0: the
 // perturbation may have left x outside it).
 __global__ void __launch_bounds__(256) k_ext_apply(const ExtArgs a) {
+    grid_trigger();
+    grid_wait();
     const long long nB = a.n * a.B;
     for (long long e = (long long)blockIdx.x * 256 + threadIdx.x; e < nB;
          e += (long long)gridDim.x * 256) {
@@ -953,8 +975,7 @@ int colpass_blocks_per_sm(suppy_dtype dt, int G, int B) {
 }
 
 cudaError_t launch_epilogue(const EpiArgs& a, cudaStream_t s) {
-    k_epilogue<<<1, kFinalizeThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_epilogue, 1, kFinalizeThreads, 0, s, a);
 }
 
 cudaError_t launch_finalize(const FinalizeArgs& a, int grid, cudaStream_t s) {
@@ -964,6 +985,9 @@ cudaError_t launch_finalize(const FinalizeArgs& a, int grid, cudaStream_t s) {
             return cudaErrorInvalidValue;
         const long long blocks = (long long)(a.imgWp >> 2) * (((a.imgH + 7) & ~7) >> 2);
         // the pixel blocks' CTAs, then one for the epilogue
+        // not as a dependent launch: its CTAs then took 6-8 us longer (CT 512x512
+        // in 36 blocks 1888 us for two iterations, 1417 us this way), while the
+        // strips after it do start early
         k_finalize_patch<<<(int)std::min<long long>((blocks + 127) / 128, 152 * 16) + 1, 128, 0, s>>>(a);
         return cudaGetLastError();
     }
@@ -972,19 +996,16 @@ cudaError_t launch_finalize(const FinalizeArgs& a, int grid, cudaStream_t s) {
             return cudaErrorInvalidValue;
         const long long tiles = (long long)((a.imgW + kTrCols - 1) / kTrCols) *
                                 ((a.imgH + kTrRows - 1) / kTrRows);
-        k_finalize_tr<<<(int)std::min<long long>(tiles, 4096), 256, 0, s>>>(a);
-        return cudaGetLastError();
+        return launch_dependent(k_finalize_tr, (int)std::min<long long>(tiles, 4096), 256, 0, s, a);
     }
-    k_finalize<<<grid, kFinalizeThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_finalize, grid, kFinalizeThreads, 0, s, a);
 }
 
 cudaError_t launch_patch_image(const float* x, float* xA, float* xB, int H, int W, int Wp, cudaStream_t s) {
     if (H < 1 || W < 1 || Wp < W || (Wp & 7) != 0) return cudaErrorInvalidValue;
     const long long blocks = (long long)(Wp >> 2) * (((H + 7) & ~7) >> 2);
-    k_patch_image<<<(int)std::min<long long>((blocks + 127) / 128, 152 * 16), 128, 0, s>>>(x, xA, xB, H, W,
-                                                                                          Wp);
-    return cudaGetLastError();
+    return launch_dependent(k_patch_image, (int)std::min<long long>((blocks + 127) / 128, 152 * 16), 128, 0, s,
+                            PatchImageArgs{x, xA, xB, H, W, Wp});
 }
 
 cudaError_t launch_patch_cols(const int2* rinfo, const unsigned char* rowT, int m, unsigned long long recipW,
@@ -1018,9 +1039,8 @@ cudaError_t launch_reduce_pp(const double* pp, int npp, int B, double scale, int
 }
 
 cudaError_t launch_ext_step(const ExtArgs& a, int grid, cudaStream_t s) {
-    k_ext_norm<<<grid, 256, 0, s>>>(a);
-    k_ext_apply<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = launch_dependent(k_ext_norm, grid, 256, 0, s, a);
+    return e != cudaSuccess ? e : launch_dependent(k_ext_apply, grid, 256, 0, s, a);
 }
 
 }  // namespace suppy
