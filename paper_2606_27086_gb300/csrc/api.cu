@@ -37,9 +37,11 @@ constexpr int kDefaultColMap = 0;
 // (254-257 us a row pass), so the rest stays with L1.  They are taken while
 // their padding stays below kStripSlots slots per entry: at 1.4 an entry costs
 // 8.6 bytes, about the streamed passes' 8, and CT and travel-time rows lie at
-// 1.05-1.10, their columns at 1.11-1.38.
+// 1.05-1.10, their columns at 1.11-1.38.  Where the packets stay in L2 bytes
+// matter less (dose matrices: rows 1.19, columns 1.40).
 constexpr int kStripRing = 160 * 1024;
-constexpr double kStripSlots = 1.4;
+constexpr double kStripSlots = 1.4, kStripSlotsL2 = 1.6;
+constexpr long long kStripL2 = 80LL * 1024 * 1024;
 
 // Stored length of an item: rows and columns start at multiples of four
 // elements and are zero-padded to a multiple of four.
@@ -519,8 +521,8 @@ suppy_status prepare_ext(suppy_ctx* c) {
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
     const long long nB = (long long)c->n * c->B;
     c->xgrid = (int)std::max<long long>(1, std::min<long long>(2LL * sms, (nB + 255) / 256));
-    if ((s = dalloc(c, &c->d_xpart, (size_t)c->xgrid * c->B)) != SUPPY_OK) return s;
-    if ((s = dalloc(c, &c->d_xticket, 1)) != SUPPY_OK) return s;
+    if ((s = dalloc(c, &c->d_xpart, (size_t)std::max(c->xgrid, sms) * c->B)) != SUPPY_OK) return s;
+    if ((s = dalloc(c, &c->d_xticket, 2)) != SUPPY_OK) return s;   // ticket; stop flag of the column pass
     if ((s = dalloc(c, &c->d_tstep, (size_t)c->B)) != SUPPY_OK) return s;
     CK(cudaMemsetAsync(c->d_xticket, 0, sizeof(unsigned), c->stream));
     if (c->mode == SUPPY_EMR) {
@@ -565,7 +567,8 @@ StripArgs strip_row_args(suppy_ctx* c, int t, float lam) {
 // EL / EMR after the column pass of block t (delta holds A^T(W d)): for EMR
 // the row pass over q = A delta (zero bounds, so d = -q; the proximity
 // machinery sums w_i q_i^2 with the multiplier ||a_i||^2), then the step.
-suppy_status enqueue_ext_step(suppy_ctx* c, const suppy_params* p, int t, int npp) {
+suppy_status enqueue_ext_step(suppy_ctx* c, const suppy_params* p, int t, const EpiArgs& epi) {
+    const int npp = epi.npp;
     int nqq = 0;
     if (c->mode == SUPPY_EMR) {
         // the launch writes one partial per CTA: check the buffer first
@@ -621,7 +624,7 @@ suppy_status enqueue_ext_step(suppy_ctx* c, const suppy_params* p, int t, int np
         }
         note_launch(c);
     }
-    ExtArgs e;
+    ExtArgs e{};
     e.x = c->d_x;
     e.delta = c->d_delta;
     e.lo = c->d_lo;
@@ -641,9 +644,23 @@ suppy_status enqueue_ext_step(suppy_ctx* c, const suppy_params* p, int t, int np
     e.lam = (float)p->lambda;
     Timed tm{c, 1};
     CK(tm.begin());
-    CK(launch_ext_step(e, c->xgrid, c->stream));
+    if (c->cstrips.d_blob) {
+        // the column pass left the norm's partials; the epilogue rides along
+        e.norm = c->d_xpart;
+        e.nnorm = c->cstrips.grid[t];
+        e.was_stopped = reinterpret_cast<const int*>(c->d_xticket + 1);
+        if (epi.last_seg) e.epi = epi;
+        CK(launch_ext_step_fused(e, c->xgrid, c->stream));
+        note_launch(c);
+    } else {
+        CK(launch_ext_step(e, c->xgrid, c->stream));
+        note_launch(c, 2);
+        if (epi.last_seg) {
+            CK(launch_epilogue(epi, c->stream));
+            note_launch(c);
+        }
+    }
     CK(tm.end());
-    note_launch(c, 2);
     return SUPPY_OK;
 }
 
@@ -755,6 +772,39 @@ suppy_status enqueue_tile_sweep(suppy_ctx* c, const suppy_params* p, const StopP
     return SUPPY_OK;
 }
 
+// Streamed column pass of block t (CSC copy).  Without an extrapolated step
+// the last block's last CTA runs the sweep epilogue (*fused).
+suppy_status launch_cols_streamed(suppy_ctx* c, int t, const EpiArgs& e2, bool ext, bool* fused) {
+    StreamArgs ca;
+    std::memset(&ca, 0, sizeof(ca));
+    ca.info = c->d_cinfo + (size_t)t * c->n;
+    ca.idx = c->d_ridx;
+    ca.val = c->d_cval;
+    ca.cta_items = c->d_ctpart + c->seg_ctpart_off[t];
+    ca.tile = c->ctile;
+    ca.stages = c->cstages;
+    ca.err = c->d_err;
+    ca.wait_cycles = c->wait_cycles;
+    ca.coef_in = c->d_coef;
+    ca.xw = c->d_x;
+    ca.lo = c->d_lo;
+    ca.hi = c->d_hi;
+    ca.zc = c->d_zc;
+    ca.delta_out = ext ? c->d_delta : nullptr;
+    ca.box_len = c->box_len;
+    ca.epi = e2;
+    *fused = !ext && e2.last_seg && c->d_cticket;
+    ca.ticket = *fused ? c->d_cticket : nullptr;
+    {
+        Timed tm{c, 1};
+        CK(tm.begin());
+        CK(launch_cols_tma(ca, c->dt, c->tGc, c->tMapc, c->seg_ctgrid[t], c->stream));
+        CK(tm.end());
+        note_launch(c);
+    }
+    return SUPPY_OK;
+}
+
 // copies_fresh: the whole-GPU perturbation phase enqueued just before left
 // the patch copies of x (a superiorized iteration), so the sweep need not
 // make them.
@@ -808,34 +858,41 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
                 note_launch(c);
             }
             if (c->strategy == 2) {
-                StripArgs ca;
-                std::memset(&ca, 0, sizeof(ca));
-                ca.blob = c->cstrips.d_blob;
-                ca.meta = c->cstrips.d_meta;
-                ca.cta = c->cstrips.d_cta + c->cstrips.cta_off[t];
-                ca.ring = kStripRing;
-                ca.keep = c->cstrips.keep;
-                ca.err = c->d_err;
-                ca.wait_cycles = c->wait_cycles;
-                ca.x = ca.xT = c->d_coef;
-                ca.xw = c->d_x;
-                ca.lo = c->d_lo;
-                ca.hi = c->d_hi;
-                ca.zc = c->d_zc;
-                ca.delta_out = ext ? c->d_delta : nullptr;
-                ca.box_len = c->box_len;
-                ca.epi = e2;
-                const bool fuse_epi = !ext && e2.last_seg && c->d_cticket;
-                ca.ticket = fuse_epi ? c->d_cticket : nullptr;
-                {
-                    Timed tm{c, 1};
-                    CK(tm.begin());
-                    CK(launch_strip(ca, c->dt, 2, c->cstrips.nw, c->cstrips.grid[t], c->stream));
-                    CK(tm.end());
-                    note_launch(c);
+                bool fuse_epi = false;
+                if (!c->cstrips.d_blob) {
+                    if ((s = launch_cols_streamed(c, t, e2, ext, &fuse_epi)) != SUPPY_OK) return s;
+                } else {
+                    StripArgs ca;
+                    std::memset(&ca, 0, sizeof(ca));
+                    ca.blob = c->cstrips.d_blob;
+                    ca.meta = c->cstrips.d_meta;
+                    ca.cta = c->cstrips.d_cta + c->cstrips.cta_off[t];
+                    ca.ring = kStripRing;
+                    ca.keep = c->cstrips.keep;
+                    ca.err = c->d_err;
+                    ca.wait_cycles = c->wait_cycles;
+                    ca.x = ca.xT = c->d_coef;
+                    ca.xw = c->d_x;
+                    ca.lo = c->d_lo;
+                    ca.hi = c->d_hi;
+                    ca.zc = c->d_zc;
+                    ca.delta_out = ext ? c->d_delta : nullptr;
+                    ca.box_len = c->box_len;
+                    ca.epi = e2;
+                    fuse_epi = !ext && e2.last_seg && c->d_cticket;
+                    ca.norm = ext ? c->d_xpart : nullptr;
+                    ca.was_stopped = ext ? reinterpret_cast<int*>(c->d_xticket + 1) : nullptr;
+                    ca.ticket = fuse_epi ? c->d_cticket : nullptr;
+                    {
+                        Timed tm{c, 1};
+                        CK(tm.begin());
+                        CK(launch_strip(ca, c->dt, 2, c->cstrips.nw, c->cstrips.grid[t], c->stream));
+                        CK(tm.end());
+                        note_launch(c);
+                    }
                 }
-                if (ext && (s = enqueue_ext_step(c, p, t, e2.npp)) != SUPPY_OK) return s;
-                if (e2.last_seg && !fuse_epi) {
+                if (ext && (s = enqueue_ext_step(c, p, t, e2)) != SUPPY_OK) return s;
+                if (e2.last_seg && !fuse_epi && !ext) {
                     CK(launch_epilogue(e2, c->stream));
                     note_launch(c);
                 }
@@ -932,37 +989,10 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
                 note_launch(c);
             }
             if (c->strategy == 2) {
-                StreamArgs ca;
-                std::memset(&ca, 0, sizeof(ca));
-                ca.info = c->d_cinfo + (size_t)t * c->n;
-                ca.idx = c->d_ridx;
-                ca.val = c->d_cval;
-                ca.cta_items = c->d_ctpart + c->seg_ctpart_off[t];
-                ca.tile = c->ctile;
-                ca.stages = c->cstages;
-                ca.err = c->d_err;
-                ca.wait_cycles = c->wait_cycles;
-                ca.coef_in = c->d_coef;
-                ca.xw = c->d_x;
-                ca.lo = c->d_lo;
-                ca.hi = c->d_hi;
-                ca.zc = c->d_zc;
-                ca.delta_out = ext ? c->d_delta : nullptr;
-                ca.box_len = c->box_len;
-                ca.epi = e2;
-                // without an extrapolated step the column pass's last CTA runs
-                // the sweep epilogue (one launch fewer per sweep)
-                const bool fuse_epi = !ext && e2.last_seg && c->d_cticket;
-                ca.ticket = fuse_epi ? c->d_cticket : nullptr;
-                {
-                    Timed tm{c, 1};
-                    CK(tm.begin());
-                    CK(launch_cols_tma(ca, c->dt, c->tGc, c->tMapc, c->seg_ctgrid[t], c->stream));
-                    CK(tm.end());
-                    note_launch(c);
-                }
-                if (ext && (s = enqueue_ext_step(c, p, t, e2.npp)) != SUPPY_OK) return s;
-                if (e2.last_seg && !fuse_epi) {
+                bool fuse_epi = false;
+                if ((s = launch_cols_streamed(c, t, e2, ext, &fuse_epi)) != SUPPY_OK) return s;
+                if (ext && (s = enqueue_ext_step(c, p, t, e2)) != SUPPY_OK) return s;
+                if (e2.last_seg && !fuse_epi && !ext) {
                     CK(launch_epilogue(e2, c->stream));
                     note_launch(c);
                 }
@@ -1023,8 +1053,8 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
                 CK(tm.end());
                 note_launch(c);
             }
-            if (ext && (s = enqueue_ext_step(c, p, t, epi.npp)) != SUPPY_OK) return s;
-            if (epi.last_seg) {
+            if (ext && (s = enqueue_ext_step(c, p, t, epi)) != SUPPY_OK) return s;
+            if (epi.last_seg && !ext) {
                 CK(launch_epilogue(epi, c->stream));
                 note_launch(c);
             }
@@ -1646,7 +1676,8 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
         first[t + 1] = kept;
     }
     const long long bytes = packets * pbytes;
-    if (packets < 1 || (double)packets * 128.0 > kStripSlots * (double)entries + 128.0 ||
+    const double slots = bytes <= kStripL2 ? kStripSlotsL2 : kStripSlots;
+    if (packets < 1 || (double)packets * 128.0 > slots * (double)entries + 128.0 ||
         (long long)most * pbytes > kStripRing / 2 || (bytes >> 4) > 0xffffffffLL)
         return SUPPY_OK;
     S.tall = tall;
@@ -1669,7 +1700,7 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
                         (S.nw < 4 && consumers / S.nw > 2.5 * per_cta)))
         S.nw *= 2;
     // packets that fit L2 (129 MB) beside the vectors stay there between sweeps
-    S.keep = bytes <= 80LL * 1024 * 1024;
+    S.keep = bytes <= kStripL2;
     // per block: contiguous strip ranges of equal packets (and a constant a
     // strip), one per SM
     std::vector<int> cta;
@@ -2544,9 +2575,12 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         if (strategy == 2 && !c->cstrips.d_blob) {
             std::vector<long long> col_blocks(c->nseg + 1);
             for (int t = 0; t <= c->nseg; ++t) col_blocks[t] = (long long)t * n;
+            // columns too unlike for strips are streamed from the CSC copy
+            bool cols_ok = false;
             if ((st = build_strips(c, c->cstrips, c->d_cinfo, c->d_ridx, c->d_cval, col_blocks, true, c->max_col,
-                                   c->nnz_csc, false, false, ok)) != SUPPY_OK)
+                                   c->nnz_csc, false, false, &cols_ok)) != SUPPY_OK)
                 return st;
+            if (!cols_ok && c->max_col > stream_max_item(kMaxTile, stream_stages_for(c->dt, kMaxTile))) *ok = false;
         }
         return SUPPY_OK;
     };
@@ -2653,6 +2687,8 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
             (!group_fits(c->tG, c->max_row, c->tile, c->stages) ||
              (c->strategy == 2 && !group_fits(c->tGc, c->max_col, c->ctile, c->cstages))))
             c->use_tma = false;
+        if (c->strips && c->strategy == 2 && !c->cstrips.d_blob && (st = build_tma_partitions(c)) != SUPPY_OK)
+            return st;
         if (c->use_tma && !c->strips) {
             if ((st = build_tma_partitions(c)) != SUPPY_OK) return st;
             if (tune_streams && !fixed_shape &&
@@ -2710,7 +2746,9 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         c->cstages = best_sh.cstages;
         c->tMapc = best_sh.tMapc;
         c->use_tma = best_sh.use_tma;
-        if (c->use_tma && !c->strips && (s = build_tma_partitions(c)) != SUPPY_OK) return s;
+        if (c->use_tma && !(c->strips && (c->strategy == 1 || c->cstrips.d_blob)) &&
+            (s = build_tma_partitions(c)) != SUPPY_OK)
+            return s;
     } else if ((s = set_up(best, o->tune != 0)) != SUPPY_OK) {
         return s;
     }
@@ -2725,7 +2763,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
     // row copy stays for the proximity)
     if (!c->strips) free_strips(c, c->rstrips);
     if (!(c->strips && c->strategy == 2)) free_strips(c, c->cstrips);
-    if (c->strips && c->strategy == 2) {
+    if (c->strips && c->strategy == 2 && c->cstrips.d_blob) {
         dfree(c, c->d_ridx);
         dfree(c, c->d_cval);
         c->d_ridx = nullptr;
@@ -3582,8 +3620,8 @@ suppy_status suppy_info_get(const suppy_ctx* cc, suppy_info* out) {
         out->block = kStripThreads;
         out->lanes_per_row = 8;
         if (c->strategy == 2) {
-            out->col_grid = c->cstrips.grid[0];
-            out->col_lanes = 8;
+            out->col_grid = c->cstrips.d_blob ? c->cstrips.grid[0] : c->seg_ctgrid[0];
+            out->col_lanes = c->cstrips.d_blob ? 8 : c->tGc;
         }
     } else if (c->use_tma) {
         out->grid = c->seg_tgrid[0];

@@ -286,6 +286,8 @@ struct StripArgs {
     const float* hi;
     const float* zc;
     float* delta_out;
+    double* norm;                // with delta_out: sums of its squares, one per CTA
+    int* was_stopped;            // with norm: the stop flag as the pass found it
     int box_len;
     EpiArgs epi;
     unsigned* ticket;
@@ -430,6 +432,10 @@ struct ExtArgs {
     unsigned* ticket;
     double* tstep;          // B step sizes
     float lam;
+    const double* norm;     // strips (B = 1): ||delta||^2 as nnorm partials, else null
+    int nnorm;
+    const int* was_stopped;
+    EpiArgs epi;            // strips: the sweep's epilogue, run by the last CTA
 };
 
 // --- launchers (defined in sweep.cu / stream.cu / perturb.cu / setup.cu) ----
@@ -528,6 +534,8 @@ cudaError_t launch_column_scaling(const int2* rinfo, const int* col, const void*
                                   suppy_dtype dt, const double* rho, int m, int n, int* counts,
                                   float* zc, cudaStream_t s);
 cudaError_t launch_ext_step(const ExtArgs& a, int grid, cudaStream_t s);
+// the same in one launch, with the norm's partials from the column pass
+cudaError_t launch_ext_step_fused(const ExtArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_to_float(const double* v, int n, float* out, cudaStream_t s);
 cudaError_t launch_colmean(const int* row_ptr, const int* col, const float* val, int m, int n,
                            double* c64, float* c32, double* work, int work_ctas,
@@ -640,6 +648,20 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// Sum of v[c * stride], c < n, by one warp in a fixed order; up to 160 values
+// cost one round of loads (a load and a dependent FP64 add a value took the
+// epilogue of 16 right-hand sides with 1216 partials 17 us).
+__device__ __forceinline__ double warp_sum_strided(const double* v, int n, int stride) {
+    double s = 0.0;
+    for (int c = threadIdx.x & 31; c < n; c += 160) {
+        double p[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) p[u] = c + 32 * u < n ? __ldcg(v + (size_t)(c + 32 * u) * stride) : 0.0;
+        s += ((p[0] + p[1]) + (p[2] + p[3])) + p[4];
+    }
+    return warp_sum(s);
+}
+
 // Column-major index (j mod W) * H + j / W of the row-major pixel j of an
 // H x W image.  j / W is the high word of j * recipW with recipW =
 // floor((2^64 - 1) / W) + 1 = 2^64 / W + e, 0 <= e <= 1: the product over 2^64
@@ -676,53 +698,64 @@ __device__ __forceinline__ float clampf(float v, float lo, float hi) {
     return fminf(fmaxf(v, lo), hi);
 }
 
-// Sweep epilogue, run by one CTA (warp w handles right-hand sides w, w + W,
-// ... for W warps): the proximity partials of the pass summed in a fixed
-// order, the monitored proximity and objective recorded, and the stopping
-// rule of Sec. 2.2.1 / 2.2.3 applied.  The CTA that runs it must be the last
-// reader of the stop flags in its launch.
-__device__ __forceinline__ void sweep_epilogue(const EpiArgs& a) {
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int b = wid; b < a.B; b += blockDim.x / 32) {
-        double s = 0.0;
-        for (int c = lane; c < a.npp; c += 32) s += a.pp[(size_t)c * a.B + b];
-        s = warp_sum(s);
-        if (lane != 0) continue;
-        RhsState& st = a.st[b];
-        if (st.stopped) continue;
-        if (a.first_seg) st.p_acc = 0.0;
-        st.p_acc += a.scale * s;
-        if (!a.last_seg) continue;
-        const double p = a.p_target ? a.p_target[b] : st.p_acc;
-        const int k = st.k;
-        if (k < a.hist_cap) {
-            a.prox_hist[(size_t)b * a.hist_cap + k] = p;
-            a.obj_hist[(size_t)b * a.hist_cap + k] =
-                st.f_valid ? st.f_cur : __longlong_as_double(0x7ff8000000000000LL);
-        }
-        // stopping rule (Sec. 2.2.1 and 2.2.3)
-        if (st.has_prev_p && fabs(p - st.p_prev) / fmax(1.0, st.p_prev) < a.sp.prox_rel)
-            st.calm += 1;
-        else
-            st.calm = 0;
-        const bool feas = (p <= a.sp.prox_abs) || (st.calm >= a.sp.patience);
-        bool objok = true;
-        if (a.sp.has_obj && a.sp.obj_rel > 0.0 && st.f_valid) {
-            objok = st.has_prev_f &&
-                    fabs(st.f_cur - st.f_prev) / fmax(1.0, fabs(st.f_prev)) < a.sp.obj_rel;
-        }
-        st.p_prev = p;
-        st.has_prev_p = 1;
-        if (st.f_valid) {
-            st.f_prev = st.f_cur;
-            st.has_prev_f = 1;
-        }
-        st.f_valid = 0;
-        st.last_prox = p;
-        st.k = k + 1;
-        if ((a.sp.use_stopping && feas && objok) || (a.sp.max_sweeps > 0 && k + 1 >= a.sp.max_sweeps))
-            st.stopped = 1;
+// Sweep epilogue of the right-hand sides [b0, b1), run by one CTA with all its
+// threads: the proximity partials of the pass summed in a fixed order by all
+// warps (several share those of one right-hand side when there are enough),
+// then one thread per right-hand side, in one warp, records the monitored
+// proximity and objective and applies the stopping rule of Sec. 2.2.1 / 2.2.3
+// (its FP64 divisions, scarce on GB300, run for 32 right-hand sides at the
+// price of one).  The CTA that runs it must be the last reader of these stop
+// flags in its launch.
+__device__ __forceinline__ void sweep_epilogue(const EpiArgs& a, int b0, int b1) {
+    __shared__ double part_s[kMaxRhs];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    const int rows = b1 - b0, share = rows < warps ? warps / rows : 1;
+    for (int w = wid; w < rows * share; w += warps) {
+        const int r = w / share, k = w - r * share;
+        const int c0 = (int)((long long)a.npp * k / share), c1 = (int)((long long)a.npp * (k + 1) / share);
+        const double s = warp_sum_strided(a.pp + (size_t)c0 * a.B + b0 + r, c1 - c0, a.B);
+        if (lane == 0) part_s[w] = s;
     }
+    __syncthreads();
+    if ((int)threadIdx.x >= rows) return;
+    const int b = b0 + threadIdx.x;
+    double sum = 0.0;
+    for (int k = 0; k < share; ++k) sum += part_s[threadIdx.x * share + k];
+    RhsState& st = a.st[b];
+    if (st.stopped) return;
+    if (a.first_seg) st.p_acc = 0.0;
+    st.p_acc += a.scale * sum;
+    if (!a.last_seg) return;
+    const double p = a.p_target ? a.p_target[b] : st.p_acc;
+    const int k = st.k;
+    if (k < a.hist_cap) {
+        a.prox_hist[(size_t)b * a.hist_cap + k] = p;
+        a.obj_hist[(size_t)b * a.hist_cap + k] =
+            st.f_valid ? st.f_cur : __longlong_as_double(0x7ff8000000000000LL);
+    }
+    // stopping rule (Sec. 2.2.1 and 2.2.3)
+    if (st.has_prev_p && fabs(p - st.p_prev) / fmax(1.0, st.p_prev) < a.sp.prox_rel)
+        st.calm += 1;
+    else
+        st.calm = 0;
+    const bool feas = (p <= a.sp.prox_abs) || (st.calm >= a.sp.patience);
+    bool objok = true;
+    if (a.sp.has_obj && a.sp.obj_rel > 0.0 && st.f_valid) {
+        objok = st.has_prev_f &&
+                fabs(st.f_cur - st.f_prev) / fmax(1.0, fabs(st.f_prev)) < a.sp.obj_rel;
+    }
+    st.p_prev = p;
+    st.has_prev_p = 1;
+    if (st.f_valid) {
+        st.f_prev = st.f_cur;
+        st.has_prev_f = 1;
+    }
+    st.f_valid = 0;
+    st.last_prox = p;
+    st.k = k + 1;
+    if ((a.sp.use_stopping && feas && objok) || (a.sp.max_sweeps > 0 && k + 1 >= a.sp.max_sweeps))
+        st.stopped = 1;
 }
+__device__ __forceinline__ void sweep_epilogue(const EpiArgs& a) { sweep_epilogue(a, 0, a.B); }
 
 }  // namespace suppy

@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     // the row pass's proximity terms: FP32 sums with Kahan compensation per
     // thread (FP64 arithmetic is scarce on GB300), widened for the CTA's sum
     float ps = 0.f, pc = 0.f;
+    double sq = 0.0;   // column pass: squares of its sums
     bool stopped = false;
     int oldest = 0, issued = 0;   // producer: strips whose ring space came back, strips issued
     if (warp == 0) {
@@ -394,8 +395,10 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
             if constexpr (KIND == 2) {
                 if (has && wi == 0 && (lane & 7) == 0) {
                     const float s = a.zc ? dot * mul : dot;
-                    if (a.delta_out) a.delta_out[item] = s;
-                    else a.xw[item] = clampf(w + s, li, ui);
+                    if (a.delta_out) {
+                        a.delta_out[item] = s;
+                        if (a.norm) sq += (double)s * (double)s;
+                    } else a.xw[item] = clampf(w + s, li, ui);
                 }
             } else {
                 const float d = clampf(dot, li, ui) - dot;
@@ -442,6 +445,7 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
         for (int q = oldest; q < issued; ++q)
             tma::mbar_wait(&full[q % kInFlight], (q / kInFlight) & 1, &never, kDrainCycles);
     }
+    if (KIND == 2 && a.norm && blockIdx.x == 0 && threadIdx.x == 0) *a.was_stopped = stopped;
     if (stopped) return;   // every thread has seen it: nothing of the launch is left out
     if constexpr (KIND != 2) {
         __shared__ double sw[kConsumers + 1];
@@ -454,6 +458,17 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
             a.pp[blockIdx.x] = s;
         }
     } else {
+        if (a.norm) {
+            __shared__ double sw[kConsumers + 1];
+            sq = warp_sum(sq);
+            if (lane == 0) sw[warp] = sq;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                double s = 0.0;
+                for (int k = 1; k <= kConsumers; ++k) s += sw[k];
+                a.norm[blockIdx.x] = s;
+            }
+        }
         __syncthreads();
         if (a.epi.last_seg && a.ticket) {
             // the last CTA to finish runs the sweep epilogue: every CTA of the
