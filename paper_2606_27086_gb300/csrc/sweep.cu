@@ -241,14 +241,141 @@ __global__ void __launch_bounds__(kSweepThreads, SCAT == 0 ? 6 : 2) k_sweep(cons
 }
 
 // ------------------------------------------------------ row pass, B = 4Q ----
+// Dot products of a row with the images of B right-hand sides: lane = e0*Q + q
+// adds entries e0, e0 + E, ... (E = 32/Q) for right-hand sides 4q..4q+3.  A
+// window of 32 entries is read by one coalesced load of a value and an index a
+// lane, the next window's while this one is gathered, and handed out by
+// shuffles: a third of the loads of a lane reading its own entries, and the Q
+// gathers of a window wait for nothing but the window.
+template <typename VT, int Q>
+__device__ __forceinline__ float4 batched_dot(const VT* __restrict__ vals, const int* __restrict__ idx,
+                                              int len, const float* __restrict__ X, int items) {
+    constexpr int E = 32 / Q;
+    constexpr int B = 4 * Q;
+    const int lane = threadIdx.x & 31;
+    const int q = lane % Q;
+    const int e0 = lane / Q;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float v = 0.f;
+    int c = 0;
+    auto window = [&](int e, float& v, int& c) {
+        v = 0.f;
+        c = 0;
+        if (e < len) {
+            v = (float)__ldg(vals + e);
+            c = __ldg(idx + e);
+            if (!CHECKED(c >= 0 && c < items && ALIGNED16(X + (size_t)c * B), 103, e)) c = 0;
+        }
+    };
+    window(lane, v, c);
+    for (int base = 0; base < len; base += 32) {
+        float vn;
+        int cn;
+        window(base + 32 + lane, vn, cn);
+#pragma unroll
+        for (int u = 0; u < Q; ++u) {
+            const float vu = __shfl_sync(0xffffffffu, v, u * E + e0);
+            const int cu = __shfl_sync(0xffffffffu, c, u * E + e0);
+            if (base + u * E + e0 < len) {
+                const float4 xv = __ldg(reinterpret_cast<const float4*>(X + (size_t)cu * B) + q);
+                acc.x = fmaf(vu, xv.x, acc.x);
+                acc.y = fmaf(vu, xv.y, acc.y);
+                acc.z = fmaf(vu, xv.z, acc.z);
+                acc.w = fmaf(vu, xv.w, acc.w);
+            }
+        }
+        v = vn;
+        c = cn;
+    }
+#pragma unroll
+    for (int o = 16; o >= Q; o >>= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+        acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+    }
+    return acc;
+}
+
+// Row pass of two-pass sweeps, B = 4, 8, 16: one warp per row; lane = e0*Q + q
+// holds right-hand sides 4q..4q+3, whose Q lanes gather the contiguous floats
+// X[col*B .. col*B+B) of an entry with 128-bit loads.  The L1 data path bounds
+// it (about one wavefront a gathered pixel).  The warps of a CTA take its rows
+// in turn: neighbouring rays gather the same pixels at the same time (L1 hits 9
+// -> 27% on 16 seismic images of 256 x 512, 26 M nonzeros) and the load is
+// even.  With the window loads and six CTAs an SM 175 -> 148 us (eight CTAs
+// spill: 220; five 151, four 196; window loads with a contiguous run of rows a
+// warp 170); 8 images 140 -> 137, 3 images 120 -> 107.  32 images are faster
+// by the general kernel below (227 against 232 us).
+template <typename VT, int Q>
+__global__ void __launch_bounds__(kSweepThreads, 6) k_rows_batched(const SweepArgs a) {
+    constexpr int B = 4 * Q;
+    constexpr int W = kSweepThreads / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int q = lane % Q;
+    const int e0 = lane / Q;
+    const int rb = a.part[blockIdx.x * W];
+    int re = a.part[blockIdx.x * W + W];
+    if (!CHECKED(rb >= 0 && rb <= re && re <= a.m, 101, blockIdx.x)) re = rb;
+    const VT* __restrict__ val = static_cast<const VT*>(a.val);
+    const int* __restrict__ colp = a.col;
+    const float* __restrict__ X = a.x;
+    bool live[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) live[t] = !a.st[4 * q + t].stopped;
+    double prox[4] = {0.0, 0.0, 0.0, 0.0};
+
+    for (int i = rb + wid; i < re; i += W) {
+        const int2 ri = a.rinfo[i];
+        const int len = ri.y;
+        if (len == 0) continue;
+        if (!CHECKED(ri.x >= 0 && (long long)ri.x + len <= a.nnz, 102, i)) continue;
+        const float4 acc = batched_dot<VT, Q>(val + ri.x, colp + ri.x, len, X, a.n);
+        if (!CHECKED(ALIGNED16(a.l + (size_t)i * B + 4 * q) && ALIGNED16(a.u + (size_t)i * B + 4 * q),
+                     104, i))
+            continue;
+        const float4 lv = __ldg(reinterpret_cast<const float4*>(a.l + (size_t)i * B) + q);
+        const float4 uv = __ldg(reinterpret_cast<const float4*>(a.u + (size_t)i * B) + q);
+        const float w = a.wr[i];
+        const float wp = a.prox_mul ? w * a.prox_mul[i] : w;
+        const float wc = a.coef_mul ? w * a.coef_mul[i] : w;
+        float d[4];
+        d[0] = clampf(acc.x, lv.x, uv.x) - acc.x;
+        d[1] = clampf(acc.y, lv.y, uv.y) - acc.y;
+        d[2] = clampf(acc.z, lv.z, uv.z) - acc.z;
+        d[3] = clampf(acc.w, lv.w, uv.w) - acc.w;
+        float cf[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (e0 == 0) prox[t] += (double)d[t] * (double)d[t] * (double)wp;
+            cf[t] = live[t] ? a.lam * wc * d[t] : 0.f;
+        }
+        if (a.coef && e0 == 0)
+            reinterpret_cast<float4*>(a.coef + (size_t)i * B)[q] = make_float4(cf[0], cf[1], cf[2], cf[3]);
+    }
+    __shared__ double sw[kSweepThreads / 32][B];
+    if (e0 == 0) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) sw[wid][4 * q + t] = prox[t];
+    }
+    __syncthreads();
+    if (threadIdx.x < B) {
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < kSweepThreads / 32; ++w) s += sw[w][threadIdx.x];
+        a.pp[(size_t)blockIdx.x * B + threadIdx.x] = s;
+    }
+}
+
 // One warp per row; lane = e*Q + q handles element slot e (E = 32/Q slots per
 // pass) and right-hand sides 4q..4q+3: the Q lanes of one element gather the
 // contiguous floats X[col*B .. col*B+B) with 128-bit loads and (one-pass)
 // scatter them back with 128-bit vector reductions.  The row is streamed from
-// HBM for the dot products and re-read through L1 for the scatter.  The
-// coefficient-writing variant is held to 32 registers (eight CTAs an SM: more
-// gathers in flight; measured 0.224 -> 0.178 ms on 16 seismic images); the
-// scatter variant stays at five CTAs an SM (it spills under the tighter bound).
+// HBM for the dot products and re-read through L1 for the scatter (in turns and
+// windows as k_rows_batched: 378 us where it takes 368 on 16 seismic images).
+// The coefficient-writing variant, of B = 32 alone, is held to 32 registers
+// (eight CTAs an SM); the scatter variant stays at five CTAs an SM (it spills
+// under the tighter bound).
 template <typename VT, int Q, int SCAT>
 __global__ void __launch_bounds__(kSweepThreads, SCAT == 0 ? 8 : 5) k_sweep_batched(const SweepArgs a) {
     constexpr int E = 32 / Q;
@@ -802,9 +929,9 @@ template <typename VT>
 SweepFn pick_batched(int B, int scat) {
     const bool one = scat != 0;
     switch (B) {
-        case 4: return one ? k_sweep_batched<VT, 1, 1> : k_sweep_batched<VT, 1, 0>;
-        case 8: return one ? k_sweep_batched<VT, 2, 1> : k_sweep_batched<VT, 2, 0>;
-        case 16: return one ? k_sweep_batched<VT, 4, 1> : k_sweep_batched<VT, 4, 0>;
+        case 4: return one ? k_sweep_batched<VT, 1, 1> : k_rows_batched<VT, 1>;
+        case 8: return one ? k_sweep_batched<VT, 2, 1> : k_rows_batched<VT, 2>;
+        case 16: return one ? k_sweep_batched<VT, 4, 1> : k_rows_batched<VT, 4>;
         case 32: return one ? k_sweep_batched<VT, 8, 1> : k_sweep_batched<VT, 8, 0>;
         default: return nullptr;
     }
