@@ -221,6 +221,7 @@ struct suppy_ctx {
     int mq = 0, nstruct = 0, ndvc = 0;
     float dvc_gamma = 0.f;
     size_t dvc_smem = 0;
+    int dvc_dose_ctas = 0, dvc_apply_ctas = 0;
     long long dvc_nnz = 0;
     int* d_qrp = nullptr;
     int* d_qcol = nullptr;
@@ -644,10 +645,10 @@ suppy_status enqueue_ext_step(suppy_ctx* c, const suppy_params* p, int t, const 
     e.lam = (float)p->lambda;
     Timed tm{c, 1};
     CK(tm.begin());
-    if (c->cstrips.d_blob) {
+    if (c->strips || c->use_tma) {
         // the column pass left the norm's partials; the epilogue rides along
         e.norm = c->d_xpart;
-        e.nnorm = c->cstrips.grid[t];
+        e.nnorm = c->cstrips.d_blob ? c->cstrips.grid[t] : c->seg_ctgrid[t];
         e.was_stopped = reinterpret_cast<const int*>(c->d_xticket + 1);
         if (epi.last_seg) e.epi = epi;
         CK(launch_ext_step_fused(e, c->xgrid, c->stream));
@@ -693,6 +694,8 @@ DvcArgs dvc_args(suppy_ctx* c, bool check_stop, int b = 0) {
     a.ndvc = c->ndvc;
     a.smem = c->dvc_smem;
     a.nnz = c->dvc_nnz;
+    a.dose_grid = c->dvc_dose_ctas;
+    a.apply_grid = c->dvc_apply_ctas;
     return a;
 }
 
@@ -706,9 +709,9 @@ suppy_status enqueue_cq_step(suppy_ctx* c) {
     for (int b = 0; b < c->B_user; ++b) {
         const DvcArgs a = dvc_args(c, true, b);
         CK(launch_dvc_dose(a, c->stream));
-        CK(launch_dvc_project(a, c->stream));
+        CK(launch_dvc_project(a, c->stream, false));
         CK(launch_dvc_apply(a, c->stream));
-        note_launch(c, 4);
+        note_launch(c, 3);
     }
     CK(tm.end());
     return SUPPY_OK;
@@ -791,6 +794,8 @@ suppy_status launch_cols_streamed(suppy_ctx* c, int t, const EpiArgs& e2, bool e
     ca.hi = c->d_hi;
     ca.zc = c->d_zc;
     ca.delta_out = ext ? c->d_delta : nullptr;
+    ca.norm = ext ? c->d_xpart : nullptr;
+    ca.was_stopped = ext ? reinterpret_cast<int*>(c->d_xticket + 1) : nullptr;
     ca.box_len = c->box_len;
     ca.epi = e2;
     *fused = !ext && e2.last_seg && c->d_cticket;
@@ -3297,6 +3302,13 @@ suppy_status set_dvc_impl(suppy_ctx* c, const suppy_csr* A, const int32_t* sptr,
     for (int k = 0; k < nstruct; ++k) max_rows = std::max(max_rows, st[k + 1] - st[k]);
     c->dvc_smem = dvc_project_smem(max_rows);
     c->dvc_nnz = A->nnz;
+    c->dvc_dose_ctas = dvc_dose_grid(mq);
+    c->dvc_apply_ctas = dvc_apply_grid(c->n, A->nnz);
+    if (c->dvc_dose_ctas < 1 || c->dvc_apply_ctas < 2) {
+        cudaGetLastError();
+        free_dvc(c);
+        return fail(c, SUPPY_ECUDA, "no resident CTA for the dose-volume kernels");
+    }
     c->dvc_on = true;
     return SUPPY_OK;
 }
@@ -3337,7 +3349,7 @@ suppy_status suppy_dvc_proximity(suppy_ctx* c, double* out) {
     for (int b = 0; b < Bu; ++b) {
         const DvcArgs a = dvc_args(c, false, b);
         CK(launch_dvc_dose(a, c->stream));
-        CK(launch_dvc_project(a, c->stream));
+        CK(launch_dvc_project(a, c->stream, true));
         note_launch(c, 3);
     }
     CK(cudaMemcpyAsync(c->h_out, c->d_target, sizeof(double) * Bu, cudaMemcpyDeviceToHost, c->stream));

@@ -219,6 +219,8 @@ struct StreamArgs {
     EpiArgs epi;
     unsigned* ticket;       // column pass of the last block: CTAs finished (the
                             // last one runs the sweep epilogue), or null
+    double* norm;           // with delta_out: each CTA's sum of squares of delta, and
+    int* was_stopped;       // the stop flag as the pass found it; or null
     // one-pass scatter on an H x W image: rows with rowT[i] set add into
     // deltaT at the column-major index (j mod W) * H + j / W (j / W by a
     // multiply-high with recipW = floor((2^64 - 1) / W) + 1).
@@ -580,16 +582,19 @@ struct DvcArgs {
     int B;                  // stride of x: the context's right-hand sides (x is n x B);
                             // x, xw, st, pd and target point at the one being stepped
     long long nnz;          // entries of A_q
+    int dose_grid, apply_grid;   // dvc_dose_grid, dvc_apply_grid
     size_t smem;            // dynamic shared memory of the projection (keys staged), or 0
 };
 
 constexpr int kDvcCluster = 8;                // CTAs (one cluster) per structure
 constexpr size_t kDvcSmemMax = 192 * 1024;   // structures up to 8 x 49152 rows stage their keys
 size_t dvc_project_smem(int max_rows);
+int dvc_dose_grid(int mq);                    // CTAs: one resident wave at most; 0 on failure
+int dvc_apply_grid(int n, long long nnz);     // likewise, 1 or less on failure
 
 cudaError_t launch_dvc_dose(const DvcArgs& a, cudaStream_t s);
-cudaError_t launch_dvc_project(const DvcArgs& a, cudaStream_t s);   // + the proximity sum
-cudaError_t launch_dvc_apply(const DvcArgs& a, cudaStream_t s);
+cudaError_t launch_dvc_project(const DvcArgs& a, cudaStream_t s, bool total);   // total: + the proximity sum
+cudaError_t launch_dvc_apply(const DvcArgs& a, cudaStream_t s);                 // + the proximity sum
 // part: nstruct x 32 chunk sums (scratch), out: nstruct norms
 cudaError_t launch_dvc_frob(const int* rp, const float* val, const int* sptr, int nstruct,
                             double* part, double* out, cudaStream_t s);

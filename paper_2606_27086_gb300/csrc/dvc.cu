@@ -4,11 +4,11 @@
 //
 //     x <- x + gamma sum_j w_j A_j^T (P_Qj(A_j x) - A_j x),
 //
-// in four launches: the doses d = A_q x (warp per row), the projections onto
+// in three launches: the doses d = A_q x (warp per row), the projections onto
 // the DVC sets (one CTA per structure: radix selection of the K-th highest
-// dose, equal doses ranked by row), the fixed-order sum of the target-space
-// proximity, and the correction gathered per column through the CSC copy of
-// A_q (warp per column, deterministic).
+// dose, equal doses ranked by row), and the correction gathered per column
+// through the CSC copy of A_q (warps per column, deterministic) beside the
+// fixed-order sum of the target-space proximity.
 //
 // Sets (reading of the paper's wording): an upper DVC (D_V <= d_ref) lets at
 // most K = floor(V N) of the structure's N voxels exceed d_ref, a lower DVC
@@ -45,30 +45,66 @@ __device__ __forceinline__ uint32_t dose_key(float f) {
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-// d_i = <a_i, x>: one warp per row, lanes strided over the row; each lane
-// issues the loads of up to eight entries at once (one DRAM round trip per
-// 256 entries of the row), then gathers x (L1-resident); fixed combination
-// order, warp tree.
+// Entries e, e + step, ... of a lane, kBatch at once, and their sum with the
+// gathered y: the loads of one batch run beside the gathers of another.
+constexpr int kBatch = 6;
+struct Batch {
+    int c[kBatch];
+    float v[kBatch];
+    __device__ __forceinline__ void load(const int* __restrict__ idx, const float* __restrict__ val, int e,
+                                         int step, int e1) {
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const bool ok = e + u * step < e1;
+            c[u] = ok ? __ldg(idx + e + u * step) : -1;
+            v[u] = ok ? __ldg(val + e + u * step) : 0.f;
+        }
+    }
+    __device__ __forceinline__ float add(float s, const float* y, int stride) const {
+        float g[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) g[u] = c[u] >= 0 ? y[(size_t)c[u] * stride] : 0.f;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) s = fmaf(v[u], g[u], s);
+        return s;
+    }
+};
+
+// d_i = <a_i, x>: one warp per row, its rows consecutive, lanes strided over
+// the row; the loads of the next row's first 192 entries are issued before
+// this row's gathers of x (L1-resident) and the first row's before grid_wait;
+// fixed combination order, warp tree.  The stream of A_q bounds it (70 MB on a
+// radiotherapy plan of 55,360 rows: 5.2 TB/s while its CTAs run); a row at a
+// time in a grid of 6920 CTAs took 19.1 us, this one 18.0.  Prefetching the
+// matrix into L2 during the perturbation phase before it lost 4 us a CQ step.
 __global__ void __launch_bounds__(kDoseThreads) k_dvc_dose(DvcArgs a) {
-    if (a.st && a.st[0].stopped) return;
+    grid_trigger();
     const int warp = (blockIdx.x * kDoseThreads + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * kDoseThreads) >> 5;
-    for (int i = warp; i < a.mq; i += nw) {
-        const int e0 = a.rp[i], e1 = a.rp[i + 1];
-        float s = 0.f;
-        for (int b = e0; b < e1; b += 256) {
-            int c[8];
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int e = b + u * 32 + lane;
-                const bool ok = e < e1;
-                c[u] = ok ? a.col[e] : 0;
-                v[u] = ok ? __ldg(a.val + e) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) s = fmaf(v[u], __ldg(a.x + (size_t)c[u] * a.B), s);
+    const int i0 = (int)((long long)a.mq * warp / nw), i1 = (int)((long long)a.mq * (warp + 1) / nw);
+    Batch next;
+    int e0 = 0, e1 = 0;
+    if (i0 < i1) {
+        e0 = a.rp[i0];
+        e1 = a.rp[i0 + 1];
+        next.load(a.col, a.val, e0 + lane, 32, e1);
+    }
+    grid_wait();
+    if (a.st && a.st[0].stopped) return;
+    for (int i = i0; i < i1; ++i) {
+        const Batch cur = next;
+        const int f0 = e0, f1 = e1;
+        if (i + 1 < i1) {
+            e0 = e1;
+            e1 = a.rp[i + 2];
+            next.load(a.col, a.val, e0 + lane, 32, e1);
+        }
+        float s = cur.add(0.f, a.x, a.B);
+        for (int b = f0 + 32 * kBatch; b < f1; b += 32 * kBatch) {
+            Batch more;
+            more.load(a.col, a.val, b + lane, 32, f1);
+            s = more.add(s, a.x, a.B);
         }
         s = warp_sum_f(s);
         if (lane == 0) a.dose[i] = s;
@@ -156,6 +192,8 @@ __device__ __forceinline__ uint32_t digit_mask(int) { return 0xffu; }
 // re-reads the doses.
 template <bool SMEM>
 __global__ void __launch_bounds__(kProjectThreads) k_dvc_project(DvcArgs a) {
+    grid_trigger();
+    grid_wait();
     if (a.st && a.st[0].stopped) return;          // uniform over the grid
     cg::cluster_group cl = cg::this_cluster();
     constexpr int CL = kDvcCluster;               // the launch's cluster size
@@ -351,65 +389,82 @@ __global__ void __launch_bounds__(kProjectThreads) k_dvc_project(DvcArgs a) {
 }
 
 // Target-space proximity: 1/2 w_j times each DVC's chunk sums (chunks in rank
-// order), the DVCs in the caller's order.
-__global__ void k_dvc_total(const double* pd, int ndvc, double* out, const RhsState* st) {
-    if (st && st[0].stopped) return;
-    if (threadIdx.x == 0) {
-        const double hw = 0.5 / (double)ndvc;
-        double t = 0.0;
-        for (int j = 0; j < ndvc; ++j) {
-            double u = 0.0;
-            for (int r = 0; r < kDvcCluster; ++r) u += pd[(size_t)j * kDvcCluster + r];
-            t += hw * u;
-        }
-        out[0] = t;
+// order), the DVCs in the caller's order; one thread.
+__device__ __forceinline__ void dvc_total(const DvcArgs& a) {
+    const double hw = 0.5 / (double)a.ndvc;
+    double t = 0.0;
+    for (int j = 0; j < a.ndvc; ++j) {
+        double u = 0.0;
+        for (int r = 0; r < kDvcCluster; ++r) u += __ldcg(a.pd + (size_t)j * kDvcCluster + r);
+        t += hw * u;
     }
+    a.target[0] = t;
+}
+__global__ void k_dvc_total(DvcArgs a) {
+    grid_trigger();
+    grid_wait();
+    if (a.st && a.st[0].stopped) return;
+    if (threadIdx.x == 0) dvc_total(a);
 }
 
 // x_j += gamma sum_i a_ij corr_i over the CSC copy: W warps per column (W
-// chosen from the mean column length), lanes strided over the column; each
-// lane issues the loads of up to eight entries at once, then gathers the
-// corrections; per-warp sums added in warp order.
+// chosen from the mean column length), lanes strided over the column, the
+// first entries of the CTA's next columns loaded before this one's gathers of
+// the corrections; per-warp sums added in warp order.  The last CTA sums the
+// target-space proximity beside the others.  The stream of the CSC copy bounds
+// it (70 MB on a radiotherapy plan of 6003 columns); a CTA and eight warps a
+// column took 26.5 us there and the sum's own launch 4.9, this one 20.9 (eight
+// warps 28.7: a barrier a column of 1455 entries; two warps the same as four).
 template <int W>
 __global__ void __launch_bounds__(kApplyThreads) k_dvc_apply(DvcArgs a) {
-    if (a.st && a.st[0].stopped) return;
     constexpr int kGroups = kApplyThreads / (32 * W);
     constexpr int kStep = 32 * W;
-    __shared__ float part[kApplyThreads / 32];
+    __shared__ float part[2][kApplyThreads / 32];
+    grid_trigger();
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = wid / W, wg = wid % W;
-    for (int j0 = blockIdx.x * kGroups; j0 < a.n; j0 += gridDim.x * kGroups) {
-        const int j = j0 + g;
-        float sum = 0.f;
-        int e1 = 0, e0 = 0;
-        if (j < a.n) {
-            e0 = a.cp[j];
-            e1 = a.cp[j + 1];
-            for (int b = e0 + wg * 32 + lane; b < e1; b += 8 * kStep) {
-                int r[8];
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int e = b + u * kStep;
-                    const bool ok = e < e1;
-                    r[u] = ok ? a.crow[e] : 0;
-                    v[u] = ok ? __ldg(a.cval + e) : 0.f;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) sum = fmaf(v[u], a.corr[r[u]], sum);
-            }
+    const int ctas = gridDim.x - 1;
+    if ((int)blockIdx.x == ctas) {
+        grid_wait();
+        if (threadIdx.x == 0 && !(a.st && a.st[0].stopped)) dvc_total(a);
+        return;
+    }
+    const int stride = ctas * kGroups, off = wg * 32 + lane;
+    int j = blockIdx.x * kGroups + g;
+    Batch next;
+    int e0 = 0, e1 = 0;
+    if (j < a.n) {
+        e0 = a.cp[j];
+        e1 = a.cp[j + 1];
+    }
+    next.load(a.crow, a.cval, e0 + off, kStep, e1);
+    grid_wait();
+    if (a.st && a.st[0].stopped) return;
+    for (int j0 = blockIdx.x * kGroups, par = 0; j0 < a.n; j0 += stride, j += stride, par ^= 1) {
+        const Batch cur = next;
+        const int f0 = e0, f1 = e1;
+        e0 = e1 = 0;
+        if (j + stride < a.n) {
+            e0 = a.cp[j + stride];
+            e1 = a.cp[j + stride + 1];
+        }
+        next.load(a.crow, a.cval, e0 + off, kStep, e1);
+        float sum = cur.add(0.f, a.corr, 1);
+        for (int b = f0 + kBatch * kStep; b < f1; b += kBatch * kStep) {
+            Batch more;
+            more.load(a.crow, a.cval, b + off, kStep, f1);
+            sum = more.add(sum, a.corr, 1);
         }
         const float ws = warp_sum_f(sum);
-        if (lane == 0) part[wid] = ws;
-        __syncthreads();
-        if (wg == 0 && lane == 0 && j < a.n && e1 > e0) {
+        if (lane == 0) part[par][wid] = ws;
+        __syncthreads();   // the next column's sums go to the other half
+        if (wg == 0 && lane == 0 && j < a.n && f1 > f0) {
             float t = 0.f;
 #pragma unroll
-            for (int w = 0; w < W; ++w) t += part[g * W + w];
+            for (int w = 0; w < W; ++w) t += part[par][g * W + w];
             float* xj = a.xw + (size_t)j * a.B;
             *xj = *xj + a.gamma * t;
         }
-        __syncthreads();
     }
 }
 
@@ -449,11 +504,25 @@ __global__ void k_dvc_frob_sum(const double* part, int nstruct, double* out) {
 
 }  // namespace
 
+// resident CTAs of a kernel on the device (the passes above run in one wave)
+template <class F>
+static int wave(F f, int threads) {
+    int dev = 0, sms = 0, nb = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, threads, 0) != cudaSuccess)
+        return 0;
+    return sms * nb;
+}
+
+int dvc_dose_grid(int mq) {
+    return (int)std::min<long long>(((long long)mq * 32 + kDoseThreads - 1) / kDoseThreads,
+                                    wave(k_dvc_dose, kDoseThreads));
+}
+
 cudaError_t launch_dvc_dose(const DvcArgs& a, cudaStream_t s) {
-    const int grid = (int)std::min<long long>(((long long)a.mq * 32 + kDoseThreads - 1) / kDoseThreads,
-                                              152LL * 64);
-    if (a.mq > 0) k_dvc_dose<<<grid, kDoseThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    if (a.mq <= 0) return cudaSuccess;
+    return launch_dependent(k_dvc_dose, a.dose_grid, kDoseThreads, 0, s, a);
 }
 
 size_t dvc_project_smem(int max_rows) {
@@ -461,20 +530,22 @@ size_t dvc_project_smem(int max_rows) {
     return b <= kDvcSmemMax ? b : 0;
 }
 
-cudaError_t launch_dvc_project(const DvcArgs& a, cudaStream_t s) {
+cudaError_t launch_dvc_project(const DvcArgs& a, cudaStream_t s, bool total) {
     if (a.nstruct > 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(a.nstruct * kDvcCluster, 1, 1);
         cfg.blockDim = dim3(kProjectThreads, 1, 1);
         cfg.dynamicSmemBytes = a.smem;
         cfg.stream = s;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = kDvcCluster;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         cudaError_t e;
         if (a.smem > 0) {
             e = cudaFuncSetAttribute(k_dvc_project<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -487,23 +558,35 @@ cudaError_t launch_dvc_project(const DvcArgs& a, cudaStream_t s) {
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_dvc_total<<<1, 32, 0, s>>>(a.pd, a.ndvc, a.target, a.st);
-    return cudaGetLastError();
+    return total ? launch_dependent(k_dvc_total, 1, 32, 0, s, a) : cudaSuccess;
+}
+
+// Warps per column from the mean column length (eight lose at 1455 entries, see
+// k_dvc_apply).
+static int apply_warps(int n, long long nnz) {
+    const long long mean = n > 0 ? nnz / n : 0;
+    return mean >= 512 ? 4 : mean >= 256 ? 2 : 1;
+}
+template <class R, class F>
+static R with_apply(int n, long long nnz, F f) {
+    switch (apply_warps(n, nnz)) {
+        case 4: return f(k_dvc_apply<4>);
+        case 2: return f(k_dvc_apply<2>);
+        default: return f(k_dvc_apply<1>);
+    }
+}
+
+int dvc_apply_grid(int n, long long nnz) {
+    const int groups = kApplyThreads / (32 * apply_warps(n, nnz));
+    const int one = with_apply<int>(n, nnz, [](auto k) { return wave(k, kApplyThreads); }) - 1;
+    return 1 + std::min((n + groups - 1) / groups, one);   // the last CTA sums the proximity
 }
 
 cudaError_t launch_dvc_apply(const DvcArgs& a, cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
-    const long long mean = a.nnz / a.n;
-    const int W = mean >= 1024 ? 8 : mean >= 512 ? 4 : mean >= 256 ? 2 : 1;
-    const int groups = kApplyThreads / (32 * W);
-    const int grid = (int)std::min<long long>((a.n + groups - 1) / groups, 152LL * 64);
-    switch (W) {
-        case 8: k_dvc_apply<8><<<grid, kApplyThreads, 0, s>>>(a); break;
-        case 4: k_dvc_apply<4><<<grid, kApplyThreads, 0, s>>>(a); break;
-        case 2: k_dvc_apply<2><<<grid, kApplyThreads, 0, s>>>(a); break;
-        default: k_dvc_apply<1><<<grid, kApplyThreads, 0, s>>>(a); break;
-    }
-    return cudaGetLastError();
+    return with_apply<cudaError_t>(a.n, a.nnz, [&](auto k) {
+        return launch_dependent(k, a.apply_grid, kApplyThreads, 0, s, a);
+    });
 }
 
 cudaError_t launch_dvc_frob(const int* rp, const float* val, const int* sptr, int nstruct,

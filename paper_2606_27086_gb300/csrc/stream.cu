@@ -618,6 +618,7 @@ struct ColWork {
     const StreamArgs& a;
     float xj = 0.f, lo = 0.f, hi = 0.f, z = 1.f;
     float nx = 0.f, nlo = 0.f, nhi = 0.f, nz = 1.f;
+    double d2 = 0.0;   // sum of squares of the delta written
     __device__ void prefetch(int j) {
         if (j >= 0) {
             const int bj = (a.box_len == 1) ? 0 : j;
@@ -647,8 +648,12 @@ struct ColWork {
         for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(gm, s, o);
         if (a.zc) s *= z;
         if (gl == 0) {
-            if (a.delta_out) a.delta_out[j] = s;
-            else a.xw[j] = clampf(xj + s, lo, hi);
+            if (a.delta_out) {
+                a.delta_out[j] = s;
+                d2 += (double)s * (double)s;
+            } else {
+                a.xw[j] = clampf(xj + s, lo, hi);
+            }
         }
         return 0.0;
     }
@@ -656,9 +661,12 @@ struct ColWork {
 
 template <typename VT, int G, int MAP>
 __global__ void __launch_bounds__(kStreamThreads, 1) k_cols_tma(const StreamArgs a) {
-    if (a.epi.st[0].stopped) return;   // the row pass left no coefficients
+    const int stopped = a.epi.st[0].stopped;
+    if (a.was_stopped && blockIdx.x == 0 && threadIdx.x == 0) *a.was_stopped = stopped;
+    if (stopped) return;   // the row pass left no coefficients
     ColWork<VT, G, MAP> work{a};
     stream_items<VT, G>(a, work);
+    if (a.norm) cta_sum_to(work.d2, a.norm + blockIdx.x);
     __syncthreads();
     if (a.epi.last_seg && a.ticket) {
         // the last CTA to finish runs the sweep epilogue: every CTA of the
