@@ -703,18 +703,34 @@ __device__ __forceinline__ float clampf(float v, float lo, float hi) {
     return fminf(fmaxf(v, lo), hi);
 }
 
+// After a block that is not a sweep's last: the proximity partials of its pass
+// added to the running sums, a warp a right-hand side (the rest of the epilogue
+// below would cost the column passes that call this their registers).
+__device__ __forceinline__ void add_proximity(const EpiArgs& a) {
+    for (int b = threadIdx.x >> 5; b < a.B; b += blockDim.x >> 5) {
+        const double s = warp_sum_strided(a.pp + b, a.npp, a.B);
+        RhsState& st = a.st[b];
+        if ((threadIdx.x & 31) == 0 && !st.stopped) st.p_acc = (a.first_seg ? 0.0 : st.p_acc) + a.scale * s;
+    }
+}
+
 // Sweep epilogue of the right-hand sides [b0, b1), run by one CTA with all its
-// threads: the proximity partials of the pass summed in a fixed order by all
-// warps (several share those of one right-hand side when there are enough),
-// then one thread per right-hand side, in one warp, records the monitored
-// proximity and objective and applies the stopping rule of Sec. 2.2.1 / 2.2.3
-// (its FP64 divisions, scarce on GB300, run for 32 right-hand sides at the
-// price of one).  The CTA that runs it must be the last reader of these stop
-// flags in its launch.
+// threads: the proximity partials of the pass summed in a fixed order (by
+// several warps a right-hand side where there are many), then one thread per
+// right-hand side, in one warp, records the monitored proximity and objective
+// and applies the stopping rule of Sec. 2.2.1 / 2.2.3 (its FP64 divisions,
+// scarce on GB300, run for 32 right-hand sides at the price of one).  It is one
+// chain of latencies at the end of a pass: the state is loaded beside the
+// partials, and the two quotients need not wait for each other.  The CTA that
+// runs it must be the last reader of these stop flags in its launch.
 __device__ __forceinline__ void sweep_epilogue(const EpiArgs& a, int b0, int b1) {
     __shared__ double part_s[kMaxRhs];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-    const int rows = b1 - b0, share = rows < warps ? warps / rows : 1;
+    const int rows = b1 - b0;
+    const int share = max(1, min(warps / rows, a.npp / 160));
+    const int b = b0 + min((int)threadIdx.x, rows - 1);
+    const RhsState was = a.st[b];
+    const double target = a.p_target ? a.p_target[b] : 0.0;
     for (int w = wid; w < rows * share; w += warps) {
         const int r = w / share, k = w - r * share;
         const int c0 = (int)((long long)a.npp * k / share), c1 = (int)((long long)a.npp * (k + 1) / share);
@@ -722,37 +738,32 @@ __device__ __forceinline__ void sweep_epilogue(const EpiArgs& a, int b0, int b1)
         if (lane == 0) part_s[w] = s;
     }
     __syncthreads();
-    if ((int)threadIdx.x >= rows) return;
-    const int b = b0 + threadIdx.x;
+    if ((int)threadIdx.x >= rows || was.stopped) return;
     double sum = 0.0;
     for (int k = 0; k < share; ++k) sum += part_s[threadIdx.x * share + k];
     RhsState& st = a.st[b];
-    if (st.stopped) return;
-    if (a.first_seg) st.p_acc = 0.0;
-    st.p_acc += a.scale * sum;
+    const double p_acc = (a.first_seg ? 0.0 : was.p_acc) + a.scale * sum;
+    st.p_acc = p_acc;
     if (!a.last_seg) return;
-    const double p = a.p_target ? a.p_target[b] : st.p_acc;
-    const int k = st.k;
+    const double p = a.p_target ? target : p_acc;
+    const int k = was.k;
     if (k < a.hist_cap) {
         a.prox_hist[(size_t)b * a.hist_cap + k] = p;
         a.obj_hist[(size_t)b * a.hist_cap + k] =
-            st.f_valid ? st.f_cur : __longlong_as_double(0x7ff8000000000000LL);
+            was.f_valid ? was.f_cur : __longlong_as_double(0x7ff8000000000000LL);
     }
     // stopping rule (Sec. 2.2.1 and 2.2.3)
-    if (st.has_prev_p && fabs(p - st.p_prev) / fmax(1.0, st.p_prev) < a.sp.prox_rel)
-        st.calm += 1;
-    else
-        st.calm = 0;
-    const bool feas = (p <= a.sp.prox_abs) || (st.calm >= a.sp.patience);
-    bool objok = true;
-    if (a.sp.has_obj && a.sp.obj_rel > 0.0 && st.f_valid) {
-        objok = st.has_prev_f &&
-                fabs(st.f_cur - st.f_prev) / fmax(1.0, fabs(st.f_prev)) < a.sp.obj_rel;
-    }
+    const double dp = fabs(p - was.p_prev) / fmax(1.0, was.p_prev);
+    const bool rule = a.sp.has_obj && a.sp.obj_rel > 0.0 && was.f_valid;
+    const double df = rule ? fabs(was.f_cur - was.f_prev) / fmax(1.0, fabs(was.f_prev)) : 0.0;
+    const int calm = was.has_prev_p && dp < a.sp.prox_rel ? was.calm + 1 : 0;
+    st.calm = calm;
+    const bool feas = (p <= a.sp.prox_abs) || (calm >= a.sp.patience);
+    const bool objok = !rule || (was.has_prev_f && df < a.sp.obj_rel);
     st.p_prev = p;
     st.has_prev_p = 1;
-    if (st.f_valid) {
-        st.f_prev = st.f_cur;
+    if (was.f_valid) {
+        st.f_prev = was.f_cur;
         st.has_prev_f = 1;
     }
     st.f_valid = 0;

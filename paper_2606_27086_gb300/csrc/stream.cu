@@ -682,18 +682,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_cols_tma(const StreamArgs
             if (threadIdx.x == 0) *a.ticket = 0u;
         }
     } else if (blockIdx.x == 0 && !a.epi.last_seg) {
-        // CTA 0 also accumulates the row pass's proximity partials of this
-        // block (the last block's are summed by its epilogue)
-        const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int b = wid; b < a.epi.B; b += kStreamThreads / 32) {
-            double s = 0.0;
-            for (int c = lane; c < a.epi.npp; c += 32) s += a.epi.pp[(size_t)c * a.epi.B + b];
-            s = warp_sum(s);
-            if (lane == 0 && !a.epi.st[b].stopped) {
-                if (a.epi.first_seg) a.epi.st[b].p_acc = 0.0;
-                a.epi.st[b].p_acc += a.epi.scale * s;
-            }
-        }
+        add_proximity(a.epi);   // the last block's are summed by its epilogue
     }
 }
 

@@ -331,10 +331,11 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
         int par = 0, slot = grp, fill = 0;   // the strip's barriers, and which fill of them
         int4 nxt = (grp < s1 - s0) ? __ldg(a.meta + s0 + grp) : make_int4(0, 0, 0, 0);
         grid_wait();
-        // a stopped system takes no step (and its row pass left no coefficients)
-        stopped = KIND == 2 ? a.epi.st[0].stopped != 0 : (a.check_stop && a.st[0].stopped);
-        if (stopped) abort_flag = 2;
-        for (int q = stopped ? s1 - s0 : grp; q < s1 - s0; q += NG, par ^= 1) {
+        // a stopped system takes no step (and its row pass left no
+        // coefficients): looked at after the first strip's sums, whose loads
+        // need not wait for the flag's
+        const int flag = KIND == 2 ? a.epi.st[0].stopped : (a.check_stop ? a.st[0].stopped : 0);
+        for (int q = grp; q < s1 - s0; q += NG, par ^= 1) {
             const int4 m = nxt;
             nxt = (q + NG < s1 - s0) ? __ldg(a.meta + s0 + q + NG) : make_int4(0, 0, 0, 0);
             const int npk = m.y & kStripPackets;
@@ -343,19 +344,22 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
             const int item = m.z + r;
             const bool has = ((m.w >> r) & 1) != 0;   // a row with entries; a column of the strip
             const unsigned char* strip = ring + strip_at(m.w);
-            float li = 0.f, ui = 0.f, w = 0.f, mul = 1.f;
-            if (KIND != 2 && has) {
-                li = __ldg(a.l + item);
-                ui = __ldg(a.u + item);
-                w = __ldg(a.wr + item);
+            // loads without a branch or a select behind them, which made the
+            // strip's sums wait for them (about 500 cycles a strip); lanes
+            // without an item repeat the strip's first
+            const int from = has ? item : m.z;
+            float li, ui, w, mul = 1.f;
+            if constexpr (KIND != 2) {
+                li = __ldg(a.l + from);
+                ui = __ldg(a.u + from);
+                w = __ldg(a.wr + from);
                 const float* mp = a.coef_mul ? a.coef_mul : a.prox_mul;
-                if (mp) mul = __ldg(mp + item);
-            }
-            if (KIND == 2 && has && wi == 0) {
-                li = __ldg(a.lo + (a.box_len == 1 ? 0 : item));
-                ui = __ldg(a.hi + (a.box_len == 1 ? 0 : item));
-                w = a.xw[item];   // owned by this strip alone during the pass
-                if (a.zc) mul = __ldg(a.zc + item);
+                mul = __ldg((mp ? mp : a.wr) + from);
+            } else if (wi == 0) {
+                li = __ldg(a.lo + (a.box_len == 1 ? 0 : from));
+                ui = __ldg(a.hi + (a.box_len == 1 ? 0 : from));
+                w = a.xw[from];   // owned by this strip alone during the pass
+                mul = __ldg((a.zc ? a.zc : a.lo) + (a.zc ? from : 0));
             }
             bool ok = bounded_wait(&full[slot], fill, &abort_flag, a.wait_cycles);
             float dot = 0.f;
@@ -379,6 +383,7 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
             if (NW > 1 && (lane & 7) == 0) part[par][cw][r] = dot;
+            if (flag) break;
             ok = group_all<NW>(grp, ok);
             if (!ok) {
                 abort_flag = 1;
@@ -434,10 +439,22 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 fill ^= 1;
             }
         }
+        stopped = flag != 0;
+        if (stopped) abort_flag = 2;
     }
     // a small kernel after the pass starts once its CTAs are through; another
     // strip pass takes each SM as it comes free and fills its ring meanwhile
     if (!a.early) grid_trigger();
+    // the values of the lanes that hold any, side by side for one warp's sum:
+    // FP64 is scarce, and every warp summing its lanes, then a thread the warps,
+    // held the end of each pass for 3950 cycles (1000 to 1600 so)
+    __shared__ float2 prox_s[KIND == 2 ? 1 : 4 * NG];
+    __shared__ double sq_s[KIND == 2 ? 4 * NG : 1];
+    if (warp > 0 && (warp - 1) % NW == 0 && (lane & 7) == 0) {
+        const int k = (warp - 1) / NW * 4 + (lane >> 3);
+        if constexpr (KIND == 2) sq_s[k] = sq;
+        else prox_s[k] = make_float2(ps, pc);
+    }
     stopped = __syncthreads_or(stopped);
     if (abort_flag && threadIdx.x == 0) {
         // let the copies in flight land before the CTA leaves
@@ -448,26 +465,18 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     if (KIND == 2 && a.norm && blockIdx.x == 0 && threadIdx.x == 0) *a.was_stopped = stopped;
     if (stopped) return;   // every thread has seen it: nothing of the launch is left out
     if constexpr (KIND != 2) {
-        __shared__ double sw[kConsumers + 1];
-        const double v = warp_sum((double)ps - (double)pc);
-        if (lane == 0) sw[warp] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int k = 1; k <= kConsumers; ++k) s += sw[k];
-            a.pp[blockIdx.x] = s;
+        if (warp == 0) {
+            double v = 0.0;
+            for (int k = lane; k < 4 * NG; k += 32) v += (double)prox_s[k].x - (double)prox_s[k].y;
+            v = warp_sum(v);
+            if (lane == 0) a.pp[blockIdx.x] = v;
         }
     } else {
-        if (a.norm) {
-            __shared__ double sw[kConsumers + 1];
-            sq = warp_sum(sq);
-            if (lane == 0) sw[warp] = sq;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double s = 0.0;
-                for (int k = 1; k <= kConsumers; ++k) s += sw[k];
-                a.norm[blockIdx.x] = s;
-            }
+        if (a.norm && warp == 0) {
+            double v = 0.0;
+            for (int k = lane; k < 4 * NG; k += 32) v += sq_s[k];
+            v = warp_sum(v);
+            if (lane == 0) a.norm[blockIdx.x] = v;
         }
         __syncthreads();
         if (a.epi.last_seg && a.ticket) {
@@ -484,7 +493,7 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 if (threadIdx.x == 0) *a.ticket = 0u;
             }
         } else if (blockIdx.x == 0 && !a.epi.last_seg) {
-            sweep_epilogue(a.epi);
+            add_proximity(a.epi);
         }
     }
 }

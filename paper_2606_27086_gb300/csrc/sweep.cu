@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(kSweepThreads, SCAT == 0 ? 8 : 5) k_sweep_batc
 // B = 1: a group of G lanes per column j streams its CSC entries and gathers
 // coef from L2; lane 0 applies x_j <- clamp(x_j + sum, lo_j, hi_j).
 template <typename VT, int G>
-__global__ void __launch_bounds__(kSweepThreads) k_colpass(const ColArgs a) {
+__global__ void __launch_bounds__(kSweepThreads, 8) k_colpass(const ColArgs a) {
     // the row pass skipped a stopped system and left no coefficients; the flag
     // cannot change during this launch (the stopping rule runs in k_epilogue)
     if (a.epi.st[0].stopped) return;
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_colpass(const ColArgs a) {
             else a.x[j] = clampf(a.x[j] + s, a.lo[bj], a.hi[bj]);
         }
     }
-    if (blockIdx.x == 0 && !a.epi.last_seg) sweep_epilogue(a.epi);
+    if (blockIdx.x == 0 && !a.epi.last_seg) add_proximity(a.epi);
 }
 
 // B = 4Q: one warp per column; lane = e*Q + q gathers the 4 coefficients of
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_colpass_batched(const ColArgs
             *xp = xv;
         }
     }
-    if (blockIdx.x == 0 && !a.epi.last_seg) sweep_epilogue(a.epi);
+    if (blockIdx.x == 0 && !a.epi.last_seg) add_proximity(a.epi);
 }
 
 // Epilogue of the last block of a two-pass sweep (it may set the stop flag, so
