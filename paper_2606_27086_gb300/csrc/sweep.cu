@@ -305,7 +305,7 @@ __device__ __forceinline__ float4 batched_dot(const VT* __restrict__ vals, const
 // -> 27% on 16 seismic images of 256 x 512, 26 M nonzeros) and the load is
 // even.  With the window loads and six CTAs an SM 175 -> 148 us (eight CTAs
 // spill: 220; five 151, four 196; window loads with a contiguous run of rows a
-// warp 170); 8 images 140 -> 137, 3 images 120 -> 107.  32 images are faster
+// warp 170); 8 images 140 -> 125, 3 images 120 -> 97.  32 images are faster
 // by the general kernel below (227 against 232 us).
 template <typename VT, int Q>
 __global__ void __launch_bounds__(kSweepThreads, 6) k_rows_batched(const SweepArgs a) {
@@ -323,7 +323,18 @@ __global__ void __launch_bounds__(kSweepThreads, 6) k_rows_batched(const SweepAr
     bool live[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) live[t] = !a.st[4 * q + t].stopped;
+    // proximity sums: in shared memory for 4 and 8 images, where registers for
+    // them spill (107 -> 97 and 137 -> 125 us; 16 images 148 -> 174)
+    constexpr bool kInShared = Q < 4;
+    __shared__ double sw[W][B];
     double prox[4] = {0.0, 0.0, 0.0, 0.0};
+    auto to_shared = [&] {
+        if (e0 == 0) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) sw[wid][4 * q + t] = prox[t];
+        }
+    };
+    if (kInShared) to_shared();
 
     for (int i = rb + wid; i < re; i += W) {
         const int2 ri = a.rinfo[i];
@@ -347,17 +358,17 @@ __global__ void __launch_bounds__(kSweepThreads, 6) k_rows_batched(const SweepAr
         float cf[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            if (e0 == 0) prox[t] += (double)d[t] * (double)d[t] * (double)wp;
+            if (e0 == 0) {
+                const double term = (double)d[t] * (double)d[t] * (double)wp;
+                if (kInShared) sw[wid][4 * q + t] += term;
+                else prox[t] += term;
+            }
             cf[t] = live[t] ? a.lam * wc * d[t] : 0.f;
         }
         if (a.coef && e0 == 0)
             reinterpret_cast<float4*>(a.coef + (size_t)i * B)[q] = make_float4(cf[0], cf[1], cf[2], cf[3]);
     }
-    __shared__ double sw[kSweepThreads / 32][B];
-    if (e0 == 0) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) sw[wid][4 * q + t] = prox[t];
-    }
+    if (!kInShared) to_shared();
     __syncthreads();
     if (threadIdx.x < B) {
         double s = 0.0;
