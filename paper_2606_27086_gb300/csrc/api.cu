@@ -38,10 +38,16 @@ constexpr int kDefaultColMap = 0;
 // their padding stays below kStripSlots slots per entry: at 1.4 an entry costs
 // 8.6 bytes, about the streamed passes' 8, and CT and travel-time rows lie at
 // 1.05-1.10, their columns at 1.11-1.38.  Where the packets stay in L2 bytes
-// matter less (dose matrices: rows 1.19, columns 1.40).
+// matter less (dose matrices: rows 1.19, columns 1.40).  Packets of up to 8 MB
+// are taken whatever their padding: a pass over them is a few microseconds of
+// latency, which the streamed passes' rings make more of (row pass in us,
+// streamed and strips: 16x16 in 16 angles 18.4 / 8.0 at 2.2 slots an entry,
+// 32x32 in 500 angles, 7.5 MB, 49.5 / 22.8 at 1.74; columns of 200 travel-time
+// rows over 100x200, 3.7 MB, 70.1 / 12.4 at 22).  Above, the strips lose where
+// padding is common: 26 MB at 2.6 slots 34.9 / 48.3.
 constexpr int kStripRing = 160 * 1024;
 constexpr double kStripSlots = 1.4, kStripSlotsL2 = 1.6;
-constexpr long long kStripL2 = 80LL * 1024 * 1024;
+constexpr long long kStripL2 = 80LL * 1024 * 1024, kStripSmall = 8LL * 1024 * 1024;
 
 // Stored length of an item: rows and columns start at multiples of four
 // elements and are zero-padded to a multiple of four.
@@ -1682,7 +1688,7 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
     }
     const long long bytes = packets * pbytes;
     const double slots = bytes <= kStripL2 ? kStripSlotsL2 : kStripSlots;
-    if (packets < 1 || (double)packets * 128.0 > slots * (double)entries + 128.0 ||
+    if (packets < 1 || (bytes > kStripSmall && (double)packets * 128.0 > slots * (double)entries + 128.0) ||
         (long long)most * pbytes > kStripRing / 2 || (bytes >> 4) > 0xffffffffLL)
         return SUPPY_OK;
     S.tall = tall;
@@ -1693,15 +1699,16 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
     // us with 8 / 4 / 2 / 1 warps: CT 512x512 scatter 269 / 214 / 234 / 332
     // (12.3 KB a strip), 1024x1024 40 angles 117 / 127 / 177 / 301 (24.6 KB),
     // 384x384 FP16 143 / 107 / 96 / 117 (6.4 KB), 128x128 blocks 11.6 / 10.4
-    // / 11.0 / 12.3 (2.7 strips a CTA); 512x512 two passes, rows 196 / 151 /
-    // 145 / 158.
+    // / 11.0 / 12.3 (2.7 strips a CTA), radiotherapy blocks 29.6 / 21.6 / 20.6
+    // / 22.5 (4.2 KB), 64x64 - / 11.7 / 11.9 / 10.5 (2.1 KB); 512x512 two
+    // passes, rows 196 / 151 / 145 / 158.
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
     const double strip_bytes = (double)bytes / std::max(kept, 1);
     const double per_cta = (double)kept / ((double)nseg * sms);
     constexpr int consumers = kStripThreads / 32 - 1;
     S.nw = 1;
-    while (S.nw < 8 && (consumers / S.nw * strip_bytes > (scatter ? 100.0 : 150.0) * 1024 ||
+    while (S.nw < 8 && (consumers / S.nw * strip_bytes > (scatter ? (S.nw == 1 ? 80.0 : 100.0) : 150.0) * 1024 ||
                         (S.nw < 4 && consumers / S.nw > 2.5 * per_cta)))
         S.nw *= 2;
     // packets that fit L2 (129 MB) beside the vectors stay there between sweeps

@@ -6,7 +6,8 @@ few hundred terms: about 1e-7 relative each).
 The sizes sit at the edges of the layout: rows of 1, 31 .. 33 and 127 .. 129
 entries (a packet holds 32 of a row), blocks whose size is not a multiple of
 four, empty rows and columns, unsorted column indices, rows whose entries lie
-further apart than a 16-bit offset reaches, a matrix too ragged for the form.
+further apart than a 16-bit offset reaches, matrices too ragged for the form and
+small ones of the same shape, which take it.
 """
 import numpy as np
 import pytest
@@ -72,14 +73,11 @@ def _takes_strips(prob, strategy, **kw):
 @pytest.mark.parametrize("length", [1, 31, 32, 33, 64, 127, 129, 500])
 @pytest.mark.parametrize("m,n", [(1, 700), (5, 3001), (601, 20011)])
 def test_row_lengths_at_packet_edges(m, n, length, strategy):
-    """One entry a row fills an eighth of its slots, and 33 take two packets:
-    the other forms serve those; nearly full packets are taken."""
+    """One entry a row fills an eighth of its slots, and 33 take two packets;
+    packets this few are taken all the same."""
     prob = _problem([length] * m, n, seed=length + m)
     got = _takes_strips(prob, strategy)
-    if strategy == pk.STRATEGY_ONE_PASS and m > 5 and length in (127, 500):
-        assert got
-    if length == 1 and m > 1:
-        assert not got
+    assert got
     _check(prob, strategy, strips=got)
 
 
@@ -131,13 +129,16 @@ def test_unsorted_rows(strategy):
 def test_offsets_beyond_sixteen_bits():
     """Entries 2100 columns apart: 31 of them fit a packet's offsets, so its
     windows are cut by the offsets, not by the slots; 4000 apart, 16 fit and
-    the other forms take the matrix."""
+    the other forms take the matrix once its packets are more than 8 MB."""
     _check(_problem([310] * 64, 1 << 20, seed=12, spread=2100), pk.STRATEGY_ONE_PASS, strips=True)
-    _check(_problem([200] * 64, 1 << 20, seed=11, spread=4000), pk.STRATEGY_ONE_PASS, strips=False)
+    _check(_problem([200] * 64, 1 << 20, seed=11, spread=4000), pk.STRATEGY_ONE_PASS, strips=True)
+    _check(_problem([200] * 4800, 1 << 20, seed=11, spread=4000), pk.STRATEGY_ONE_PASS, strips=False)
 
 
-def test_ragged_rows_take_the_other_forms():
-    _check(synth.random_problem(700, 20011, seed=4, mean_len=3), pk.STRATEGY_ONE_PASS, strips=False)
+@pytest.mark.parametrize("m,n,strips", [(1, 3, True), (5, 40, True), (700, 20011, True), (80000, 20011, False)])
+@pytest.mark.parametrize("strategy", STRATS)
+def test_ragged_rows_take_the_other_forms_unless_small(m, n, strips, strategy):
+    _check(synth.random_problem(m, n, seed=4, mean_len=3), strategy, strips=strips)
 
 
 def test_fixed_forms_stay_fixed():
