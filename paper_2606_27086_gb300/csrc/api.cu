@@ -1730,6 +1730,37 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
     meta.resize(kept);
     if ((s = dalloc(c, &S.d_blob, (size_t)bytes)) == SUPPY_ENOMEM) return SUPPY_OK;   // the other forms need less
     if (s != SUPPY_OK) return s;
+    // A CTA's consumer groups take its strips in turn; towards the end the
+    // largest go first, so that the groups end together (they ended up to a
+    // third of a pass apart where strips are few and unlike).  The last eleven
+    // rounds and the remainder: 301x217 row pass 34.9 -> 31.5 us, dose rows
+    // 21.7 -> 20.8.  The scatter keeps to the last round, since neighbouring
+    // strips at work together reduce into the same lines: 199x333 rays 22.9 ->
+    // 21.8, 384x384 FP16 92.2 -> 91.3, and with eleven rounds 92.2 -> 97.7.
+    {
+        std::vector<int> order;
+        std::vector<int4> pair;
+        const int groups = consumers / S.nw;
+        for (int t = 0; t < nseg; ++t)
+            for (int g = 0; g < S.grid[t]; ++g) {
+                const int k0 = cta[S.cta_off[t] + g], k1 = cta[S.cta_off[t] + g + 1];
+                const int from = k0 + std::max(0, (k1 - k0) / groups - (scatter ? 1 : 11)) * groups;
+                order.resize(k1 - from);
+                std::iota(order.begin(), order.end(), from);
+                std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+                    return (meta[a].y & kStripPackets) > (meta[b].y & kStripPackets);
+                });
+                pair.clear();
+                for (int k : order) {
+                    pair.push_back(meta[k]);
+                    pair.push_back(strips[k]);
+                }
+                for (int k = from; k < k1; ++k) {
+                    meta[k] = pair[2 * (k - from)];
+                    strips[k] = pair[2 * (k - from) + 1];
+                }
+            }
+    }
     // every CTA's ring, laid out ahead: a strip goes in one piece behind the
     // newest one, or at the ring's start, once the oldest strips in the way
     // (and all but kStripInFlight - 1) have been read
