@@ -1107,8 +1107,8 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
 }
 
 // copies: when not null, the phase also leaves x in the patch layouts of the
-// one-pass sweep that follows it (whole-GPU phase, patch numbering), and
-// *copies says whether it does.
+// one-pass sweep that follows it (whole-GPU phase of a TV objective, patch
+// numbering), and *copies says whether it does.
 suppy_status enqueue_perturb(suppy_ctx* c, const suppy_params* p, int record_only, bool* copies = nullptr) {
     PerturbArgs a{};
     a.x = c->d_x;
@@ -1140,7 +1140,10 @@ suppy_status enqueue_perturb(suppy_ctx* c, const suppy_params* p, int record_onl
     const bool patch_next = c->strategy == 1 && c->tr_patch && c->B == 1 &&
                             (c->strips || (c->use_tma && c->scat == 1 && c->d_rowT && c->tr_on && c->d_colP));
     if (copies) *copies = false;
-    if (copies && patch_next && c->wide && !record_only) {
+    // a phase that walks the unknowns as an image leaves the copies; an
+    // element-wise one walks a range (c->W = n), so the sweep makes them
+    const bool image = c->obj == SUPPY_OBJ_TV_ISO || c->obj == SUPPY_OBJ_TV_ANISO;
+    if (copies && patch_next && image && c->wide && !record_only) {
         a.pA = c->d_xA;
         a.pB = c->d_xB;
         a.pWp = c->gWp;

@@ -151,9 +151,9 @@ struct PerturbArgs {
     unsigned* ticket;       // whole-GPU kernel: grid barrier {arrivals, generation}
     int* err;               // whole-GPU kernel: error word (2: a barrier timed out)
     long long wait_cycles;  // whole-GPU kernel: budget of one barrier wait (SM clock cycles)
-    // whole-GPU kernel, one right-hand side: when set, the phase also leaves
-    // x in the wide / tall patch layouts (padded width pWp) for the one-pass
-    // sweep that follows it
+    // whole-GPU kernel, one right-hand side and a TV objective (the others have
+    // H x W = 1 x n here): when set, the phase also leaves x in the wide / tall
+    // patch layouts (padded width pWp) for the one-pass sweep that follows it
     float* pA;
     float* pB;
     int pWp;

@@ -1495,7 +1495,7 @@ bool wide_phase_tiles(int obj, int n, int H, int W, int sms, PhaseTiles* out) {
 
 cudaError_t launch_phase_tiles(const PerturbArgs& args, const PhaseTiles& t, cudaStream_t s) {
     PerturbArgs a = args;
-    if (!a.ticket || !a.err || !a.part) return cudaErrorInvalidValue;
+    if (!a.ticket || !a.err || !a.part || (a.pA && elem_obj(a.obj))) return cudaErrorInvalidValue;
     set_phase_tiles(a, t);
     const size_t smem = phase_smem(elem_obj(a.obj), t.h, t.w);
     auto kern = phase_fn(a.obj, true, phase_threads(t));
@@ -1535,7 +1535,7 @@ cudaError_t launch_variance(float* x, float* xprev, long long n, int B, RhsState
 }
 
 cudaError_t launch_perturb_wide(const PerturbArgs& a, int grid, cudaStream_t s) {
-    if (!a.ticket || !a.err || !a.part || grid < 1) return cudaErrorInvalidValue;
+    if (!a.ticket || !a.err || !a.part || grid < 1 || (a.pA && elem_obj(a.obj))) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(kPhaseThreads, 1, 1);
