@@ -46,7 +46,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,
     kernels verify indices and vector alignment and report the first violation
     instead of accessing memory."""
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(INCLUDE, "suppy.h")]
+    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + [os.path.join(INCLUDE, "suppy.h")]
     lib = LIB_CHECKED if checked else LIB
     if not force and not _stale(lib, srcs + headers + [__file__]):
         return lib

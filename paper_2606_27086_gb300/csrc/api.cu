@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "strip_rule.h"
 
 using namespace suppy;
 
@@ -33,21 +34,7 @@ constexpr int kMaxTile = 4096;
 constexpr int kDefaultRowMap = 0;
 constexpr int kDefaultColMap = 0;
 
-// Strip-ordered passes.  Ring bytes: CT 512x512 ran the same from 96 to 192 KB
-// (254-257 us a row pass), so the rest stays with L1.  They are taken while
-// their padding stays below kStripSlots slots per entry: at 1.4 an entry costs
-// 8.6 bytes, about the streamed passes' 8, and CT and travel-time rows lie at
-// 1.05-1.10, their columns at 1.11-1.38.  Where the packets stay in L2 bytes
-// matter less (dose matrices: rows 1.19, columns 1.40).  Packets of up to 8 MB
-// are taken whatever their padding: a pass over them is a few microseconds of
-// latency, which the streamed passes' rings make more of (row pass in us,
-// streamed and strips: 16x16 in 16 angles 18.4 / 8.0 at 2.2 slots an entry,
-// 32x32 in 500 angles, 7.5 MB, 49.5 / 22.8 at 1.74; columns of 200 travel-time
-// rows over 100x200, 3.7 MB, 70.1 / 12.4 at 22).  Above, the strips lose where
-// padding is common: 26 MB at 2.6 slots 34.9 / 48.3.
-constexpr int kStripRing = 160 * 1024;
-constexpr double kStripSlots = 1.4, kStripSlotsL2 = 1.6;
-constexpr long long kStripL2 = 80LL * 1024 * 1024, kStripSmall = 8LL * 1024 * 1024;
+constexpr long long kColFixed = 8;   // work of a column beside its entries
 
 // Stored length of an item: rows and columns start at multiples of four
 // elements and are zero-padded to a multiple of four.
@@ -1516,7 +1503,7 @@ suppy_status build_csc(suppy_ctx* c, const std::vector<int>& rp, const int* hcol
         cinfo[k] = make_int2((int)off, (int)cnt[k]);
         const int t = (int)(k / n), j = (int)(k % n);
         long long* pr = c->cpref.data() + (size_t)t * (n + 1);
-        pr[j + 1] = pr[j] + cnt[k] + 8;     // column work: entries plus a fixed cost
+        pr[j + 1] = pr[j] + cnt[k] + kColFixed;   // column work: entries plus a fixed cost
         real += cinfo[k].y;
         cnt[k] = off;                       // becomes the cursor
         off += pad4(cinfo[k].y);
@@ -1627,6 +1614,12 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
                           long long entries, bool scatter, bool patch, bool* ok) {
     *ok = false;
     if (max_len < 1 || max_len > kStripMaxItem) return SUPPY_OK;
+    const int pbytes = strip_packet_bytes(c->dt == SUPPY_F32 ? 4 : 2, scatter);
+    auto len = [&](size_t t, long long i) -> long long {   // entries (rows: padded to four)
+        const long long* w = columns ? c->cpref.data() + t * (c->n + 1LL) + (i - block_of[t]) : c->rpref.data() + i;
+        return w[1] - w[0] - (columns ? kColFixed : 0);
+    };
+    if (!strips_possible(block_of, len, pbytes, entries)) return SUPPY_OK;
     const int nseg = (int)block_of.size() - 1;
     std::vector<int4> strips;
     std::vector<int> seg_first(nseg + 1, 0);
@@ -1637,7 +1630,6 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
         seg_first[t + 1] = (int)strips.size();
     }
     const int ns = (int)strips.size();
-    const int pbytes = strip_packet_bytes(c->dt == SUPPY_F32 ? 4 : 2, scatter);
     TempGuard tg;
     tg.s = c->stream;
     suppy_status s;
@@ -1690,10 +1682,7 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
         first[t + 1] = kept;
     }
     const long long bytes = packets * pbytes;
-    const double slots = bytes <= kStripL2 ? kStripSlotsL2 : kStripSlots;
-    if (packets < 1 || (bytes > kStripSmall && (double)packets * 128.0 > slots * (double)entries + 128.0) ||
-        (long long)most * pbytes > kStripRing / 2 || (bytes >> 4) > 0xffffffffLL)
-        return SUPPY_OK;
+    if (!strips_pay(packets, most, pbytes, entries)) return SUPPY_OK;
     S.tall = tall;
     // Warps a strip: as few as leave the strips in work about half the ring
     // (the scatter holds a strip until it is added; the other passes give it
