@@ -504,9 +504,11 @@ suppy_status suppy_timing_enable(suppy_ctx* ctx, int32_t enable);
 suppy_status suppy_kernel_time(suppy_ctx* ctx, int32_t kind, double* total_ms, int64_t* launches);
 
 /* Budget of every bounded device-side wait of this context's kernels (ring
- * stages of the streamed passes, chunk counters of the tiled sweep, grid
- * barriers of the whole-GPU perturbation phase), in SM clock cycles; 0
- * restores the default (4e9 cycles, about two seconds).  A wait that runs out
+ * stages of the streamed passes, strips in the ring of the strip-ordered
+ * passes, chunk counters of the tiled sweep, grid barriers of the whole-GPU
+ * perturbation phase), in SM clock cycles; 0 restores the default (4e9 cycles,
+ * about two seconds).  A wait's budget covers that wait alone, not the kernel
+ * ahead in the stream.  A wait that runs out
  * makes its kernel stop and the next synchronizing call return SUPPY_ETIMEOUT,
  * after which the context's synchronisation words are reset and the context
  * stays usable.  A diagnostic knob (no paper counterpart): a short budget lets

@@ -309,6 +309,9 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 }
                 issued = b - s0 + __popc(__ballot_sync(0xffffffffu, done && b + lane < s1));
                 if (__all_sync(0xffffffffu, done)) break;
+                // the ring is full, and nothing comes back before the kernel
+                // ahead is over: it is waited for before a wait's budget starts
+                grid_wait();
                 ok = __all_sync(0xffffffffu, bounded_wait(&empty[back], back_fill, &abort_flag, a.wait_cycles));
                 if (!ok) break;
                 ++oldest;
