@@ -275,10 +275,9 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     }
     __syncthreads();
     if (a.early) grid_trigger();
-    // the row pass's proximity terms: FP32 sums with Kahan compensation per
-    // thread (FP64 arithmetic is scarce on GB300), widened for the CTA's sum
-    float ps = 0.f, pc = 0.f;
-    double sq = 0.0;   // column pass: squares of its sums
+    // FP64 sums of the lanes that hold an item: the proximity terms (row pass),
+    // the squares of the sums (column pass)
+    double sq = 0.0;
     bool stopped = false;
     int oldest = 0, issued = 0;   // producer: strips whose ring space came back, strips issued
     if (warp == 0) {
@@ -412,10 +411,7 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 const float d = clampf(dot, li, ui) - dot;
                 const float coef = a.lam * w * d * (a.coef_mul ? mul : 1.f);
                 if (has && wi == 0 && (lane & 7) == 0) {
-                    const float t = d * d * w * (a.prox_mul ? mul : 1.f);
-                    const float y = t - pc, sum = ps + y;
-                    pc = (sum - ps) - y;
-                    ps = sum;
+                    sq += (double)d * (double)d * (double)(a.prox_mul ? w * mul : w);
                     if (KIND == 0 && a.coef) a.coef[item] = coef;
                 }
                 if constexpr (KIND == 1) {
@@ -451,13 +447,8 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     // the values of the lanes that hold any, side by side for one warp's sum:
     // FP64 is scarce, and every warp summing its lanes, then a thread the warps,
     // held the end of each pass for 3950 cycles (1000 to 1600 so)
-    __shared__ float2 prox_s[KIND == 2 ? 1 : 4 * NG];
-    __shared__ double sq_s[KIND == 2 ? 4 * NG : 1];
-    if (warp > 0 && (warp - 1) % NW == 0 && (lane & 7) == 0) {
-        const int k = (warp - 1) / NW * 4 + (lane >> 3);
-        if constexpr (KIND == 2) sq_s[k] = sq;
-        else prox_s[k] = make_float2(ps, pc);
-    }
+    __shared__ double sq_s[4 * NG];
+    if (warp > 0 && (warp - 1) % NW == 0 && (lane & 7) == 0) sq_s[(warp - 1) / NW * 4 + (lane >> 3)] = sq;
     stopped = __syncthreads_or(stopped);
     if (abort_flag && threadIdx.x == 0) {
         // let the copies in flight land before the CTA leaves
@@ -467,20 +458,13 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     }
     if (KIND == 2 && a.norm && blockIdx.x == 0 && threadIdx.x == 0) *a.was_stopped = stopped;
     if (stopped) return;   // every thread has seen it: nothing of the launch is left out
-    if constexpr (KIND != 2) {
-        if (warp == 0) {
-            double v = 0.0;
-            for (int k = lane; k < 4 * NG; k += 32) v += (double)prox_s[k].x - (double)prox_s[k].y;
-            v = warp_sum(v);
-            if (lane == 0) a.pp[blockIdx.x] = v;
-        }
-    } else {
-        if (a.norm && warp == 0) {
-            double v = 0.0;
-            for (int k = lane; k < 4 * NG; k += 32) v += sq_s[k];
-            v = warp_sum(v);
-            if (lane == 0) a.norm[blockIdx.x] = v;
-        }
+    if (warp == 0 && (KIND != 2 || a.norm)) {
+        double v = 0.0;
+        for (int k = lane; k < 4 * NG; k += 32) v += sq_s[k];
+        v = warp_sum(v);
+        if (lane == 0) (KIND != 2 ? a.pp : a.norm)[blockIdx.x] = v;
+    }
+    if constexpr (KIND == 2) {
         __syncthreads();
         if (a.epi.last_seg && a.ticket) {
             // the last CTA to finish runs the sweep epilogue: every CTA of the
