@@ -635,7 +635,7 @@ suppy_status enqueue_ext_step(suppy_ctx* c, const suppy_params* p, int t, const 
     e.part = c->d_xpart;
     e.ticket = c->d_xticket;
     e.tstep = c->d_tstep;
-    e.lam = (float)p->lambda;
+    e.lam = p->lambda;
     Timed tm{c, 1};
     CK(tm.begin());
     if (c->strips || c->use_tma) {

@@ -433,7 +433,7 @@ struct ExtArgs {
     double* part;           // grid x B x 1 partials of ||delta||^2
     unsigned* ticket;
     double* tstep;          // B step sizes
-    float lam;
+    double lam;
     const double* norm;     // strips (B = 1): ||delta||^2 as nnorm partials, else null
     int nnorm;
     const int* was_stopped;

@@ -1041,6 +1041,14 @@ __global__ void __launch_bounds__(256) k_ext_norm(const ExtArgs a) {
     if (threadIdx.x == 0) *a.ticket = 0u;
 }
 
+// v as the sum of two floats.  lambda t multiplies the whole correction: its
+// rounding to one float is an error in every unknown alike, which was most of
+// the step's distance from an FP64 one.
+__device__ __forceinline__ float2 two_floats(double v) {
+    const float hi = (float)v;
+    return make_float2(hi, isfinite(hi) ? (float)(v - (double)hi) : 0.f);
+}
+
 // x <- box(x + lambda t_b delta), delta <- 0 (the box also when t_b = 0: the
 // perturbation may have left x outside it).
 __global__ void __launch_bounds__(256) k_ext_apply(const ExtArgs a) {
@@ -1051,10 +1059,10 @@ __global__ void __launch_bounds__(256) k_ext_apply(const ExtArgs a) {
          e += (long long)gridDim.x * 256) {
         const int b = (int)(e % a.B);
         const long long j = e / a.B;
-        const float t = a.lam * (float)a.tstep[b];
+        const float2 t = two_floats(a.lam * a.tstep[b]);
         const long long bj = (a.box_len == 1) ? 0 : j;
         const float d = a.delta[e];
-        a.x[e] = clampf(a.x[e] + t * d, a.lo[bj], a.hi[bj]);
+        a.x[e] = clampf(a.x[e] + fmaf(t.x, d, t.y * d), a.lo[bj], a.hi[bj]);
         a.delta[e] = 0.f;
     }
 }
@@ -1066,7 +1074,7 @@ __global__ void __launch_bounds__(256) k_ext_apply(const ExtArgs a) {
 // instead of three: norm 9.9, apply 3.5 and epilogue 5.9 us of a 301x217 EMR
 // iteration became 6.0 us.
 __global__ void __launch_bounds__(256) k_ext_fused(const ExtArgs a) {
-    __shared__ float t_s;
+    __shared__ float2 t_s;
     grid_trigger();
     grid_wait();
     const int apply = a.epi.st ? gridDim.x - 1 : gridDim.x;
@@ -1090,18 +1098,18 @@ __global__ void __launch_bounds__(256) k_ext_fused(const ExtArgs a) {
                 if (a.method == SUPPY_EL && d2 > 0.0) t = num / d2;
                 if (a.method == SUPPY_EMR && num > 0.0) t = d2 / num;
             }
-            t_s = a.lam * (float)t;
+            t_s = two_floats(a.lam * t);
         }
     }
     __syncthreads();
-    const float t = t_s;
+    const float2 t = t_s;
     for (long long e = e0; e < a.n; e += (long long)apply * 256) {
         if (e != e0) {
             x = a.x[e];
             d = a.delta[e];
         }
         const long long bj = (a.box_len == 1) ? 0 : e;
-        a.x[e] = clampf(x + t * d, a.lo[bj], a.hi[bj]);
+        a.x[e] = clampf(x + fmaf(t.x, d, t.y * d), a.lo[bj], a.hi[bj]);
         a.delta[e] = 0.f;
     }
 }
