@@ -153,11 +153,19 @@ __device__ __forceinline__ float gather(const float* x, int base, unsigned o) {
         : "l"(x + (base + (int)o)), "r"(o));
     return g;
 }
+// Sums a lane adds its products to.  Four keep the error of the two-pass sweep
+// where the streamed passes have it (CT 257x257, DROP, distance from FP64
+// 7.15e-8 streamed, 7.17e-8 with two, 7.10e-8 with four; same time); the
+// scatter's row pass has no registers for them (512x512 1332 -> 1342 us a call)
+// and is the more exact one as it is (1.21e-7 streamed, 1.14e-7).
+template <int KIND>
+constexpr int kSums = KIND == 1 ? 2 : 4;
+
 // N packets from p: their loads, then their gathers together, then the
 // products, so that they cost one gather latency.
 template <typename VT, int KIND, int N>
 __device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, const float* __restrict__ x,
-                                            float& acc0, float& acc1) {
+                                            float (&acc)[kSums<KIND>]) {
     int base[N];
     uint2 w[N];
     float4 v[N];
@@ -177,10 +185,10 @@ __device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, co
     }
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        acc0 = fmaf(v[k].x, g[k][0], acc0);
-        acc1 = fmaf(v[k].y, g[k][1], acc1);
-        acc0 = fmaf(v[k].z, g[k][2], acc0);
-        acc1 = fmaf(v[k].w, g[k][3], acc1);
+        acc[0] = fmaf(v[k].x, g[k][0], acc[0]);
+        acc[1] = fmaf(v[k].y, g[k][1], acc[1]);
+        acc[2 % kSums<KIND>] = fmaf(v[k].z, g[k][2], acc[2 % kSums<KIND>]);
+        acc[3 % kSums<KIND>] = fmaf(v[k].w, g[k][3], acc[3 % kSums<KIND>]);
     }
 }
 
@@ -367,15 +375,15 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
             float dot = 0.f;
             if (ok) {
                 const float* xs = tall ? a.xT : a.x;
-                float acc0 = 0.f, acc1 = 0.f;
+                float acc[kSums<KIND>] = {};
                 int p = p0;
                 const unsigned char* sp = strip + p0 * Packet<VT, KIND>::kBytes;
                 for (; p + 4 <= p1; p += 4, sp += 4 * Packet<VT, KIND>::kBytes)
-                    dot_packets<VT, KIND, 4>(sp, lane, xs, acc0, acc1);
-                if (p1 - p == 3) dot_packets<VT, KIND, 3>(sp, lane, xs, acc0, acc1);
-                else if (p1 - p == 2) dot_packets<VT, KIND, 2>(sp, lane, xs, acc0, acc1);
-                else if (p1 - p == 1) dot_packets<VT, KIND, 1>(sp, lane, xs, acc0, acc1);
-                dot = acc0 + acc1;
+                    dot_packets<VT, KIND, 4>(sp, lane, xs, acc);
+                if (p1 - p == 3) dot_packets<VT, KIND, 3>(sp, lane, xs, acc);
+                else if (p1 - p == 2) dot_packets<VT, KIND, 2>(sp, lane, xs, acc);
+                else if (p1 - p == 1) dot_packets<VT, KIND, 1>(sp, lane, xs, acc);
+                dot = KIND == 1 ? acc[0] + acc[1] : (acc[0] + acc[1]) + (acc[2 % kSums<KIND>] + acc[3 % kSums<KIND>]);
             }
             if (KIND != 1) {
                 // the strip is read once: its ring space goes back now
