@@ -88,7 +88,8 @@ struct suppy_ctx {
     float* d_xA = nullptr;          // x in the wide / tall patch layouts (the gathers)
     float* d_xB = nullptr;
     int gWp = 0;                    // image width rounded up to a multiple of 8
-    size_t acc_len = 0;             // floats of d_delta and d_deltaT (padded grid when a grid is set)
+    size_t acc_len = 0;             // floats of d_deltaT and the patch copies (padded grid when a grid is set)
+    size_t delta_len = 0;           // floats of d_delta: acc_len or more
     float* d_g = nullptr;
     float* d_lo = nullptr;
     float* d_hi = nullptr;
@@ -535,6 +536,13 @@ suppy_status prepare_ext(suppy_ctx* c) {
     return SUPPY_OK;
 }
 
+// Floats between the copies of the accumulator that the strips add into (0: one
+// accumulator).
+int delta_copy(const suppy_ctx* c) {
+    const bool copies = c->strips && c->strategy == 1 && c->scat == 2 && c->mode == SUPPY_DROP;
+    return copies ? (c->n + 3) & ~3 : 0;
+}
+
 // Row pass of block t over the strip-ordered copy.
 StripArgs strip_row_args(suppy_ctx* c, int t, float lam) {
     StripArgs a;
@@ -551,6 +559,7 @@ StripArgs strip_row_args(suppy_ctx* c, int t, float lam) {
     a.wr = c->d_wr;
     a.x = a.xT = c->d_x;
     a.delta = a.deltaT = c->d_delta;
+    a.copy = delta_copy(c);
     a.pp = c->d_pp;
     a.st = c->d_st;
     a.lam = lam;
@@ -898,6 +907,7 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
                 FinalizeArgs f{};
                 f.x = c->d_x;
                 f.delta = c->d_delta;
+                f.copy = delta_copy(c);
                 if (strip_patch) {
                     f.deltaT = c->d_deltaT;
                     f.imgW = c->gW;
@@ -1569,18 +1579,26 @@ void free_csc(suppy_ctx* c) {
     c->cpref.shrink_to_fit();
 }
 
+// An accumulator of at least len floats, all zero.
+suppy_status grow_delta(suppy_ctx* c, size_t len) {
+    if (len <= c->delta_len) return SUPPY_OK;
+    float* d = nullptr;
+    suppy_status s = dalloc(c, &d, len);
+    if (s != SUPPY_OK) return s;
+    dfree(c, c->d_delta);
+    c->d_delta = d;
+    c->delta_len = len;
+    CK(cudaMemsetAsync(c->d_delta, 0, sizeof(float) * len, c->stream));
+    return SUPPY_OK;
+}
+
 // Both accumulators of the one-pass scatter over the grid padded to multiples
 // of 8 (the patch numbering's lines; the padding is never added into).
 suppy_status alloc_accumulators(suppy_ctx* c) {
     c->gWp = (c->gW + 7) & ~7;
     const size_t acc = std::max((size_t)c->n, (size_t)((c->gH + 7) & ~7) * (size_t)c->gWp);
     suppy_status s;
-    if (acc > c->acc_len) {
-        dfree(c, c->d_delta);
-        c->d_delta = nullptr;
-        if ((s = dalloc(c, &c->d_delta, acc)) != SUPPY_OK) return s;
-        CK(cudaMemsetAsync(c->d_delta, 0, sizeof(float) * acc, c->stream));
-    }
+    if ((s = grow_delta(c, acc)) != SUPPY_OK) return s;
     c->acc_len = acc;
     if (c->d_deltaT) return SUPPY_OK;
     if ((s = dalloc(c, &c->d_deltaT, acc)) != SUPPY_OK) return s;
@@ -2066,7 +2084,7 @@ suppy_status time_config(suppy_ctx* c, float* ms_out, int nsweeps) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->d_st, st.data(), sizeof(RhsState) * c->B, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess && c->d_delta)
-        e = cudaMemsetAsync(c->d_delta, 0, sizeof(float) * std::max(nB, c->acc_len), c->stream);
+        e = cudaMemsetAsync(c->d_delta, 0, sizeof(float) * c->delta_len, c->stream);
     if (e == cudaSuccess && c->d_deltaT)
         e = cudaMemsetAsync(c->d_deltaT, 0, sizeof(float) * c->acc_len, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -2455,7 +2473,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
     if ((s = dalloc(c, &c->d_x, nB)) != SUPPY_OK) return s;
     if ((s = dalloc(c, &c->d_delta, nB)) != SUPPY_OK) return s;
     CK(cudaMemsetAsync(c->d_delta, 0, nB * sizeof(float), c->stream));
-    c->acc_len = nB;
+    c->acc_len = c->delta_len = nB;
     CK(launch_box_init(c->d_x, c->d_lo, c->d_hi, (long long)nB, c->B, c->box_len, nullptr, 0,
                        c->stream));
     note_launch(c);
@@ -2606,6 +2624,8 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         if (patch) {
             if ((st = alloc_accumulators(c)) != SUPPY_OK) return st;
             if ((st = alloc_patch_copies(c)) != SUPPY_OK) return st;
+        } else if (strategy == 1 && smem_ok && c->mode == SUPPY_DROP) {
+            if ((st = grow_delta(c, (size_t)kDeltaCopies * ((n + 3) & ~3))) != SUPPY_OK) return st;
         }
         if (strategy == 2 && !c->cstrips.d_blob) {
             std::vector<long long> col_blocks(c->nseg + 1);

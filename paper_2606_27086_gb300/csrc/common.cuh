@@ -110,6 +110,7 @@ struct FinalizeArgs {
     int patch, imgWp;
     float* xA;
     float* xB;
+    int copy;               // > 0: kDeltaCopies accumulators, this many floats apart (a multiple of 4)
 };
 
 // Column pass of the two-pass sweep: x_j <- box(x_j + sum_i a_ij coef_i)
@@ -254,6 +255,18 @@ constexpr int kStripInFlight = 48;         // strips a CTA's ring holds at most
 // still be in the ring when this one is copied in (6 bits)
 __host__ __device__ constexpr int strip_at(int w) { return ((w >> 4) & 0x3fff) << 4; }
 __host__ __device__ constexpr int strip_live(int w) { return (w >> 18) & 0x3f; }
+// DROP on unknowns that the staged scatter of k_sweep holds in shared memory
+// (64 KB): CTA c adds its corrections into copy c mod kDeltaCopies of the
+// accumulator and the box step sums the copies, so that a correction is a sum of
+// sums as it is there.  One accumulator takes every ray's share one by one, and
+// DROP's corrections are of x's size (Cimmino and BIP divide them by the rows:
+// the same distance from FP64 with every form).  Two sweeps, distance from
+// FP64: staged / one accumulator / 2 / 4 / 8 copies: CT 64x64 8.7e-8 / 14.8e-8 /
+// 9.6e-8 / 7.9e-8 / 7.3e-8, 128x128 13.1 / 14.6 / 9.8 / 8.0 / 7.5, rays through
+// 60x100 3.21 / 3.28 / 3.16 / 3.16 / 3.14.  A sweep of 64x64 takes 11.7 us with
+// one accumulator and 10.3 with four (fewer reductions meet), 60x100 with TV
+// 22.3 and 23.2 (the box step reads more).
+constexpr int kDeltaCopies = 4;
 __host__ __device__ constexpr int strip_packet_bytes(int value_bytes, bool scatter) {
     return 16 + (scatter ? 64 : 0) + 128 * 2 + 128 * value_bytes;   // bases, flags, offsets, values
 }
@@ -275,6 +288,7 @@ struct StripArgs {
     const float* xT;
     float* delta;
     float* deltaT;
+    int copy;                    // floats from one copy of the accumulator to the next, 0: a single one
     float* coef;
     const float* coef_mul;
     const float* prox_mul;

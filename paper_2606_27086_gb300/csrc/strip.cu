@@ -260,8 +260,8 @@ __device__ __forceinline__ void scatter_packet(const unsigned char* sp, int lane
 }
 
 // KIND 0: row pass, coefficients out; 1: row pass with the scatter by L2
-// reductions; 2: column pass.
-template <typename VT, int NW, int KIND>
+// reductions (COPIES: into kDeltaCopies accumulators); 2: column pass.
+template <typename VT, int NW, int KIND, bool COPIES>
 __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     extern __shared__ __align__(128) unsigned char ring[];
     __shared__ __align__(8) uint64_t full[kInFlight], empty[kInFlight];
@@ -431,7 +431,8 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                     float c1 = __shfl_down_sync(0xffffffffu, c0, 8), c2 = __shfl_down_sync(0xffffffffu, c0, 16),
                           c3 = __shfl_down_sync(0xffffffffu, c0, 24);
                     if (__any_sync(0xffffffffu, c0 != 0.f)) {
-                        float* dst = tall ? a.deltaT : a.delta;
+                        float* dst = COPIES ? a.delta + (blockIdx.x % kDeltaCopies) * a.copy
+                                            : (tall ? a.deltaT : a.delta);
                         const unsigned char* sp = strip + p0 * Packet<VT, KIND>::kBytes;
                         for (int p = p0; p < p1; ++p, sp += Packet<VT, KIND>::kBytes)
                             scatter_packet<VT>(sp, lane, c0, c1, c2, c3, dst);
@@ -667,26 +668,27 @@ __global__ void __launch_bounds__(128) k_strip_build(const StripBuild b) {
 
 using StripFn = void (*)(StripArgs);
 
-template <typename VT, int KIND>
+template <typename VT, int KIND, bool COPIES = false>
 StripFn pick_nw(int nw) {
     switch (nw) {
-        case 1: return k_strip<VT, 1, KIND>;
-        case 2: return k_strip<VT, 2, KIND>;
-        case 4: return k_strip<VT, 4, KIND>;
-        default: return k_strip<VT, 8, KIND>;
+        case 1: return k_strip<VT, 1, KIND, COPIES>;
+        case 2: return k_strip<VT, 2, KIND, COPIES>;
+        case 4: return k_strip<VT, 4, KIND, COPIES>;
+        default: return k_strip<VT, 8, KIND, COPIES>;
     }
 }
 
 template <typename VT>
-StripFn pick_kind(int kind, int nw) {
+StripFn pick_kind(int kind, int nw, bool copies) {
     if (kind == 0) return pick_nw<VT, 0>(nw);
-    return kind == 1 ? pick_nw<VT, 1>(nw) : pick_nw<VT, 2>(nw);
+    if (kind == 2) return pick_nw<VT, 2>(nw);
+    return copies ? pick_nw<VT, 1, true>(nw) : pick_nw<VT, 1>(nw);
 }
 
-StripFn strip_fn(suppy_dtype dt, int kind, int nw) {
-    if (dt == SUPPY_F32) return pick_kind<float>(kind, nw);
-    if (dt == SUPPY_BF16) return pick_kind<__nv_bfloat16>(kind, nw);
-    return pick_kind<__half>(kind, nw);
+StripFn strip_fn(suppy_dtype dt, int kind, int nw, bool copies) {
+    if (dt == SUPPY_F32) return pick_kind<float>(kind, nw, copies);
+    if (dt == SUPPY_BF16) return pick_kind<__nv_bfloat16>(kind, nw, copies);
+    return pick_kind<__half>(kind, nw, copies);
 }
 
 template <typename VT>
@@ -702,7 +704,7 @@ cudaError_t build(const StripBuild& b, int fill, int grid, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_strip(const StripArgs& a, suppy_dtype dt, int kind, int nw, int grid, cudaStream_t s) {
-    StripFn f = strip_fn(dt, kind, nw);
+    StripFn f = strip_fn(dt, kind, nw, a.copy > 0);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, a.ring);
     if (e != cudaSuccess) return e;
     return launch_dependent(f, grid, kStripThreads, a.ring, s, a);

@@ -617,19 +617,43 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_epilogue(const EpiArgs a) 
 }
 
 // ------------------------------------------------------------- finalize ----
+__device__ __forceinline__ float add(float a, float b) { return a + b; }
+__device__ __forceinline__ float4 add(float4 a, float4 b) {
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+// The correction of four elements (one): the accumulator's, or the sum of its
+// copies in a fixed order, which go back to zero.
+template <bool COPIES, class T>
+__device__ __forceinline__ T take_delta(T* d, long long v, int copy) {
+    T s[COPIES ? kDeltaCopies : 1];
+#pragma unroll
+    for (int k = 0; k < (COPIES ? kDeltaCopies : 1); ++k) s[k] = d[v + (long long)k * copy];
+#pragma unroll
+    for (int k = 0; k < (COPIES ? kDeltaCopies : 1); ++k) d[v + (long long)k * copy] = T{};
+    if constexpr (COPIES) {
+#pragma unroll
+        for (int o = kDeltaCopies / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < o; ++k) s[k] = add(s[k], s[k + o]);
+    }
+    return s[0];
+}
+
 // x <- clamp(x + delta, lo, hi), delta <- 0 (n x B elements, 128-bit); CTA 0
 // also runs the sweep epilogue.
+template <bool COPIES>
 __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const FinalizeArgs a) {
     grid_trigger();
     grid_wait();
     long long nv = a.nB >> 2;
-    if (!CHECKED(ALIGNED16(a.x) && ALIGNED16(a.delta), 201, 0)) nv = 0;
+    if (!CHECKED(ALIGNED16(a.x) && ALIGNED16(a.delta) && (a.copy & 3) == 0, 201, 0)) nv = 0;
     float4* x4 = reinterpret_cast<float4*>(a.x);
     float4* d4 = reinterpret_cast<float4*>(a.delta);
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += stride) {
         float4 xv = x4[v];
-        float4 dv = d4[v];
+        float4 dv = take_delta<COPIES>(d4, v, a.copy >> 2);
         float lo[4], hi[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -649,14 +673,13 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const FinalizeArg
         xv.z = clampf(xv.z + dv.z, lo[2], hi[2]);
         xv.w = clampf(xv.w + dv.w, lo[3], hi[3]);
         x4[v] = xv;
-        d4[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (blockIdx.x == 0) {
         for (long long idx = 4 * nv + threadIdx.x; idx < a.nB; idx += blockDim.x) {
             const long long j = (a.box_len == 1) ? 0 : idx / a.B;
-            const float d = a.zc ? a.delta[idx] * a.zc[idx / a.B] : a.delta[idx];
+            const float s = take_delta<COPIES>(a.delta, idx, a.copy);
+            const float d = a.zc ? s * a.zc[idx / a.B] : s;
             a.x[idx] = clampf(a.x[idx] + d, a.lo[j], a.hi[j]);
-            a.delta[idx] = 0.f;
         }
         sweep_epilogue(a.epi);
     }
@@ -1194,7 +1217,10 @@ cudaError_t launch_finalize(const FinalizeArgs& a, int grid, cudaStream_t s) {
                                 ((a.imgH + kTrRows - 1) / kTrRows);
         return launch_dependent(k_finalize_tr, (int)std::min<long long>(tiles, 4096), 256, 0, s, a);
     }
-    return launch_dependent(k_finalize, grid, kFinalizeThreads, 0, s, a);
+    // accumulators of up to 64 KB each: small CTAs spread their loads over the SMs
+    if (a.copy > 0)
+        return launch_dependent(k_finalize<true>, (int)std::max<long long>(1, ((a.nB >> 2) + 63) / 64), 64, 0, s, a);
+    return launch_dependent(k_finalize<false>, grid, kFinalizeThreads, 0, s, a);
 }
 
 cudaError_t launch_patch_image(const float* x, float* xA, float* xB, int H, int W, int Wp, cudaStream_t s) {
