@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -189,6 +190,7 @@ struct suppy_ctx {
         long long tall = 0;             // rows in strips of tall patches
     };
     bool strips = false;            // the sweep uses them
+    bool strips_tried = false;      // their copies were asked for at create
     StripSet rstrips, cstrips;
     int* d_err = nullptr;           // set by a kernel whose bounded wait gave up
     long long wait_cycles = kDefaultWaitCycles;   // budget of one bounded device wait
@@ -1654,7 +1656,11 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
     int4* d_strips = nullptr;
     if ((s = stage(c, strips.data(), strips.size(), 0, &d_strips, tg.v)) != SUPPY_OK) return s;
     void* q = nullptr;
-    CK(cudaMalloc(&q, sizeof(int4) * (size_t)std::max(ns, 1)));
+    cudaError_t e = cudaMalloc(&q, sizeof(int4) * (size_t)std::max(ns, 1));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, SUPPY_ENOMEM, std::string("strip records: ") + cudaGetErrorString(e));
+    }
     tg.v.push_back(q);
     StripBuild b;
     std::memset(&b, 0, sizeof(b));
@@ -2060,7 +2066,10 @@ suppy_status time_config(suppy_ctx* c, float* ms_out, int nsweeps) {
     suppy_params_default(&p);
     const size_t nB = (size_t)c->n * c->B;
     float* xs = nullptr;
-    CK(cudaMalloc(&xs, sizeof(float) * nB));
+    if (cudaError_t e = cudaMalloc(&xs, sizeof(float) * nB); e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, SUPPY_ENOMEM, std::string("tuning: ") + cudaGetErrorString(e));
+    }
     std::vector<RhsState> st(c->B);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaMemcpyAsync(xs, c->d_x, sizeof(float) * nB, cudaMemcpyDeviceToDevice, c->stream);
@@ -2204,7 +2213,8 @@ suppy_status tune_tma(suppy_ctx* c, bool tune_map) {
 }
 
 suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, const float* box_lo,
-                         const float* box_hi, const suppy_opts* o, void* stream, suppy_ctx* c) {
+                         const float* box_hi, const suppy_opts* o, void* stream, bool strips_wanted,
+                         suppy_ctx* c) {
     if (!A || !l || !u || !box_lo || !box_hi || !o)
         return fail(c, SUPPY_EINVAL, "NULL argument to suppy_create");
     if (A->m < 0 || A->n < 1 || A->nnz < 0 || !A->row_ptr || (A->nnz > 0 && (!A->col || !A->val)))
@@ -2599,7 +2609,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
     // takes them in the patch numbering on an image grid too large for the
     // staged scatter (smaller images fit L1 and L2 in any numbering, and the
     // patch copies of x would cost a launch), else in the plain one.
-    const bool strips_allowed = c->B == 1 && o->tma == 0 && !o->stream_tile && !o->stream_stages &&
+    const bool strips_allowed = strips_wanted && c->B == 1 && o->tma == 0 && !o->stream_tile && !o->stream_stages &&
                                 !o->stream_lanes && !o->stream_map && !o->stream_col_map &&
                                 o->scatter_transpose == 0 && want != 3 && A->nnz > 0;
     const bool strip_patch = tr_grid && !smem_ok &&
@@ -2612,6 +2622,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         const bool patch = strategy == 1 && strip_patch;
         suppy_status st;
         *ok = true;
+        c->strips_tried = true;
         if (strips_are != strategy) {
             free_strips(c, c->rstrips);
             strips_are = -1;
@@ -2787,6 +2798,7 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         c->strips = best.strip;
         if (best.strip) {
             bool pays = false;
+            if (best.strategy == 1) free_strips(c, c->cstrips);   // as when it was timed
             if ((s = make_strips(best.strategy, &pays)) != SUPPY_OK) return s;
             if (!pays) return fail(c, SUPPY_ENOMEM, "the strip-ordered copy no longer fits");
         }
@@ -2801,9 +2813,8 @@ suppy_status create_impl(const suppy_csr* A, const float* l, const float* u, con
         c->cstages = best_sh.cstages;
         c->tMapc = best_sh.tMapc;
         c->use_tma = best_sh.use_tma;
-        if (c->use_tma && !(c->strips && (c->strategy == 1 || c->cstrips.d_blob)) &&
-            (s = build_tma_partitions(c)) != SUPPY_OK)
-            return s;
+        const bool cols_streamed = c->strips && c->strategy == 2 && !c->cstrips.d_blob;
+        if (((c->use_tma && !c->strips) || cols_streamed) && (s = build_tma_partitions(c)) != SUPPY_OK) return s;
     } else if ((s = set_up(best, o->tune != 0)) != SUPPY_OK) {
         return s;
     }
@@ -3075,16 +3086,27 @@ suppy_status suppy_create(const suppy_csr* A, const float* l, const float* u,
                           void* stream, suppy_ctx** out) {
     if (!out) return fail(nullptr, SUPPY_EINVAL, "out is NULL");
     *out = nullptr;
-    suppy_ctx* c = new (std::nothrow) suppy_ctx();
-    if (!c) return fail(nullptr, SUPPY_ENOMEM, "host allocation failed");
-    suppy_status s = create_impl(A, l, u, box_lo, box_hi, opts, stream, c);
-    if (s != SUPPY_OK) {
+    // the strips are copies beside those that every other form needs: a create
+    // that runs out of memory with them is made again without
+    for (const bool strips : {true, false}) {
+        suppy_ctx* c = new (std::nothrow) suppy_ctx();
+        if (!c) return fail(nullptr, SUPPY_ENOMEM, "host allocation failed");
+        suppy_status s;
+        try {
+            s = create_impl(A, l, u, box_lo, box_hi, opts, stream, strips, c);
+        } catch (const std::bad_alloc&) {
+            s = fail(c, SUPPY_ENOMEM, "host allocation failed");
+        }
+        if (s == SUPPY_OK) {
+            *out = c;
+            return SUPPY_OK;
+        }
+        const bool again = s == SUPPY_ENOMEM && c->strips_tried;
         g_err = c->err;
         destroy_impl(c);
-        return s;
+        if (!again) return s;
     }
-    *out = c;
-    return SUPPY_OK;
+    return SUPPY_ENOMEM;   // not reached: the second attempt returns
 }
 
 void suppy_destroy(suppy_ctx* c) { destroy_impl(c); }
