@@ -188,6 +188,8 @@ struct suppy_ctx {
         int nw = 4;                     // warps per strip (1, 2, 4 or 8)
         int keep = 0;                   // the packets stay in L2 between sweeps
         long long tall = 0;             // rows in strips of tall patches
+        long long bytes = 0;            // of d_blob
+        int count = 0;                  // strips
     };
     bool strips = false;            // the sweep uses them
     bool strips_tried = false;      // their copies were asked for at create
@@ -552,6 +554,11 @@ StripArgs strip_row_args(suppy_ctx* c, int t, float lam) {
     a.blob = c->rstrips.d_blob;
     a.meta = c->rstrips.d_meta;
     a.cta = c->rstrips.d_cta + c->rstrips.cta_off[t];
+    a.blob_bytes = c->rstrips.bytes;
+    a.strips = c->rstrips.count;
+    a.items = c->m;
+    // the patch layouts of x and the accumulators, or x and delta themselves
+    a.x_len = a.delta_len = c->strategy == 1 && c->tr_patch ? (long long)c->acc_len : c->n;
     a.ring = kStripRing;
     a.keep = c->rstrips.keep;
     a.err = c->d_err;
@@ -876,6 +883,10 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
                     ca.blob = c->cstrips.d_blob;
                     ca.meta = c->cstrips.d_meta;
                     ca.cta = c->cstrips.d_cta + c->cstrips.cta_off[t];
+                    ca.blob_bytes = c->cstrips.bytes;
+                    ca.strips = c->cstrips.count;
+                    ca.items = c->n;
+                    ca.x_len = c->m;
                     ca.ring = kStripRing;
                     ca.keep = c->cstrips.keep;
                     ca.err = c->d_err;
@@ -1095,6 +1106,7 @@ suppy_status enqueue_sweep(suppy_ctx* c, const suppy_params* p, bool copies_fres
         CK(cudaStreamSynchronize(c->stream));
         int w[3];
         CK(read_check_word(w));
+        if (!w[0]) CK(read_check_word_strip(w));
         if (w[0])
             return fail(c, SUPPY_EINVAL, "checked build: kernel check " + std::to_string(w[0]) +
                                              " failed at index " +
@@ -1708,6 +1720,8 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
     const long long bytes = packets * pbytes;
     if (!strips_pay(packets, most, pbytes, entries)) return SUPPY_OK;
     S.tall = tall;
+    S.bytes = bytes;
+    S.count = kept;
     // Warps a strip: as few as leave the strips in work about half the ring
     // (the scatter holds a strip until it is added; the other passes give it
     // back at once), since every warp pays about 150 instructions a strip --

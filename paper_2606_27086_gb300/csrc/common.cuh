@@ -274,6 +274,10 @@ struct StripArgs {
     const unsigned char* blob;   // packets
     const int4* meta;            // per strip {offset / 16, packets and flags, first item, mask and place}
     const int* cta;              // grid + 1 strip boundaries
+    // sizes, for the checked build: bytes of the blob, strips, items (bounds or
+    // unknowns), floats behind x and xT, floats behind delta and deltaT
+    long long blob_bytes, x_len, delta_len;
+    int strips, items;
     int ring;                    // bytes of the shared-memory ring
     int early;                   // 1: the next kernel is another strip pass (one CTA an SM)
     int keep;                    // 1: the packets fit L2 beside the vectors (normal eviction priority)
@@ -618,6 +622,7 @@ cudaError_t launch_dvc_frob(const int* rp, const float* val, const int* sptr, in
 // device word (kernel tag, index) and the access is skipped.
 cudaError_t read_check_word(int* out3);   // {tag, index low, index high}; resets the word
 cudaError_t read_check_word_perturb(int* out3);
+cudaError_t read_check_word_strip(int* out3);
 
 // Set the message suppy_last_error(NULL) returns on this thread (api.cu).
 void set_thread_error(const std::string& msg);

@@ -15,37 +15,14 @@
 
 #include <cooperative_groups.h>
 
+#include "check.cuh"
 #include "common.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace suppy {
 
-#ifdef SUPPY_CHECKED
-__device__ int g_check_p[3];
-__device__ __noinline__ bool check_fail_p(int tag, long long idx) {
-    if (atomicCAS(&g_check_p[0], 0, tag) == 0) {
-        g_check_p[1] = (int)(idx & 0xffffffffLL);
-        g_check_p[2] = (int)(idx >> 32);
-    }
-    return false;
-}
-#define PCHECKED(cond, tag, idx) ((cond) ? true : check_fail_p((tag), (long long)(idx)))
-#else
-#define PCHECKED(cond, tag, idx) true
-#endif
-
-cudaError_t read_check_word_perturb(int* out3) {
-#ifdef SUPPY_CHECKED
-    cudaError_t e = cudaMemcpyFromSymbol(out3, g_check_p, sizeof(int) * 3);
-    if (e != cudaSuccess) return e;
-    int z[3] = {0, 0, 0};
-    return cudaMemcpyToSymbol(g_check_p, z, sizeof(int) * 3);
-#else
-    out3[0] = out3[1] = out3[2] = 0;
-    return cudaSuccess;
-#endif
-}
+cudaError_t read_check_word_perturb(int* out3) { return take_check_words(out3); }
 
 namespace {
 
@@ -676,8 +653,13 @@ __global__ void __launch_bounds__(NT) k_phase(const PerturbArgs a) {
     const int H = KIND == 2 ? 1 : a.H, W = KIND == 2 ? n : a.W;
     // the first xh rows (xw columns) of rectangles are one pixel larger
     const int ti = (int)((unsigned)tile / (unsigned)a.TC), tj = tile - ti * a.TC;
-    const int h = a.th + (ti < a.xh ? 1 : 0), w = a.tw + (tj < a.xw ? 1 : 0), own = h * w;
+    int h = a.th + (ti < a.xh ? 1 : 0), w = a.tw + (tj < a.xw ? 1 : 0);
     const int r0 = ti * a.th + min(ti, a.xh), c0 = tj * a.tw + min(tj, a.xw);
+    if (!CHECKED(h <= a.tmh && w <= a.tmw && r0 + h <= H && c0 + w <= W && (long long)H * W == n &&
+                     (!a.pA || (KIND != 2 && W <= a.pWp)),
+                 401, tile))
+        h = w = 0;
+    const int own = h * w;
     const bool lin = KIND == 2 && obj == SUPPY_OBJ_LINEAR;
     // y with a halo of one pixel up / left and two down / right (the
     // subgradient is needed one pixel down / right of the rectangle)

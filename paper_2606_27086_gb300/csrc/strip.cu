@@ -50,10 +50,13 @@
 #include <algorithm>
 #include <climits>
 
+#include "check.cuh"
 #include "common.cuh"
 #include "tma.cuh"
 
 namespace suppy {
+
+cudaError_t read_check_word_strip(int* out3) { return take_check_words(out3); }
 
 namespace {
 
@@ -165,7 +168,7 @@ constexpr int kSums = KIND == 1 ? 2 : 4;
 // products, so that they cost one gather latency.
 template <typename VT, int KIND, int N>
 __device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, const float* __restrict__ x,
-                                            float (&acc)[kSums<KIND>]) {
+                                            long long x_len, float (&acc)[kSums<KIND>]) {
     int base[N];
     uint2 w[N];
     float4 v[N];
@@ -179,9 +182,12 @@ __device__ __forceinline__ void dot_packets(const unsigned char* p, int lane, co
     float g[N][4];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        const unsigned o[4] = {w[k].x & 0xffffu, w[k].x >> 16, w[k].y & 0xffffu, w[k].y >> 16};
+        unsigned o[4] = {w[k].x & 0xffffu, w[k].x >> 16, w[k].y & 0xffffu, w[k].y >> 16};
 #pragma unroll
-        for (int s = 0; s < 4; ++s) g[k][s] = gather(x, base[k], o[s]);
+        for (int s = 0; s < 4; ++s) {
+            if (!CHECKED(o[s] == kPad || (base[k] >= 0 && base[k] + (long long)o[s] < x_len), 501, base[k])) o[s] = kPad;
+            g[k][s] = gather(x, base[k], o[s]);
+        }
     }
 #pragma unroll
     for (int k = 0; k < N; ++k) {
@@ -222,7 +228,7 @@ __device__ __forceinline__ void red_unless(unsigned f, float* p, float v) {
 // coefficients of the lane's item and of those after it (0 past the strip).
 template <typename VT>
 __device__ __forceinline__ void scatter_packet(const unsigned char* sp, int lane, float c0, float c1, float c2,
-                                               float c3, float* __restrict__ dst) {
+                                               float c3, float* __restrict__ dst, long long dst_len) {
     using Pk = Packet<VT, 1>;
     constexpr int kItem = 8 * 4 * (int)sizeof(VT);   // bytes from one item's values to the next's
     const int word = *reinterpret_cast<const int*>(sp + 4 * (lane >> 3));
@@ -252,11 +258,15 @@ __device__ __forceinline__ void scatter_packet(const unsigned char* sp, int lane
     }
     // a row inside its slab adds nothing of its own
     if (c0 == 0.f) f |= ~(f >> 4) & 0xfu;
+    const unsigned off[4] = {ix.x & 0xffffu, ix.x >> 16, ix.y & 0xffffu, ix.y >> 16};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (!CHECKED(((f >> k) & 1u) || (base >= 0 && base + (long long)off[k] < dst_len), 502, base)) f |= 1u << k;
     float* const d = dst + base;
-    red_unless<1u>(f, d + (ix.x & 0xffffu), s[0]);
-    red_unless<2u>(f, d + (ix.x >> 16), s[1]);
-    red_unless<4u>(f, d + (ix.y & 0xffffu), s[2]);
-    red_unless<8u>(f, d + (ix.y >> 16), s[3]);
+    red_unless<1u>(f, d + off[0], s[0]);
+    red_unless<2u>(f, d + off[1], s[1]);
+    red_unless<4u>(f, d + off[2], s[2]);
+    red_unless<8u>(f, d + off[3], s[3]);
 }
 
 // KIND 0: row pass, coefficients out; 1: row pass with the scatter by L2
@@ -268,7 +278,8 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     __shared__ float part[2][kConsumers][4];
     __shared__ volatile int abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s0 = a.cta[blockIdx.x], s1 = a.cta[blockIdx.x + 1];
+    int s0 = a.cta[blockIdx.x], s1 = a.cta[blockIdx.x + 1];
+    if (!CHECKED(s0 >= 0 && s0 <= s1 && s1 <= a.strips && ALIGNED16(ring) && ALIGNED16(a.blob), 503, blockIdx.x)) s0 = s1 = 0;
     constexpr int NG = kConsumers / NW;
     // a group waits for the fills of its own barriers only, in order: the wait
     // for one fill can never be taken for the fill before it
@@ -304,7 +315,11 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
             nxt = (b + 32 + lane < s1) ? a.meta[b + 32 + lane] : make_int4(0, 0, 0, 0);
             const int q = b - s0 + lane;
             const int need = q - strip_live(m.w);
-            const uint32_t bytes = (uint32_t)((m.y & kStripPackets) * Packet<VT, KIND>::kBytes);
+            uint32_t bytes = (uint32_t)((m.y & kStripPackets) * Packet<VT, KIND>::kBytes);
+            if (!CHECKED(strip_at(m.w) + (long long)bytes <= a.ring &&
+                             ((long long)(unsigned)m.x << 4) + bytes <= a.blob_bytes,
+                         504, b + lane))
+                bytes = 0;
             bool done = b + lane >= s1;
             for (;;) {
                 if (!done && need <= oldest) {
@@ -346,7 +361,12 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
         // need not wait for the flag's
         const int flag = KIND == 2 ? a.epi.st[0].stopped : (a.check_stop ? a.st[0].stopped : 0);
         for (int q = grp; q < s1 - s0; q += NG, par ^= 1) {
-            const int4 m = nxt;
+            int4 m = nxt;
+            constexpr long long kBytes = Packet<VT, KIND>::kBytes;
+            if (!CHECKED(strip_at(m.w) + (m.y & kStripPackets) * kBytes <= a.ring &&
+                             m.z >= 0 && m.z + (31 - __clz((m.w & 15) | 1)) < a.items,
+                         505, s0 + q))
+                m = make_int4(0, 0, 0, 0);
             nxt = (q + NG < s1 - s0) ? __ldg(a.meta + s0 + q + NG) : make_int4(0, 0, 0, 0);
             const int npk = m.y & kStripPackets;
             const bool tall = (m.y & kStripTall) != 0;
@@ -379,10 +399,10 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 int p = p0;
                 const unsigned char* sp = strip + p0 * Packet<VT, KIND>::kBytes;
                 for (; p + 4 <= p1; p += 4, sp += 4 * Packet<VT, KIND>::kBytes)
-                    dot_packets<VT, KIND, 4>(sp, lane, xs, acc);
-                if (p1 - p == 3) dot_packets<VT, KIND, 3>(sp, lane, xs, acc);
-                else if (p1 - p == 2) dot_packets<VT, KIND, 2>(sp, lane, xs, acc);
-                else if (p1 - p == 1) dot_packets<VT, KIND, 1>(sp, lane, xs, acc);
+                    dot_packets<VT, KIND, 4>(sp, lane, xs, a.x_len, acc);
+                if (p1 - p == 3) dot_packets<VT, KIND, 3>(sp, lane, xs, a.x_len, acc);
+                else if (p1 - p == 2) dot_packets<VT, KIND, 2>(sp, lane, xs, a.x_len, acc);
+                else if (p1 - p == 1) dot_packets<VT, KIND, 1>(sp, lane, xs, a.x_len, acc);
                 dot = KIND == 1 ? acc[0] + acc[1] : (acc[0] + acc[1]) + (acc[2 % kSums<KIND>] + acc[3 % kSums<KIND>]);
             }
             if (KIND != 1) {
@@ -433,9 +453,10 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                     if (__any_sync(0xffffffffu, c0 != 0.f)) {
                         float* dst = COPIES ? a.delta + (blockIdx.x % kDeltaCopies) * a.copy
                                             : (tall ? a.deltaT : a.delta);
+                        const long long dst_len = COPIES ? a.copy : a.delta_len;
                         const unsigned char* sp = strip + p0 * Packet<VT, KIND>::kBytes;
                         for (int p = p0; p < p1; ++p, sp += Packet<VT, KIND>::kBytes)
-                            scatter_packet<VT>(sp, lane, c0, c1, c2, c3, dst);
+                            scatter_packet<VT>(sp, lane, c0, c1, c2, c3, dst, dst_len);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&empty[slot]);

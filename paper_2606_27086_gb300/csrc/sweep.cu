@@ -15,37 +15,12 @@
 //    of coef from L2, no atomics at all (bitwise deterministic).
 #include <algorithm>
 
+#include "check.cuh"
 #include "common.cuh"
 
 namespace suppy {
 
-#ifdef SUPPY_CHECKED
-__device__ int g_check[3];
-__device__ __noinline__ bool check_fail(int tag, long long idx) {
-    if (atomicCAS(&g_check[0], 0, tag) == 0) {
-        g_check[1] = (int)(idx & 0xffffffffLL);
-        g_check[2] = (int)(idx >> 32);
-    }
-    return false;
-}
-#define CHECKED(cond, tag, idx) ((cond) ? true : check_fail((tag), (long long)(idx)))
-#define ALIGNED16(p) ((((uintptr_t)(p)) & 15u) == 0)
-#else
-#define CHECKED(cond, tag, idx) true
-#define ALIGNED16(p) true
-#endif
-
-cudaError_t read_check_word(int* out3) {
-#ifdef SUPPY_CHECKED
-    cudaError_t e = cudaMemcpyFromSymbol(out3, g_check, sizeof(int) * 3);
-    if (e != cudaSuccess) return e;
-    int z[3] = {0, 0, 0};
-    return cudaMemcpyToSymbol(g_check, z, sizeof(int) * 3);
-#else
-    out3[0] = out3[1] = out3[2] = 0;
-    return cudaSuccess;
-#endif
-}
+cudaError_t read_check_word(int* out3) { return take_check_words(out3); }
 
 namespace {
 
