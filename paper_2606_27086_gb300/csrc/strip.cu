@@ -145,13 +145,15 @@ struct Packet {
     static constexpr int kIdx = KIND == 1 ? 80 : 16, kVal = kIdx + 256;   // after bases and flags
 };
 
-// x[base + o], 0 in an empty slot.
+// x[base + o], 0 in an empty slot.  A coherent load: this kernel may have started
+// before the one that writes x ended, so x is not read-only for its lifetime, as
+// .nc would promise (same times either way).
 __device__ __forceinline__ float gather(const float* x, int base, unsigned o) {
     float g;
     asm("{\n\t.reg .pred p;\n\t"
         "setp.ne.u32 p, %2, 65535;\n\t"
         "mov.f32 %0, 0f00000000;\n\t"
-        "@p ld.global.nc.f32 %0, [%1];\n\t}"
+        "@p ld.global.f32 %0, [%1];\n\t}"
         : "=f"(g)
         : "l"(x + (base + (int)o)), "r"(o));
     return g;
