@@ -885,8 +885,31 @@ def ours(args):
     if world > 1:
         torch.distributed.barrier()
     if rank == 0:
-        print(json.dumps(res), flush=True)
+        detail = json.dumps(res)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                f.write(detail + "\n")
+        else:
+            log(f"[bench] detail {detail}")
+        print(json.dumps(headline(res)), flush=True)
     return 0
+
+
+def headline(res: dict) -> dict:
+    """The result line: the whole record but for the secondary workloads, of which
+    it keeps one figure each, so that it stays a line of about four kilobytes (the
+    record itself, some 27, goes to stderr or --detail FILE)."""
+    out = {k: v for k, v in res.items() if k not in ("variants", "precision", "serving", "cpu_baseline")}
+    out["launch_shape"] = {k: v for k, v in res["launch_shape"].items() if v}
+    if "variants" in res:
+        out["variants"] = {k: float(f"{v['value']:.4g}") for k, v in res["variants"].items()
+                           if isinstance(v, dict) and "value" in v}
+    if "serving" in res:
+        out["serving"] = {k: {q: float(f"{v[q]:.4g}") for q in ("solves_per_s", "p50_s", "p99_s") if q in v}
+                          for k, v in res["serving"].items() if isinstance(v, dict) and "solves_per_s" in v}
+    if "cpu_baseline" in res:
+        out["cpu_baseline"] = {k: res["cpu_baseline"].get(k) for k in ("value", "unit", "cores", "kind")}
+    return out
 
 
 def pinned_opts(pk, pin: str) -> dict:
@@ -1010,6 +1033,9 @@ def main():
                          "1 column-major rows, 2 patches (one pass), -1 off] as a plain run's "
                          "launch_shape reports it (e.g. 1,4096,6,32,2,2,2), for runs under a "
                          "profiler, whose serialised launches distort the tuner's timings")
+    ap.add_argument("--detail", default="", metavar="FILE",
+                    help="write the whole record (secondary workloads, precision, serving) to FILE "
+                         "instead of stderr; the result line on stdout is its short form")
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=12.0)
     ap.add_argument("--serve-requests", type=int, default=512,
