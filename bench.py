@@ -864,7 +864,7 @@ def ours(args):
            "roofline": roof, "kernels": per, "e2e": e2e,
            "gpu_launches": int(nl), "clocks": clocks, "create_s": t_create,
            "sweeps_per_step": SWEEPS,
-           "launch_shape": {k: info[k] for k in ("strategy", "scatter", "tma", "tiles", "chunks",
+           "launch_shape": {k: info[k] for k in ("strategy", "block", "scatter", "tma", "tiles", "chunks",
                                                   "tile_warps1", "tile_warps2", "tile_coef_warps",
                                                   "tile_ring", "tile_stream_bytes",
                                                   "tile_segments", "tile", "stages", "col_tile",
@@ -872,6 +872,11 @@ def ours(args):
                                                   "lanes_per_row", "col_lanes",
                                                   "transposed_rows", "scatter_patch",
                                                   "perturb_cluster")}}
+    res["launch_shape"]["pin"] = pin_of(info)   # rebuilds it without timing
+    if info["block"] == STRIP_BLOCK:
+        # the shape of the streamed passes, which the strips do not run
+        for k in ("tile", "stages", "col_tile", "col_stages", "map", "col_map"):
+            res["launch_shape"].pop(k)
     if args.pin:
         res["launch_shape"]["pinned"] = args.pin
     ctx.close()
@@ -912,9 +917,23 @@ def headline(res: dict) -> dict:
     return out
 
 
+STRIP_BLOCK = 800   # threads per CTA of the strip-ordered passes (suppy_info.block)
+
+
+def pin_of(info: dict) -> str:
+    """The --pin of a context's launch configuration.  Strips have no shape to
+    give: the strategy with every streaming option left open takes them."""
+    if info["block"] == STRIP_BLOCK:
+        return f"{info['strategy']},0,0,0,0,0,0"
+    tr = 0 if info["strategy"] == 3 else (2 if info["scatter_patch"] else 1) if info["transposed_rows"] else -1
+    return ",".join(str(v) for v in (info["strategy"], info["tile"], info["stages"],
+                                     info["lanes_per_row"] if info["tma"] else 0, info["map"], info["col_map"], tr))
+
+
 def pinned_opts(pk, pin: str) -> dict:
     """from_problem options of a --pin launch configuration
-    (strategy,tile,stages,lanes,map,col_map[,pixel numbering])."""
+    (strategy,tile,stages,lanes,map,col_map[,pixel numbering]; zeros leave an
+    option open)."""
     vals = [int(v) for v in pin.split(",")]
     st_, tile, stages, lanes, mp, cmp_ = vals[:6]
     tr = vals[6] if len(vals) > 6 else -1
@@ -1031,8 +1050,9 @@ def main():
                     help="build the headline context with this launch configuration instead of "
                          "tuning it: strategy,tile,stages,lanes,map,col_map[,pixel numbering: "
                          "1 column-major rows, 2 patches (one pass), -1 off] as a plain run's "
-                         "launch_shape reports it (e.g. 1,4096,6,32,2,2,2), for runs under a "
-                         "profiler, whose serialised launches distort the tuner's timings")
+                         "launch_shape reports it under pin (e.g. 1,4096,6,32,2,2,2; "
+                         "1,0,0,0,0,0,0 for strips), for runs under a profiler, whose serialised "
+                         "launches distort the tuner's timings")
     ap.add_argument("--detail", default="", metavar="FILE",
                     help="write the whole record (secondary workloads, precision, serving) to FILE "
                          "instead of stderr; the result line on stdout is its short form")

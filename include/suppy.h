@@ -296,7 +296,9 @@ typedef struct {
     int32_t lanes_per_row;        /* launch shape chosen for the sweep       */
     int32_t elems_in_regs;        /* row elements a lane holds between dot and scatter */
     int32_t grid;                 /* CTAs of the sweep launch                */
-    int32_t block;                /* threads per CTA of the sweep launch     */
+    int32_t block;                /* threads per CTA of the sweep launch: 800 for the
+                                   * strip-ordered passes, 768 for the streamed ones,
+                                   * 256 for the register-fed ones           */
     int32_t perturb_cluster;      /* CTAs per cluster of the perturbation    */
     int64_t device_bytes;         /* device memory held by the context       */
     int32_t strategy;             /* 1 one pass, 2 two passes, 3 tiled one pass */
@@ -304,9 +306,13 @@ typedef struct {
     int32_t col_lanes;            /* two passes: lanes per column            */
     int32_t col_grid;             /* two passes: CTAs of the column pass     */
     int32_t tma;                  /* 1: the sweep streams A by bulk copies   */
-    int32_t tile, stages;         /* streaming row pass: ring tile length (elements), stages */
-    int32_t col_tile, col_stages; /* streaming column pass: the same       */
-    int32_t map, col_map;         /* streaming lane maps (opts.stream_map: 1 or 2) */
+    /* the shape of the streamed passes: ring tile length (elements), stages and
+     * lane maps (opts.stream_map: 1 or 2).  With strips (block 800) it is the
+     * one the streamed passes would have and does not describe what runs; the
+     * same form is built again by its strategy with every streaming option 0 */
+    int32_t tile, stages;
+    int32_t col_tile, col_stages; /* column pass                             */
+    int32_t map, col_map;
     /* tiled sweep (strategy 3): tiles (= CTAs), chunks, warps of the dot
      * products, of the scatter and of the coefficients, ring bytes, bytes and
      * segments of the tile streams; zero for the other strategies */
