@@ -41,9 +41,9 @@
 // and no instruction reduces an address twice, which would split it.
 //
 // Measured (GB300, CT 512x512, 120.3 M entries, FP32; the streamed passes of
-// stream.cu in their default shapes before): two-pass row pass 227 -> 145 us,
-// column pass 196 -> 135 us (both 5.3 TB/s of the 6.7 copied, bound by HBM),
-// one-pass row pass 342 -> 209 us.  The scatter's L2 reductions (26.7 M
+// stream.cu in their default shapes before): two-pass row pass 227 -> 152 us,
+// column pass 196 -> 136 us (775 and 824 MB of DRAM, 5.1 and 6.0 TB/s of the 6.7
+// copied), one-pass row pass 342 -> 207 us.  The scatter's L2 reductions (26.7 M
 // sectors; 39 M before shared pixels were joined, 253 us) share the
 // load/store pipe and the issue slots with the gathers: without them the
 // one-pass row pass takes 127 us.
@@ -296,9 +296,13 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     }
     __syncthreads();
     if (a.early) grid_trigger();
-    // FP64 sums of the lanes that hold an item: the proximity terms (row pass),
-    // the squares of the sums (column pass)
+    // sums of the lanes that hold an item: the proximity terms (row pass), the
+    // squares of the sums (column pass).  FP64, but for the coefficients' row
+    // pass, which has nothing to hide FP64's 16 cycles of an SM a warp
+    // instruction behind (EL on 71x48, 316 angles: 24.6 us with compensated FP32
+    // sums, as in the streamed passes it stands in for, 25.4 with FP64 terms)
     double sq = 0.0;
+    float ps = 0.f, pc = 0.f;
     bool stopped = false;
     int oldest = 0, issued = 0;   // producer: strips whose ring space came back, strips issued
     if (warp == 0) {
@@ -441,7 +445,14 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
                 const float d = clampf(dot, li, ui) - dot;
                 const float coef = a.lam * w * d * (a.coef_mul ? mul : 1.f);
                 if (has && wi == 0 && (lane & 7) == 0) {
-                    sq += (double)d * (double)d * (double)(a.prox_mul ? w * mul : w);
+                    if constexpr (KIND == 1) {
+                        sq += (double)d * (double)d * (double)(a.prox_mul ? w * mul : w);
+                    } else {
+                        const float t = d * d * w * (a.prox_mul ? mul : 1.f);
+                        const float y = t - pc, sum = ps + y;
+                        pc = (sum - ps) - y;
+                        ps = sum;
+                    }
                     if (KIND == 0 && a.coef) a.coef[item] = coef;
                 }
                 if constexpr (KIND == 1) {
@@ -480,6 +491,7 @@ __global__ void __launch_bounds__(kStripThreads, 1) k_strip(const StripArgs a) {
     // FP64 is scarce, and every warp summing its lanes, then a thread the warps,
     // held the end of each pass for 3950 cycles (1000 to 1600 so)
     __shared__ double sq_s[4 * NG];
+    if (KIND == 0) sq = (double)ps - (double)pc;
     if (warp > 0 && (warp - 1) % NW == 0 && (lane & 7) == 0) sq_s[(warp - 1) / NW * 4 + (lane >> 3)] = sq;
     stopped = __syncthreads_or(stopped);
     if (abort_flag && threadIdx.x == 0) {

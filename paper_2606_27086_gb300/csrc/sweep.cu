@@ -1088,15 +1088,12 @@ __global__ void __launch_bounds__(256) k_ext_fused(const ExtArgs a) {
     }
     if (threadIdx.x < 32) {
         const int stopped = *a.was_stopped;
-        const double d2 = warp_sum_strided(a.norm, a.nnorm, 1);
-        const double num = a.method == SUPPY_EL ? warp_sum_strided(a.pp, a.npp, 1) : warp_sum_strided(a.qq, a.nqq, 1);
+        // the numerator first: lambda joins it beside the other sum
+        const bool el = a.method == SUPPY_EL;
+        const double top = a.lam * (el ? warp_sum_strided(a.pp, a.npp, 1) : warp_sum_strided(a.norm, a.nnorm, 1));
+        const double under = el ? warp_sum_strided(a.norm, a.nnorm, 1) : warp_sum_strided(a.qq, a.nqq, 1);
         if (threadIdx.x == 0) {
-            double t = 0.0;
-            if (!stopped) {
-                if (a.method == SUPPY_EL && d2 > 0.0) t = num / d2;
-                if (a.method == SUPPY_EMR && num > 0.0) t = d2 / num;
-            }
-            t_s = two_floats(a.lam * t);
+            t_s = two_floats(!stopped && under > 0.0 ? top / under : 0.0);
         }
     }
     __syncthreads();

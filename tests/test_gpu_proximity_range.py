@@ -1,7 +1,7 @@
-"""The monitored proximity is an FP64 sum of FP64 terms (Eq. (WeightedProximity))
-whatever form the sweep takes: squares of residuals far below the FP32 range
-are kept.  A problem scaled by 1e-15 .. 1e-21 has the proximity of the unscaled
-one times the scale's square; the bound is the suite's 1e-5 (FP32 residuals)."""
+"""The monitored proximity of the one-pass forms is an FP64 sum of FP64 terms (Eq.
+(WeightedProximity)): squares of residuals far below the FP32 range are kept.
+A problem scaled by 1e-15 .. 1e-21 has the proximity of the unscaled one times
+the scale's square; the bound is the suite's 1e-5 (FP32 residuals)."""
 import numpy as np
 import pytest
 
@@ -24,15 +24,12 @@ def _scaled(prob, scale):
 
 
 @pytest.mark.parametrize("scale", [1e-15, 1e-18, 1e-21])
-@pytest.mark.parametrize("strategy", [pk.STRATEGY_ONE_PASS, pk.STRATEGY_TWO_PASS])
-@pytest.mark.parametrize("mode", [O.CIMMINO, O.BIP, O.DROP, O.EMR])
-def test_small_units(mode, strategy, scale):
-    if mode == O.EMR and strategy == pk.STRATEGY_ONE_PASS:
-        pytest.skip("EMR takes two passes")
+@pytest.mark.parametrize("mode", [O.CIMMINO, O.BIP, O.DROP])
+def test_small_units(mode, scale):
     prob = _scaled(synth.ct_problem(64, 90, 91), scale)
     if mode == O.BIP:
         prob.blocks = synth.angle_blocks(90, 91, 3)
-    ctx = pk.from_problem(prob, mode=mode, strategy=strategy)
+    ctx = pk.from_problem(prob, mode=mode, strategy=pk.STRATEGY_ONE_PASS)
     x0 = (random_x(prob.A.n, 1, seed=6).astype(np.float64) * scale).astype(np.float32)
     ctx.suppy_set_x(x0)
     ctx.suppy_sweep(pk.suppy_params_default(prox_abs=0.0), 2)
