@@ -77,7 +77,10 @@ typedef enum {
 
 /* Storage type of A's values on the device.  BF16/FP16 are rounded to nearest
  * even from the FP32 input; every accumulation stays FP32 (dot products,
- * corrections) or FP64 (row norms, proximity, objective, acceptance).
+ * corrections) or FP64 (row norms, proximity, objective, acceptance; the
+ * proximity monitored by the streamed passes, suppy_info block 768, and by the
+ * strips of two-pass sweeps is summed in compensated FP32 within a thread and
+ * FP64 beyond).
  * SUPPY_HALF_AUTO stores 16 bits in the format with the smaller rounding
  * error on this matrix: per entry the error bound is max(2^-11 |v|, 2^-25)
  * for FP16 (its unit roundoff, and half its subnormal spacing) and 2^-8 |v|
@@ -169,7 +172,9 @@ typedef struct {
      * numbering or plain loads asked for (the four options below), strategies
      * 1 and 2 read strip-ordered copies of A when neighbouring rows (columns)
      * are alike enough: four at a time, as packets of 128 entries with 16-bit
-     * offsets, about 6.3 bytes per FP32 entry and copy beside the row copy. */
+     * offsets, about 6.3 bytes per FP32 entry (7 with the scatter) and copy
+     * beside the row copy; the CSC entries go once column strips are built.  A
+     * create that runs out of memory with them is made again without. */
     /* Streaming of A through shared memory by bulk asynchronous copies (TMA)
      * for one right-hand side: 0 automatic (used when eligible), -1 off. */
     int32_t tma;

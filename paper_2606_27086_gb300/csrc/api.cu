@@ -1730,8 +1730,9 @@ suppy_status build_strips(suppy_ctx* c, suppy_ctx::StripSet& S, const int2* info
     // (12.3 KB a strip), 1024x1024 40 angles 117 / 127 / 177 / 301 (24.6 KB),
     // 384x384 FP16 143 / 107 / 96 / 117 (6.4 KB), 128x128 blocks 11.6 / 10.4
     // / 11.0 / 12.3 (2.7 strips a CTA), radiotherapy blocks 29.6 / 21.6 / 20.6
-    // / 22.5 (4.2 KB), 64x64 - / 11.7 / 11.9 / 10.5 (2.1 KB); 512x512 two
-    // passes, rows 196 / 151 / 145 / 158.
+    // / 22.5 (4.2 KB), 64x64 - / 11.7 / 11.9 / 10.5 (2.1 KB).  The rows of
+    // 512x512 in two passes measured 196 / 151 / 145 / 158: the line at 150 KB
+    // gives them four, two would be 4% faster there.
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
     const double strip_bytes = (double)bytes / std::max(kept, 1);
