@@ -953,11 +953,11 @@ def profile_case(case: int, steps: int, warm: int = 0, pin: str = "") -> int:
     two-pass sweep, one perturbation cluster per image); case 8: CT 384x384
     with EMR and the variance rule evaluated every iteration (extrapolation
     and variance kernels); case 9: CT 384x384 with the register-fed two-pass
-    sweep (no bulk copies), the cluster perturbation with the image bands in
-    shared memory, and the standalone proximity and objective evaluations
+    sweep (no bulk copies), the cluster perturbation with the image in shared
+    memory, and the standalone proximity and objective evaluations
     (two each, after the iterations); case 10: a 2048x2048 image over a
-    random slab system (20000 rows) with TV, whose image bands exceed a
-    cluster's shared memory, so the cluster perturbation reads them from
+    random slab system (20000 rows) with TV, whose image exceeds a cluster's
+    shared memory, so the cluster perturbation reads them from
     global memory; case 11: CT 384x384 with the tiled one-pass sweep.
     The profiled iterations run inside the NVTX range "profile", so that
     `ncu --nvtx --nvtx-include profile/` skips the tuning launches and the
